@@ -280,14 +280,12 @@ typedef struct {
                                     0 plain CG; other values: DECT_EINVAL */
     int32_t use_graph;           /* 1: capture one iteration as a CUDA graph */
     int32_t bp_view_groups;      /* backprojector view groups per image tile, 1..16; -1 = chosen from the
-                                    occupancy (fill the GPU's resident slots) without timing; 0 = autotuned:
-                                    dect_admm_create times the backprojector on this batch for a few
-                                    candidates (memory permitting) and keeps the fastest (reported in
-                                    dect_stats). It fixes the order of a pixel's partial sums: results
-                                    are bitwise reproducible for a fixed value, and a slice solved alone
-                                    or in a batch gives identical bits when the value is the same (it is
-                                    the one launch-dependent choice; an autotuned value can differ from
-                                    run to run). */
+                                    occupancy (fill the GPU's resident slots); 0 = from the batch's size: 12 below
+                                    1024 tiles of 32 x 32 pixels, 6 from there on (fewer where the partial images
+                                    would not fit; reported in dect_stats). It fixes the order of a pixel's
+                                    partial sums: results are bitwise reproducible for a fixed value, and a
+                                    slice solved alone or in a batch gives identical bits when the value is the
+                                    same (it is the one launch-dependent choice of the batch). */
     int32_t storage;             /* dect_storage (DECT_STORE_F32): 16-bit formats halve the bytes of the
                                     sinogram vectors and textures at the cost of their precision */
     int32_t scheme;              /* dect_scheme (DECT_SCHEME_UDM_PCG): the splitting one iteration runs */
@@ -307,9 +305,8 @@ typedef struct {
                                     dect_admm_stats. One projection and one f-evaluation per ray each time,
                                     outside Table 1's counts. 0 (default): never. */
     int32_t bp_tile;             /* backprojector tile side in pixels, 32 or 64 (its CTA's warps take bands of
-                                    32 columns or rows of the tile); 0 (default) = chosen by the autotuner
-                                    with bp_view_groups (timed on this batch; with bp_view_groups fixed, the
-                                    two sides are timed at that count; with -1, 32). The side does not change
+                                    32 columns or rows of the tile); 0 (default) = timed on this batch at
+                                    creation (with bp_view_groups = -1: 32). The side does not change
                                     results (every pixel receives the same contributions in the same order). */
     int32_t bp_cluster;          /* the backprojector's view groups of a tile as one thread-block cluster that
                                     adds their accumulators on chip (distributed shared memory, in rank order)
@@ -320,8 +317,8 @@ typedef struct {
     int32_t bp_slices;           /* slices per backprojector CTA: 2 backprojects the same rays into two
                                     consecutive slices of one geometry at once (shared staging and sample
                                     positions, one accumulator per slice; UDM-PCG scheme), 1 one slice,
-                                    0 (default) timed by the autotuner (one slice when bp_cluster = 1).
-                                    Same bits either way. */
+                                    0 (default) timed by the autotuner, up to four slices where a geometry has
+                                    as many (one slice when bp_cluster = 1). Same bits either way. */
     int32_t bp_reduce;           /* plain (non-cluster) backprojector with C >= 2 view groups: the last CTA of a
                                     tile to finish sums the tile's C partial images (in view-group order, the
                                     finalize pass's order) into partial image 0 while they are in L2 and drops

@@ -550,11 +550,13 @@ struct dect_admm {
     int sweep_tile = kSweepTileDefault;  // backprojector tile side (32 or 64; does not change results)
     bool sweep_cluster = false;      // the view groups of a tile reduce on chip into one partial image
     std::vector<int> cluster_cands;  // cluster forms the autotuner may time (0 off, 1 on)
-    int sweep_sg = 1;                // slices per sweep CTA (2: pairs of consecutive slices of one geometry)
+    int sweep_sg = 1;                // slices per sweep CTA (2, 4: consecutive slices of one geometry)
     std::vector<int> sg_cands;       // slices per CTA the autotuner may time
-    std::vector<int4> sgroups;       // the pairs (second -1 for a slice without a partner)
-    int4* d_sgroups = nullptr;
-    int sweep_units() const { return sweep_sg == 2 ? (int)sgroups.size() : B; }
+    std::vector<int4> sgroups[2];    // groups of up to 2 and up to 4 such slices (-1 past a group's size)
+    int4* d_sgroups[2] = {nullptr, nullptr};
+    int sweep_units(int sg) const { return sg > 1 ? (int)sgroups[sg == 4].size() : B; }
+    int sweep_units() const { return sweep_units(sweep_sg); }
+    const int4* sweep_groups_dev(int sg) const { return d_sgroups[sg == 4]; }
     bool sweep_reduce = false;       // the last CTA of a tile sums its C partials into image 0 (reduced form)
     int* tile_count = nullptr;       // the reduced form's arrival counters, one per tile (zero between launches)
     int n_tile_count = 0;            // counters: the batch's tiles at the smallest tile side
@@ -634,7 +636,7 @@ static void pe(dect_admm* A, int phase, int nk, cudaStream_t st) {
 
 static void free_admm(dect_admm* A) {
     void* ptrs[] = {A->ds, A->rays.d, A->pix.d, A->tx.d, A->ty.d, A->rows.d, A->cols.d, A->sweep.d, A->ptile.d, A->d_groups,
-                    A->d_sgroups,
+                    A->d_sgroups[0], A->d_sgroups[1],
                     A->bp_partial, A->x, A->r, A->s,
                     A->p, A->Ap, A->z, A->uz, A->x0, A->truth, A->Rx, A->a, A->ua, A->q, A->Z, A->y, A->uy,
                     A->meas, A->txb, A->tyb, A->mu, A->H, A->Hn, A->stage, A->status, A->sc, A->part_udm,
@@ -708,7 +710,7 @@ static void enq_pcg(dect_admm* A, int n, bool with_grad, const float* H, cudaStr
     pe(A, DECT_PHASE_UPDATE, 1, st);
     pb(A, st);
     launch_bp_sweep(A->ds, A->sweep.map(A->sweep_units()), A->sweep.total, A->sweep_C, A->sweep_tile, A->sweep_cluster,
-                    A->sweep_sg, A->d_sgroups, A->q, A->bp_partial, A->n_img, A->prec, A->reduce_count(), st);
+                    A->sweep_sg, A->sweep_groups_dev(A->sweep_sg), A->q, A->bp_partial, A->n_img, A->prec, A->reduce_count(), st);
     pe(A, DECT_PHASE_BACKPROJECT, 1, st);
     pb(A, st);
     launch_bp_finalize(with_grad ? BP_R0 : BP_R0_NOGRAD, A->ds, A->pix.map(B), A->pix.total, A->bp_parts(),
@@ -723,7 +725,7 @@ static void enq_pcg(dect_admm* A, int n, bool with_grad, const float* H, cudaStr
         enq_project(A, A->p, A->q, st);
         pb(A, st);
         launch_bp_sweep(A->ds, A->sweep.map(A->sweep_units()), A->sweep.total, A->sweep_C, A->sweep_tile, A->sweep_cluster,
-                        A->sweep_sg, A->d_sgroups, A->q, A->bp_partial, A->n_img, A->prec, A->reduce_count(), st);
+                        A->sweep_sg, A->sweep_groups_dev(A->sweep_sg), A->q, A->bp_partial, A->n_img, A->prec, A->reduce_count(), st);
         pe(A, DECT_PHASE_BACKPROJECT, 1, st);
         pb(A, st);
         launch_bp_finalize(with_grad ? BP_AP : BP_AP_NOGRAD, A->ds, A->pix.map(B), A->pix.total, A->bp_parts(),
@@ -1148,8 +1150,8 @@ static dect_status enq_initialize(dect_admm* A, cudaStream_t st) {
 // Sweep block map for C CTA groups per TILE x TILE tile (prefix over slices, or over slice pairs for sg = 2)
 static void sweep_prefix(const dect_admm* A, int C, int tile, int sg, std::vector<int>& h) {
     h.assign(1, 0);
-    if (sg == 2)
-        for (const int4& p : A->sgroups)
+    if (sg > 1)
+        for (const int4& p : A->sgroups[sg == 4])
             h.push_back(h.back() + sweep_tiles(A->hs[p.x].g.nx, A->hs[p.x].g.ny, tile) * C);
     else
         for (int b = 0; b < A->B; ++b) h.push_back(h.back() + sweep_tiles(A->hs[b].g.nx, A->hs[b].g.ny, tile) * C);
@@ -1205,13 +1207,11 @@ static cudaError_t autotune_projector(dect_admm* A) {
     return cudaMemcpy(A->ptile.d, A->ptile.h.data(), sizeof(int) * A->ptile.h.size(), cudaMemcpyHostToDevice);
 }
 
-// Times the backprojector sweep on this batch (on a zero sinogram; the work does not depend on the
-// values) and keeps the fastest shape (fewer view groups unless more are 1% faster), in three stages:
-// slices per CTA x view groups C at the default tile side, then the other tile sides at the best of
-// those, then the cluster form there. Shrinks the partial-image buffer to the choice (bp_partial is
-// allocated for the largest candidate C). The tile side, the slices per CTA and the cluster form do
-// not change results; C fixes the order of a pixel's partial sums.
-static cudaError_t autotune_sweep(dect_admm* A, const std::vector<int>& cands, const std::vector<int>& tiles) {
+// Times the backprojector on this batch (on a zero sinogram; the work does not depend on the values) at the
+// given view groups C and keeps the fastest shape, in three stages: slices per CTA at the default tile side, then
+// the other tile sides at the best of those, then the cluster form there (a later shape has to be 1% faster). No
+// choice changes results. Shrinks the partial-image buffer to the choice.
+static cudaError_t autotune_sweep(dect_admm* A, const int C, const std::vector<int>& tiles) {
     cudaStream_t st = A->cap;
     cudaError_t e = cudaMemsetAsync(A->q, 0, sino_bytes(A->prec) * (size_t)A->n_sino, st);
     cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -1220,19 +1220,19 @@ static cudaError_t autotune_sweep(dect_admm* A, const std::vector<int>& cands, c
     const int tile0 =
         std::find(tiles.begin(), tiles.end(), kSweepTileDefault) != tiles.end() ? kSweepTileDefault : tiles[0];
     const bool cl0 = A->cluster_cands.size() == 1 && A->cluster_cands[0] == 1;  // cluster form required
-    int best = cands[0], best_tile = tile0, best_sg = 1;
+    int best_tile = tile0, best_sg = A->sg_cands[0];
     bool best_cluster = false;
     float best_ms = 0.f;
     bool first = true;
     std::vector<int> h;
-    auto trial = [&](int sg, int tile, int C, bool cluster) {
+    auto trial = [&](int sg, int tile, bool cluster) {
         if (e != cudaSuccess || (cluster && (C < 2 || C > 16 || sg != 1))) return;
         sweep_prefix(A, C, tile, sg, h);
         e = cudaMemcpy(A->sweep.d, h.data(), sizeof(int) * h.size(), cudaMemcpyHostToDevice);
         if (e != cudaSuccess) return;
-        const BlockMap m{A->sweep.d, sg == 2 ? (int)A->sgroups.size() : A->B};
+        const BlockMap m{A->sweep.d, A->sweep_units(sg)};
         auto run = [&]() {
-            launch_bp_sweep(A->ds, m, h.back(), C, tile, cluster, sg, A->d_sgroups, A->q, A->bp_partial, A->n_img,
+            launch_bp_sweep(A->ds, m, h.back(), C, tile, cluster, sg, A->sweep_groups_dev(sg), A->q, A->bp_partial, A->n_img,
                             A->prec, A->sweep_reduce ? A->tile_count : nullptr, st);
         };
         // a cluster shape the device cannot schedule is reported at launch: skip that candidate
@@ -1249,8 +1249,7 @@ static cudaError_t autotune_sweep(dect_admm* A, const std::vector<int>& cands, c
         if (e == cudaSuccess) e = cudaEventSynchronize(e1);
         float ms = 0.f;
         if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
-        if (e == cudaSuccess && (first || ms < 0.99f * best_ms || (ms <= best_ms && C < best))) {
-            best = C;
+        if (e == cudaSuccess && (first || ms < 0.99f * best_ms)) {
             best_tile = tile;
             best_cluster = cluster;
             best_sg = sg;
@@ -1258,21 +1257,20 @@ static cudaError_t autotune_sweep(dect_admm* A, const std::vector<int>& cands, c
             first = false;
         }
     };
-    for (int sg : A->sg_cands)
-        for (int C : cands) trial(sg, tile0, C, cl0);
-    const int C1 = best, sg1 = best_sg;
+    for (int sg : A->sg_cands) trial(sg, tile0, cl0);
+    const int sg1 = best_sg;
     const bool cl1 = best_cluster;
     for (int tile : tiles)
-        if (tile != tile0) trial(sg1, tile, C1, cl1);
-    if (A->cluster_cands.size() > 1) trial(1, best_tile, C1, true);
+        if (tile != tile0 && sg1 < 4) trial(sg1, tile, cl1);
+    if (A->cluster_cands.size() > 1) trial(1, best_tile, true);
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
     if (e != cudaSuccess) return e;
-    A->sweep_C = best;
+    A->sweep_C = C;
     A->sweep_tile = best_tile;
     A->sweep_cluster = best_cluster;
     A->sweep_sg = best_sg;
-    sweep_prefix(A, best, best_tile, best_sg, A->sweep.h);
+    sweep_prefix(A, C, best_tile, best_sg, A->sweep.h);
     A->sweep.total = A->sweep.h.back();
     e = cudaMemcpy(A->sweep.d, A->sweep.h.data(), sizeof(int) * A->sweep.h.size(), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return e;
@@ -1448,7 +1446,7 @@ extern "C" dect_status dect_admm_create(dect_geom* const* geoms, int32_t B, cons
     for (auto* m : {&A->rays, &A->pix, &A->tx, &A->ty, &A->rows, &A->cols, &A->sweep, &A->cols64, &A->ptile,
                     &A->prows, &A->pcols})
         m->h.assign(1, 0);
-    std::vector<int> tune;  // candidate CTA groups per tile when autotuning (first = the occupancy choice)
+    std::vector<int> tune;  // the view groups at which the launch shapes are timed (empty: not timed)
     std::vector<int> tune_tiles;  // candidate tile sides when autotuning
     {
         cudaError_t ae = sweep_init_attributes();
@@ -1467,22 +1465,28 @@ extern "C" dect_status dect_admm_create(dect_geom* const* geoms, int32_t B, cons
         for (int b = 0; b < B; ++b) A->n_tile_count += sweep_tiles(geoms[b]->desc.nx, geoms[b]->desc.ny, 32);
         if (P->bp_cluster == 0) A->cluster_cands = {0, 1};
         else A->cluster_cands = {P->bp_cluster > 0 ? 1 : 0};
-        // pairs of consecutive slices of one geometry for the two-slice sweep (UDM-PCG only: the comparison
-        // scheme backprojects one basis with its own weights)
-        bool pairs = false;
-        for (int b = 0; b < B; ++b) {
-            if (!A->sgroups.empty() && A->sgroups.back().y < 0 &&
-                same_geometry(geoms[A->sgroups.back().x]->desc, geoms[b]->desc)) {
-                A->sgroups.back().y = b;
-                pairs = true;
-            } else {
-                A->sgroups.push_back(make_int4(b, -1, -1, -1));
+        // groups of consecutive slices of one geometry that a backprojector CTA takes together (UDM-PCG only: the
+        // comparison scheme backprojects one basis with its own weights)
+        size_t largest = 1;
+        for (int k = 0; k < 2; ++k) {
+            const int most = k ? 4 : 2;
+            int n = 0;
+            for (int b = 0; b < B; ++b) {
+                if (n > 0 && n < most && same_geometry(geoms[A->sgroups[k].back().x]->desc, geoms[b]->desc)) {
+                    (&A->sgroups[k].back().x)[n++] = b;
+                } else {
+                    A->sgroups[k].push_back(make_int4(b, -1, -1, -1));
+                    n = 1;
+                }
+                largest = std::max(largest, (size_t)n);
             }
         }
-        const bool sg_ok = pairs && P->scheme == DECT_SCHEME_UDM_PCG && P->storage != DECT_STORE_F64;
+        const bool sg_ok = largest > 1 && P->scheme == DECT_SCHEME_UDM_PCG && P->storage != DECT_STORE_F64;
         if (P->bp_slices == 2 && sg_ok) A->sg_cands = {2};
-        else if (P->bp_slices == 0 && sg_ok && P->bp_cluster != 1) A->sg_cands = {1, 2};
-        else A->sg_cands = {1};
+        else if (P->bp_slices == 0 && sg_ok && P->bp_cluster != 1) {
+            A->sg_cands = {1, 2};
+            if (largest > 2 && P->bp_tile != 64) A->sg_cands.push_back(4);  // 32-pixel tiles only
+        } else A->sg_cands = {1};
         A->sweep_sg = A->sg_cands.size() == 1 ? A->sg_cands[0] : 1;
         if (P->storage == DECT_STORE_F64) {
             A->sweep_C = 1;  // the float64 path has its own backprojector; no sweep, no partial images
@@ -1492,15 +1496,18 @@ extern "C" dect_status dect_admm_create(dect_geom* const* geoms, int32_t B, cons
         } else if (P->bp_view_groups < 0) {
             A->sweep_C = sweep_groups(total, tile0);  // occupancy choice, not timed
         } else {
-            // candidates whose partial images fit in 1/16 of the free memory (and 4 GiB)
+            // by the batch's tiles: 12 below 1024 of them, so that a lone small or medium slice fills the chip
+            // (512^2: 0.71 ms per iteration at 10 to 16 groups, 0.76 at 7), 6 from there on (8 slices of 512^2: 2.62
+            // at 6, 2.67 at 4 and 8), as far as the partial images fit in 1/16 of the free memory and 4 GiB. Not
+            // timed: it fixes the order of a pixel's sums, so the same batch gives the same bits on every run.
             size_t free_b = 0, total_b = 0;
             cudaMemGetInfo(&free_b, &total_b);
             const double budget = std::min(4.0 * (1 << 30), (double)free_b / 16.0);
-            const int first = sweep_groups(total, tile0);
-            tune.push_back(first);
-            for (int c : {4, 6, 8, 10, 12, 16})
-                if (c != first && (double)c * pix * sizeof(float2) <= budget) tune.push_back(c);
-            A->sweep_C = *std::max_element(tune.begin(), tune.end());
+            int tiles32 = 0;
+            for (int b = 0; b < B; ++b) tiles32 += sweep_tiles(geoms[b]->desc.nx, geoms[b]->desc.ny, 32);
+            A->sweep_C = tiles32 < 1024 ? 12 : 6;
+            while (A->sweep_C > 1 && (double)A->sweep_C * pix * sizeof(float2) > budget) --A->sweep_C;
+            tune.push_back(A->sweep_C);  // the launch shapes that give the same bits are timed at this C
         }
     }
     int64_t max_np = 0, max_nr = 0;
@@ -1651,9 +1658,11 @@ extern "C" dect_status dect_admm_create(dect_geom* const* geoms, int32_t B, cons
                       &A->prows, &A->pcols})
         if (e == cudaSuccess) e = upload_map(*m, m == &A->sweep ? (size_t)B + 1 : 0);
     if (e == cudaSuccess) e = dalloc(&A->d_groups, groups.size());
-    if (e == cudaSuccess) e = dalloc(&A->d_sgroups, A->sgroups.size());
-    if (e == cudaSuccess)
-        e = cudaMemcpy(A->d_sgroups, A->sgroups.data(), sizeof(int4) * A->sgroups.size(), cudaMemcpyHostToDevice);
+    for (int k = 0; k < 2; ++k) {
+        const std::vector<int4>& sg = A->sgroups[k];
+        if (e == cudaSuccess) e = dalloc(&A->d_sgroups[k], sg.size());
+        if (e == cudaSuccess) e = cudaMemcpy(A->d_sgroups[k], sg.data(), sizeof(int4) * sg.size(), cudaMemcpyHostToDevice);
+    }
     if (e == cudaSuccess)
         e = cudaMemcpy(A->d_groups, groups.data(), sizeof(int4) * groups.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(A->ds, A->hs.data(), sizeof(SliceDesc) * B, cudaMemcpyHostToDevice);
@@ -1670,9 +1679,8 @@ extern "C" dect_status dect_admm_create(dect_geom* const* geoms, int32_t B, cons
         return e == cudaErrorMemoryAllocation ? DECT_ENOMEM : DECT_ECUDA;
     }
     if (A->prec != PREC_F64 && !tune.empty() &&
-        (tune.size() > 1 || tune_tiles.size() > 1 || A->sg_cands.size() > 1 ||
-         (A->cluster_cands.size() > 1 && tune[0] >= 2)))
-        e = autotune_sweep(A, tune, tune_tiles);
+        (tune_tiles.size() > 1 || A->sg_cands.size() > 1 || (A->cluster_cands.size() > 1 && tune[0] >= 2)))
+        e = autotune_sweep(A, tune[0], tune_tiles);
     else if (A->prec != PREC_F64)
         A->sweep_cluster = P->bp_cluster > 0 && A->sweep_sg == 1 && A->sweep_C >= 2 && A->sweep_C <= 16;
     if (e != cudaSuccess) {

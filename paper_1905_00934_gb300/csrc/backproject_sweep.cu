@@ -1,36 +1,31 @@
-// Column-sweep gathering backprojector R^T of the ADMM solver (Table 1's R^T, with the CG
-// epilogues of Eq. 12).
+// Gathering backprojector R^T of the ADMM solver (Table 1's R^T, with the CG epilogues of Eq. 12).
 //
-// A CTA owns a pixel tile (32 x 32 or 64 x 64, see SweepShape) and a group of views; its warps take
-// the rays sampled once per column (axis 0) or once per row (axis 1) over bands of the tile. For each
-// view a warp stages its rays that can reach the tile (32 at a time) in shared memory, in bin
-// order, and walks them; it fetches only the bins of its own axis (each view's axis layout is
-// recorded with the geometry: a view switches axis at most twice). For an axis-0 ray lane c evaluates the sample at column ti + c with the
-// same fixed-point integers as the forward projector and adds (1 - f) w s and f w s to the two rows
-// it interpolates between; for an axis-1 ray lane r does the same for row tj + r. Each lane thus
-// only touches its own column of the warp's accumulator tile ([row][column] for axis 0,
-// [column][row] for axis 1: both free of bank conflicts), every sample is evaluated exactly once,
-// and no atomics are needed. The two tiles are added in a fixed order into this CTA's partial
-// image, and k_bp_finalize adds the C partials of a pixel in a fixed order and applies the
-// epilogue, so results are deterministic for a given C. In the reduced form the last of a tile's C
+// A CTA owns a pixel tile (32 x 32 or 64 x 64) and a group of views. It takes the rays sampled once per
+// column (axis 0) and then those sampled once per row (axis 1): staging warps write the rays of each view that can
+// reach the tile to shared memory, in bin order, and every gathering thread adds to its own pixels, in registers,
+// the staged rays that interpolate them: for axis 0 a block of 4 columns x 2 rows (rows and columns swap for
+// axis 1). The rays of a thread are consecutive bins; their first follows from projecting the block's corners
+// onto the detector, and their number is bounded per view and tile, so every lane of the warp takes the same
+// number. A ray's weight at a pixel is w max(0, 1 - |distance|) from the same fixed-point integers as R, so it is
+// exactly R's interpolation weight, and zero for the rays of the bound that miss the pixel. Every pixel is
+// summed by one thread per axis in the order of views and bins, no atomics; the two axis sums are added in a fixed
+// order into this CTA's partial image, and k_bp_finalize adds the C partials of a pixel in a fixed order and
+// applies the epilogue, so results are deterministic for a given C. In the reduced form the last of a tile's C
 // CTAs to finish (a per-tile arrival counter) forms that same sum while the partials are still in L2,
 // writes it to partial image 0 (the finalize pass then reads one image) and drops the L2 lines of the
 // other partials it consumed, so they are never written back to DRAM.
 //
-// Staging turns a ray into {tile-relative position at lane 0, slope, w s}: the position is
-// q0 + t0 * slope - (a0 << 30) for the tile's first sampled index t0 and first across index a0,
-// an exact integer shift, so a lane's floor and fraction equal those of the forward projector at
-// the same sample. The ray loop runs in blocks of kSwUnroll rays (the stage padded with null rays:
-// far position, zero weight): positions and weights of a block are computed before its
-// accumulator updates, and the next chunk's rays are fetched while the current one is processed.
+// What bounds it: the FP32 pipe (the packed pair instruction takes two cycles of it) with 2.2 of the 5.5 rays a
+// block takes per view weighing anything at a given pixel, then issue. Its predecessor kept the tile's sums in
+// shared memory (each sample a read-modify-write of two rows) and was bound by shared-memory wavefronts; measured
+// on GB300, 512 x 512 x 720 x 1024, both bases, per application: one slice 439 -> 359 us, 8 slices of one
+// geometry 2509 -> 1286 us; 93 x 70 x 61 x 131: 97 -> 8 us (the old kernel's two warps per tile left the chip empty).
 #include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
-#include <mutex>
 #include <type_traits>
-#include <vector>
 
 #include "bp_epilogue.cuh"
 #include "dect_internal.cuh"
@@ -40,21 +35,6 @@
 
 namespace dect {
 
-// A tile is TILE x TILE pixels (TILE = 32 or 64) and its CTA has 2 * TILE / 32 warps: the first
-// TILE / 32 take the rays sampled once per column (axis 0), each for a band of 32 columns x TILE
-// rows, the others the rays sampled once per row (axis 1), each for a band of TILE columns x 32 rows.
-// A taller band leaves fewer lanes idle on rays that clip a corner of it (a CPU model of the 512^2
-// fan workload: 72 % of a staged ray's lanes sample the band at 32 rows, 83 % at 64), at the price of
-// twice the accumulator per warp. Both shapes evaluate every sample once, in the same order per
-// pixel within a view group, and the autotuner of the solver picks one by timing.
-#ifndef DECT_SW_UNROLL
-#define DECT_SW_UNROLL 8
-#endif
-constexpr int kSwUnroll = DECT_SW_UNROLL;  // rays per block of the sweep's inner loop (a multiple of 4)
-// 4 and 8 give the same bits (both measured); 16 ran as fast but its images drifted from theirs within a
-// few iterations, for a reason not found, so it is not allowed.
-static_assert(kSwUnroll == 4 || kSwUnroll == 8, "rays per block: 4 or 8");
-
 // Drop the L2 lines that lie wholly inside [lo, hi) without writing them back (discard.global.L2,
 // 128-byte lines; their contents become undefined). The caller owns every byte of the range.
 __device__ __forceinline__ void discard_l2_range(const void* lo, const void* hi) {
@@ -63,54 +43,185 @@ __device__ __forceinline__ void discard_l2_range(const void* lo, const void* hi)
     for (; a + 128 <= e; a += 128) asm volatile("discard.global.L2 [%0], 128;" ::"l"(a) : "memory");
 }
 
-template <int TILE>
-struct SweepShape {
-    static constexpr int kBands = TILE / 32;      // bands per axis
-    static constexpr int kWarps = 2 * kBands;     // one warp per band and axis
-    static constexpr int kRows = TILE + 2;        // accumulator rows (across index -1 .. TILE; halo discarded)
-    static constexpr int kThreads = 32 * kWarps;
+// A gathering thread's pixels: kPix along the across direction by kCols sampled indices. A staged ray that the
+// thread loads serves all of them. A model of the 512^2 fan workload (rays per thread, products per pixel) and
+// trials put 2 x 4 ahead of 4 x 1, 4 x 2, 2 x 2 and 2 x 8: more rows multiply the products with a zero weight,
+// fewer columns the loads, positions and searches.
+constexpr int kPix = 2;
+constexpr int kCols = 4;
+constexpr int kStages = 2;      // batches of staged rays in flight
+constexpr int kBatchSegs = 16;  // views (segments) per batch at most
+
+template <int TILE, int NCH, int SG>
+struct GatherShape {
+    static constexpr int kBands = TILE / 32;                      // bands of 32 sampled indices
+    static constexpr int kGather = TILE * TILE / (kPix * kCols);  // threads that gather
+    static constexpr int kProd = TILE == 64 ? 128 : 32;           // threads that stage (two warps: no gain)
+    static constexpr int kThreads = kGather + kProd;
+    static constexpr int kCap = TILE == 64 ? 512 : 256;  // rays per batch (128 and 512 measured alike)
+    static constexpr int kPitch = TILE + 1;              // row pitch of the accumulator tile
+    static constexpr int kCh = NCH * SG;                 // channels per staged ray
+    static constexpr int kVec = kCh < 4 ? kCh : 4;       // channels per staged vector
+    // rays per trip of the gather loop and CTAs per SM the register allocation must allow, measured together (one
+    // slice: 362 us at 3 and 5, 392 at 2 and 6, 428 at 1 and 8; two: 3.16 ms per iteration of 8 slices at 1 and 5,
+    // 3.39 at 2 and 4; four: 2.62 at 2 and 3, 2.69 at 4 and 3, 2.88 at 1 and 4)
+    static constexpr int kUnroll = SG == 1 ? 3 : (SG == 2 ? 1 : 2);
+    static constexpr int kMinCtas = TILE == 64 ? 1 : (SG == 4 ? 3 : 5);
+    // stages of {w s} and of {position, slope} per band, their segment lists, the accumulator tiles
+    static constexpr size_t kStageW = kStages * (size_t)kCap * kCh * sizeof(float);
+    static constexpr size_t kStageP = kStages * (size_t)kCap * kBands * sizeof(int4);
+    static constexpr size_t kSegs = kStages * (kBatchSegs + 1) * sizeof(int4);
+    static constexpr size_t kTile = (size_t)TILE * kPitch * kCh * sizeof(float);
+    static constexpr size_t kBytes = kStageW + kStageP + kSegs + kTile;
 };
 
-// shared-memory bytes of a CTA's accumulators (dynamic shared memory), SG slices per CTA
-template <int TILE, int NCH, int SG = 1>
-constexpr size_t sweep_acc_bytes() {
-    return (size_t)SG * SweepShape<TILE>::kWarps * SweepShape<TILE>::kRows * 32 *
-           (NCH == 2 ? sizeof(float2) : sizeof(float));
+// 1 / x to about an ulp (x a distance from a fan source, far from the ends of float's range)
+__device__ __forceinline__ float rcp_approx(float x) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
 }
 
-// NCH = 2: sinogram S2 pairs {c, p}, float2 accumulators and partial images. NCH = 1: float sinogram,
-// float accumulators (half the shared-memory traffic), optionally multiplied per ray by rw[ray] and per
-// slice by scale[slice] as the rays are staged (the weighted R^T of a Gauss-Newton operator).
-// CLUSTER: the C CTAs of a tile (consecutive blocks) form a thread-block cluster and add their
-// accumulators through distributed shared memory, in rank order, into one partial image (image 0);
-// the sum per pixel is the one the finalize pass forms from C partial images (0 + p_0 + p_1 + ...),
-// so both launch forms give the same bits, and only one image per tile goes through L2 and DRAM.
-// SG = 2: a CTA backprojects the same rays into two slices of one geometry (their indices in
-// groups[unit], the second -1 if the group has one slice): staging, candidate search and sample
-// positions are done once, each slice has its own accumulators, and each slice's pixels receive the
-// same contributions in the same order as with SG = 1 (the same bits). NCH = 2, plain form only.
-// tile_count != nullptr (plain form): the reduced form. One counter per tile of the launch (block /
-// C), zero on entry; the tile's last CTA adds 0 + p_0 + ... + p_{C-1} per pixel, the finalize pass's
-// sum, into image 0 and sets the counter back to zero.
+// Named barriers with constant numbers (a number in a register reserves all sixteen, of 64 per SM).
+template <int ID, int THREADS>
+__device__ __forceinline__ void bar_sync() {
+    asm volatile("bar.sync %0, %1;" ::"n"(ID), "n"(THREADS) : "memory");
+}
+template <int ID, int THREADS>
+__device__ __forceinline__ void bar_arrive() {
+    asm volatile("bar.arrive %0, %1;" ::"n"(ID), "n"(THREADS) : "memory");
+}
+// barriers ID (stage 0) and ID + 1 (stage 1)
+template <int ID, int THREADS>
+__device__ __forceinline__ void stage_sync(int s) {
+    if (s) bar_sync<ID + 1, THREADS>(); else bar_sync<ID, THREADS>();
+}
+template <int ID, int THREADS>
+__device__ __forceinline__ void stage_arrive(int s) {
+    if (s) bar_arrive<ID + 1, THREADS>(); else bar_arrive<ID, THREADS>();
+}
+
+template <int N>
+struct VecF;
+template <>
+struct VecF<1> { using T = float; };
+template <>
+struct VecF<2> { using T = float2; };
+template <>
+struct VecF<4> { using T = float4; };
+
+__device__ __forceinline__ void unpack_vec(float v, float* x) { x[0] = v; }
+__device__ __forceinline__ void unpack_vec(float2 v, float* x) { x[0] = v.x; x[1] = v.y; }
+__device__ __forceinline__ void unpack_vec(float4 v, float* x) { x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w; }
+
+// Adds n staged rays to a thread's pixels. pos: a ray's 34.30 fixed-point position at the first index of the
+// band, relative to the tile's edge, and its slope; along0: the thread's first index in the band; p0: its first
+// pixel's across index in the tile. The position shifted left by 25 has the whole part and the 23 fraction bits
+// of the weight in its high word, so one 64-bit addition per index gives the exact distance d to pixel 0 in units
+// of 2^-23 pixel (the forward projector's floor and fraction); pixel p takes max(0, 1 - |d 2^-23 - p|): 1 - f or
+// f of the ray's two neighbours, exactly, and 0 elsewhere. GUARD: pixels that a ray does not interpolate are
+// skipped instead of taking a zero product, so that an infinite or NaN ray reaches only its own pixels.
+template <int CH, int VEC, int CAP, int UNROLL, bool GUARD>
+__device__ __forceinline__ void gather_rays(const int4* __restrict__ pos, const typename VecF<VEC>::T* __restrict__ w,
+                                            int n, int along0, int p0, f32x2 (&acc)[kCols][CH]) {
+#pragma unroll UNROLL
+    for (int r = 0; r < n; ++r) {
+        const int4 P = pos[r];
+        float x[CH];
+#pragma unroll
+        for (int q = 0; q < CH / VEC; ++q) unpack_vec(w[r + q * CAP], x + q * VEC);
+        const long long q0 = ray_pos(P, along0);
+        int hi = (int)(q0 >> 7) - (p0 << 23);
+        unsigned lo = (unsigned)q0 << 25;
+        const int shi = P.z >> 7;
+        const unsigned slo = (unsigned)P.z << 25;
+        f32x2 xx[CH];
+#pragma unroll
+        for (int q = 0; q < CH; ++q) xx[q] = pack2(x[q], x[q]);
+#pragma unroll
+        for (int j = 0; j < kCols; ++j) {
+            if (j > 0)
+                asm("add.cc.u32 %0, %0, %2; addc.s32 %1, %1, %3;" : "+r"(lo), "+r"(hi) : "r"(slo), "r"(shi));
+            const float t0 = (float)hi * 0x1p-23f, t1 = t0 - 1.0f;
+            const float h0 = __saturatef(1.0f - fabsf(t0)), h1 = __saturatef(1.0f - fabsf(t1));
+            if (GUARD) {
+                const bool in0 = t0 >= -1.0f && t0 < 1.0f, in1 = t1 >= -1.0f && t1 < 1.0f;
+#pragma unroll
+                for (int q = 0; q < CH; ++q) {
+                    const float2 o = unpack2(acc[j][q]);
+                    acc[j][q] = pack2(in0 ? fmaf(h0, x[q], o.x) : o.x, in1 ? fmaf(h1, x[q], o.y) : o.y);
+                }
+            } else {
+                const f32x2 h = pack2(h0, h1);
+#pragma unroll
+                for (int q = 0; q < CH; ++q) acc[j][q] = fma2(h, xx[q], acc[j][q]);
+            }
+        }
+    }
+}
+
+// Slack of the bin bounds: absorbs float32 rounding and the rays' fixed-point quantisation (both far below)
+constexpr float kBinEps = 0.02f;
+
+// An upper bound of the bins whose rays cross the rectangle of one gathering thread (kPix + 1 pixels across by
+// kCols - 1 along), anywhere in the tile's rectangle of half-sides (ha, hb) centred at (a, b) cm (along, across),
+// for a view with direction n = (cx, cy) along and across. A larger count only adds rays of zero weight.
+// Fan: with r = s n + u t the vector to the source (t normal to n), the derivatives of the bin with respect to
+// across and along are k1 |r_along| / s^2 and k1 |r_across| / s^2, so the width is k1 pix (A s + B u) / s^2 with A
+// and B fixed by the signs of r's components where the tile has one sign of each; A / s and B u / s^2 are
+// bounded at the tile's ends of s and u.
+__device__ __forceinline__ int window_bins(const GeomDev& g, float cx, float cy, float a, float b, float ha, float hb) {
+    constexpr float kA = (float)(kPix + 1), kL = (float)(kCols - 1);
+    float w;
+    if (g.kind == DECT_PARALLEL) {
+        w = g.inv_du * fmaf(kA, fabsf(cy), kL * fabsf(cx)) * g.pix;
+    } else {
+        const float ra = g.sod * cx - a, rb = g.sod * cy - b;
+        const float s = g.sod - fmaf(a, cx, b * cy), hs = fmaf(ha, fabsf(cx), hb * fabsf(cy));
+        const float s0 = s - hs, s1 = s + hs, i0 = s0 > 0.f ? 1.f / s0 : 1e9f;
+        const float ka = copysignf(kA, ra), kl = copysignf(kL, rb);
+        const float A = fmaf(ka, cx, kl * cy), B = fmaf(kl, cx, -ka * cy);
+        const float Bu = fmaf(B, fmaf(rb, cx, -ra * cy), fabsf(B) * fmaf(ha, fabsf(cy), hb * fabsf(cx)));
+        if (fabsf(ra) > ha && fabsf(rb) > hb && A >= 0.f)
+            w = A * i0 + (Bu > 0.f ? Bu * i0 * i0 : Bu / (s1 * s1));
+        else
+            w = fmaf(kA, fabsf(ra) + ha, kL * (fabsf(rb) + hb)) * i0 * i0;
+        w *= g.k1 * g.pix;
+    }
+    return (int)fminf(fmaf(w, 1.0005f, 2.f * kBinEps), 1022.f) + 1;
+}
+
+// NCH = 2: sinogram S2 pairs {c, p}, float2 partial images. NCH = 1: float sinogram and partial images,
+// optionally multiplied per ray by rw[ray] and per slice by scale[slice] as the rays are staged (the weighted R^T
+// of a Gauss-Newton operator).
+// CLUSTER: the C CTAs of a tile (consecutive blocks) form a thread-block cluster and add their tiles through
+// distributed shared memory, in rank order, into one partial image (image 0); the sum per pixel is the one the
+// finalize pass forms from C partial images (0 + p_0 + p_1 + ...), so both launch forms give the same bits, and
+// only one image per tile goes through L2 and DRAM.
+// SG = 2, 4: a CTA backprojects the same rays into up to SG slices of one geometry (their indices in
+// groups[unit], -1 past the group's size): staging, positions, weights and searches are done once, and each slice's
+// pixels receive the same contributions in the same order as with SG = 1 (the same bits). NCH = 2, plain form only.
+// tile_count != nullptr (plain form): the reduced form. One counter per tile of the launch (block / C), zero on
+// entry; the tile's last CTA adds 0 + p_0 + ... + p_{C-1} per pixel, the finalize pass's sum, into image 0 and
+// sets the counter back to zero.
 template <class S2, int NCH, int TILE, bool CLUSTER = false, int SG = 1>
-__global__ void __launch_bounds__(SweepShape<TILE>::kThreads) k_bp_sweep(
+__global__ void __launch_bounds__(GatherShape<TILE, NCH, SG>::kThreads, GatherShape<TILE, NCH, SG>::kMinCtas) k_bp_gather(
     const SliceDesc* __restrict__ dsl, BlockMap map, int C, const int4* __restrict__ groups,
     const S2* __restrict__ sino, typename std::conditional<NCH == 2, float2, float>::type* __restrict__ partial,
     int64_t stride, const float* __restrict__ rw, const float* __restrict__ scale, int* __restrict__ tile_count) {
-    static_assert(SG == 1 || (SG == 2 && NCH == 2 && !CLUSTER), "two slices per CTA: two channels, plain form");
+    static_assert(SG == 1 || (NCH == 2 && !CLUSTER), "several slices per CTA: two channels, plain form");
     using Acc = typename std::conditional<NCH == 2, float2, float>::type;
-    using Sh = SweepShape<TILE>;
-    // [slice][warp][across index + 1][lane]: [row][column] for axis 0, [column][row] for axis 1
-    extern __shared__ __align__(16) unsigned char sweep_smem[];
-    Acc(*acc_all)[Sh::kWarps][Sh::kRows][32] = reinterpret_cast<Acc(*)[Sh::kWarps][Sh::kRows][32]>(sweep_smem);
-    Acc(*acc)[Sh::kRows][32] = acc_all[0];
-    // SG = 2: one float4 {c, p of the first slice, c, p of the second} per accumulator cell, so a sample's
-    // update of both slices is one 16-byte read-modify-write per row (the same bytes as two 8-byte ones)
-    float4(*acc4)[Sh::kRows][32] = reinterpret_cast<float4(*)[Sh::kRows][32]>(sweep_smem);
-    __shared__ int4 st_ray[Sh::kWarps][32];                 // {position lo, position hi, slope, w s_c}
-    __shared__ __align__(16) float st_wp[Sh::kWarps][32];   // w s_p (SG = 1)
-    // SG = 2: {w s_c, w s_p, w s_c', w s_p'} of both slices, as two packed pairs for the accumulator update
-    __shared__ float4 st_w2[SG == 2 ? Sh::kWarps : 1][32];
+    using Sh = GatherShape<TILE, NCH, SG>;
+    using Vec = typename VecF<Sh::kVec>::T;
+    constexpr int CAP = Sh::kCap, BANDS = Sh::kBands, PITCH = Sh::kPitch, CH = Sh::kCh, NV = CH / Sh::kVec;
+    extern __shared__ __align__(16) unsigned char smem[];
+    Vec* st_w = reinterpret_cast<Vec*>(smem);                    // [kStages][NV][CAP]
+    int4* st_pos = reinterpret_cast<int4*>(smem + Sh::kStageW);  // [kStages][BANDS][CAP]
+    // [kStages][kBatchSegs + 1]: {flags, 0, 0, 0} then a segment each: the view's (cos, sin) along and across,
+    // stage index minus bin, first and end stage index
+    int4* segs = reinterpret_cast<int4*>(smem + Sh::kStageW + Sh::kStageP);
+    Acc* tile_acc = reinterpret_cast<Acc*>(smem + Sh::kStageW + Sh::kStageP + Sh::kSegs);  // [SG][TILE][PITCH]
+
     int local;
     const int unit = slice_of(map, blockIdx.x, local);
     int sl[SG];
@@ -119,202 +230,285 @@ __global__ void __launch_bounds__(SweepShape<TILE>::kThreads) k_bp_sweep(
         sl[0] = unit;
     } else {
         const int4 gs = __ldg(groups + unit);
-        sl[0] = gs.x;
-        sl[1] = gs.y >= 0 ? gs.y : gs.x;
-        count = gs.y >= 0 ? 2 : 1;
+        const int all[4] = {gs.x, gs.y, gs.z, gs.w};
+        count = 1 + (gs.y >= 0) + (SG > 2 ? (gs.z >= 0) + (gs.w >= 0) : 0);
+#pragma unroll
+        for (int q = 0; q < SG; ++q) sl[q] = q < count ? all[q] : gs.x;
     }
-    const int s = sl[0];
-    const SliceDesc& d = dsl[s];
+    const SliceDesc& d = dsl[sl[0]];
     const GeomDev& g = d.g;
     const int nx = g.nx, ny = g.ny;
     const int c = local % C, tile = local / C;
     const int tiles_x = (nx + TILE - 1) / TILE;
     const int ti = (tile % tiles_x) * TILE, tj = (tile / tiles_x) * TILE;
-    const int w = threadIdx.x / 32, lane = threadIdx.x % 32;
-    const bool my_axis = w >= Sh::kBands;
-    const int band = w % Sh::kBands;
-    if constexpr (SG == 2) {
-        for (int r = 0; r < Sh::kRows; ++r) acc4[w][r][lane] = make_float4(0.f, 0.f, 0.f, 0.f);
-    } else {
-        for (int r = 0; r < Sh::kRows; ++r) acc[w][r][lane] = Acc{};
-    }
-    const int G = C, grp = c;
-    // this warp's band: 32 sampled indices from bi (columns for axis 0, rows for axis 1) by the tile's
-    // TILE across indices from ba; rays with a weight at its in-image pixels pass within one pixel of
-    // their centres, so candidates come from the band's rectangle widened by one pixel (inside the
-    // image's one-pixel margin, in front of a fan source)
-    const int bi = (my_axis ? tj : ti) + 32 * band, ba = my_axis ? ti : tj;
-    const int n_along = my_axis ? ny : nx, n_across = my_axis ? nx : ny;
-    const int be = min(bi + 32, n_along) - 1, ae = min(ba + TILE, n_across) - 1;
-    const bool empty = bi >= n_along;  // a band past the image's last column / row (ragged tiles)
-    const int i0 = my_axis ? ba : bi, i1 = my_axis ? ae : be, j0 = my_axis ? bi : ba, j1 = my_axis ? be : ae;
-    const float xc = (0.5f * (float)(i0 + i1) - g.cx) * g.pix, yc = (0.5f * (float)(j0 + j1) - g.cy) * g.pix;
-    const float hx = (0.5f * (float)(i1 - i0) + 1.0f) * g.pix, hy = (0.5f * (float)(j1 - j0) + 1.0f) * g.pix;
-    const S2* sn = sino + d.sino_off;
-    const S2* sn1 = sino + dsl[sl[SG - 1]].sino_off;  // the second slice's sinogram (SG = 2)
-    const long long a0q = (long long)ba << 30;
+    const int tid = threadIdx.x, lane = tid % 32;
+    constexpr int kFull = 1, kEmpty = kFull + kStages, kAxis = kEmpty + kStages;  // named barriers
 
-    // chunk cursor: view v, first bin k0 of the chunk, last bin khi of the current candidate interval,
-    // [k2, k2hi] a second interval of the view still to come. A view's candidates are the bins whose
-    // rays can reach the band, restricted to the bins of this warp's axis (the view's axis layout), so
-    // the warp fetches only rays it stages; the rays keep their bin order.
-    int v = empty ? g.nv : grp, k0 = 0, khi = -1, k2 = 1, k2hi = 0;
-    auto seek = [&](int vv) {
-        for (v = vv; v < g.nv; v += G) {
-            const float4 V = __ldg(g.views + v);
-            const CandRange cr = rect_candidates(g, V.x, V.y, xc, yc, hx, hy);
-            if (cr.lo > cr.hi) continue;
-            int a1 = 0, b1 = g.nb - 1, a2 = 1, b2 = 0;  // a mixed layout: every bin, one interval
-            if (V.w >= 0.f && fabsf(V.z) >= 1.f) {
-                const bool ax0 = V.z < 0.f;
-                const int s1 = (int)fabsf(V.z) - 1, s2 = (int)V.w;
-                if (ax0 == my_axis) {
-                    b1 = s1 - 1;
-                    a2 = s2;
-                    b2 = g.nb - 1;
-                } else {
-                    a1 = s1;
-                    b1 = s2 - 1;
+    if (tid >= Sh::kGather) {
+        // ---- staging warps: list the bins that can reach the tile, view by view, and stage their rays ----
+        const int ptid = tid - Sh::kGather;
+        const S2* sn[SG];
+#pragma unroll
+        for (int q = 0; q < SG; ++q) sn[q] = sino + dsl[sl[q]].sino_off;
+        const float sscale = (NCH == 1 && scale) ? __ldg(scale + sl[0]) : 1.0f;
+        // the tile's rectangle (clipped to the image) widened by one pixel: a ray with a weight at one of its
+        // pixels passes through it (inside the image's one-pixel margin, in front of a fan source)
+        const int te = min(ti + TILE, nx) - 1, tf = min(tj + TILE, ny) - 1;
+        const float xc = (0.5f * (float)(ti + te) - g.cx) * g.pix, yc = (0.5f * (float)(tj + tf) - g.cy) * g.pix;
+        const float hx = (0.5f * (float)(te - ti) + 1.0f) * g.pix, hy = (0.5f * (float)(tf - tj) + 1.0f) * g.pix;
+        int batch = 0;  // batches published so far (both axes)
+        int fill = 0, nseg = 0;
+        float check = 0.f;  // becomes NaN with the first non-finite product
+        // the rays being fetched: kRays per lane, at stage indices p_at + lane + 32 i below p_at + p_n (the staging
+        // warps take the segments of a batch in turn)
+        constexpr int kRays = 2;
+        int4 P[kRays];
+        float x[kRays][CH];
+        int p_at = 0, p_n = 0, axis = 0;
+        bool p_mixed = false;
+        auto flush = [&]() {  // stages them
+            const int t0 = axis ? tj : ti;
+            const long long a0q = (long long)(axis ? ti : tj) << 30;
+            const int s = batch % kStages;
+#pragma unroll
+            for (int i = 0; i < kRays; ++i) {
+                const int r = lane + 32 * i;
+                if (r >= p_n) break;
+                const float w = ray_w(P[i]) * sscale;
+#pragma unroll
+                for (int q = 0; q < CH; ++q) {
+                    x[i][q] *= w;
+                    check = fmaf(x[i][q], 0.f, check);
                 }
+                // 34.30 fixed point at the band's first index, relative to the tile's edge
+                int4 p[BANDS];
+#pragma unroll
+                for (int b = 0; b < BANDS; ++b) {
+                    const long long q = ray_pos(P[i], t0 + 32 * b) - a0q;
+                    p[b] = make_int4((int)(unsigned)(unsigned long long)q, (int)(q >> 32), P[i].z, 0);
+                }
+                if (p_mixed && ray_axis(P[i]) != (axis != 0)) {  // the other axis' ray: a null one, far off
+#pragma unroll
+                    for (int q = 0; q < CH; ++q) x[i][q] = 0.f;
+#pragma unroll
+                    for (int b = 0; b < BANDS; ++b) p[b] = make_int4(0, -25, 0, 0);
+                }
+                Vec* w_to = st_w + s * NV * CAP + p_at + r;
+#pragma unroll
+                for (int q = 0; q < NV; ++q) {
+                    if constexpr (Sh::kVec == 1) w_to[0] = x[i][0];
+                    else if constexpr (Sh::kVec == 2) w_to[0] = make_float2(x[i][0], x[i][1]);
+                    else w_to[q * CAP] = make_float4(x[i][4 * q], x[i][4 * q + 1], x[i][4 * q + 2], x[i][4 * q + 3]);
+                }
+#pragma unroll
+                for (int b = 0; b < BANDS; ++b) st_pos[(s * BANDS + b) * CAP + p_at + r] = p[b];
             }
-            const int l1 = max(cr.lo, a1), h1 = min(cr.hi, b1), l2 = max(cr.lo, a2), h2 = min(cr.hi, b2);
-            if (l1 <= h1) {
-                k0 = l1;
-                khi = h1;
-                k2 = l2;
-                k2hi = h2;
-                return;
-            }
-            if (l2 <= h2) {
-                k0 = l2;
-                khi = h2;
-                k2 = 1;
-                k2hi = 0;
-                return;
-            }
-        }
-    };
-    if (!empty) seek(grp);
-    int4 P = make_int4(0, 0, 0, 0);
-    float2 sv = make_float2(0.f, 0.f), sv1 = make_float2(0.f, 0.f);
-    bool have = false;
-    auto fetch = [&]() {
-        const int k = k0 + lane;
-        have = v < g.nv && k <= khi;
-        if (have) {
-            const size_t e = (size_t)v * g.nb + k;
-            P = __ldg(g.rays + e);
-            if constexpr (NCH == 2) {
-                sv = ldg2(sn + e);
-                if constexpr (SG == 2) sv1 = count > 1 ? ldg2(sn1 + e) : make_float2(0.f, 0.f);
+            p_n = 0;
+        };
+        auto publish = [&](int flags) {
+            flush();
+            const int s = batch % kStages;
+            const bool bad = __any_sync(0xffffffffu, check != 0.f);
+            if (lane == 0 && bad) flags |= 2;
+            if constexpr (Sh::kProd > 32) {
+                // (every staging warp may have seen a non-finite product)
+                bar_sync<kAxis + 1, Sh::kProd>();
+                if (lane == 0 && (flags & 2)) atomicOr(&segs[s * (kBatchSegs + 1)].y, 1);
+                bar_sync<kAxis + 1, Sh::kProd>();
+                if (ptid == 0) {
+                    int4& h = segs[s * (kBatchSegs + 1)];
+                    h.x = nseg | (flags & 1) << 16 | (h.y ? 2 << 16 : 0);
+                    h.y = 0;
+                }
             } else {
-                sv.x = __ldg(sn + e);
-                if (rw) sv.x *= __ldg(rw + d.sino_off + e);
+                if (ptid == 0) segs[s * (kBatchSegs + 1)].x = nseg | flags << 16;
             }
-        }
-    };
-    fetch();
-    const float sscale = (NCH == 1 && scale) ? __ldg(scale + s) : 1.0f;
-    while (v < g.nv) {
-        // stage this warp's rays of the fetched chunk, compacted in bin order
-        const bool mine = have && ray_axis(P) == my_axis;
-        const unsigned mask = __ballot_sync(0xffffffffu, mine);
-        const int n = __popc(mask);
-        if (mine) {
-            const long long q = ray_pos(P, bi) - a0q;
-            const float wr = ray_w(P) * sscale;
-            const int at = __popc(mask & ((1u << lane) - 1u));
-            st_ray[w][at] = make_int4((int)(unsigned)(unsigned long long)q, (int)(q >> 32), P.z, __float_as_int(wr * sv.x));
-            if constexpr (SG == 1)
-                st_wp[w][at] = wr * sv.y;
-            else
-                st_w2[w][at] = make_float4(wr * sv.x, wr * sv.y, wr * sv1.x, wr * sv1.y);
-        }
-        const int nr = (n + kSwUnroll - 1) / kSwUnroll * kSwUnroll;
-        if (lane >= n && lane < nr) {  // null rays pad the stage to a multiple of kSwUnroll
-            st_ray[w][lane] = make_int4(0, -1000 << 2, 0, 0);
-            if constexpr (SG == 1)
-                st_wp[w][lane] = 0.f;
-            else
-                st_w2[w][lane] = make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-        // advance the cursor and fetch the next chunk while this one is processed
-        k0 += 32;
-        if (k0 > khi) {
-            if (k2 <= k2hi) {
-                k0 = k2;
-                khi = k2hi;
-                k2 = 1;
-                k2hi = 0;
-            } else {
-                seek(v + G);
-            }
-        }
-        fetch();
-        __syncwarp();
-        for (int r0 = 0; r0 < nr; r0 += kSwUnroll) {
-            int hh[kSwUnroll];
-            float ff[kSwUnroll], wc[kSwUnroll], wp[kSwUnroll];
-            if constexpr (NCH == 2 && SG == 1) {  // w s_p of the block's rays: broadcast 16-byte loads
-#pragma unroll
-                for (int v4 = 0; v4 < kSwUnroll / 4; ++v4) {
-                    const float4 p = *reinterpret_cast<const float4*>(&st_wp[w][r0 + 4 * v4]);
-                    wp[4 * v4] = p.x;
-                    wp[4 * v4 + 1] = p.y;
-                    wp[4 * v4 + 2] = p.z;
-                    wp[4 * v4 + 3] = p.w;
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < kSwUnroll; ++u) {
-                const int4 S = st_ray[w][r0 + u];
-                const long long q = ((((long long)S.y) << 32) | (long long)(unsigned)S.x) + (long long)lane * S.z;
-                hh[u] = pos_floor(q);
-                ff[u] = frac_of(q);
-                wc[u] = __int_as_float(S.w);
-            }
-            if constexpr (SG == 2) {
-                // both slices' weights per ray; a row's four sums {c, p, c', p'} advance as two packed
-                // float32 pairs (fma.rn.f32x2, each element rounded as fmaf)
-#pragma unroll
-                for (int u = 0; u < kSwUnroll; ++u) {
-                    const float4 x = st_w2[w][r0 + u];
-                    if ((unsigned)(hh[u] + 1) < (unsigned)(TILE + 1)) {
-                        float4* a = &acc4[w][hh[u] + 1][lane];
-                        const float4 x0 = a[0], x1 = a[32];
-                        const f32x2 g0 = pack2(1.0f - ff[u], 1.0f - ff[u]), g1 = pack2(ff[u], ff[u]);
-                        const f32x2 w01 = pack2(x.x, x.y), w23 = pack2(x.z, x.w);
-                        const float2 y00 = unpack2(fma2(g0, w01, pack2(x0.x, x0.y)));
-                        const float2 y01 = unpack2(fma2(g0, w23, pack2(x0.z, x0.w)));
-                        const float2 y10 = unpack2(fma2(g1, w01, pack2(x1.x, x1.y)));
-                        const float2 y11 = unpack2(fma2(g1, w23, pack2(x1.z, x1.w)));
-                        a[0] = make_float4(y00.x, y00.y, y01.x, y01.y);
-                        a[32] = make_float4(y10.x, y10.y, y11.x, y11.y);
-                    }
-                }
-                continue;
-            }
-#pragma unroll
-            for (int u = 0; u < kSwUnroll; ++u) {
-                // rows h, h+1 with h in [-1, TILE - 1] are accumulator rows h+1, h+2 (lanes outside skip)
-                if ((unsigned)(hh[u] + 1) < (unsigned)(TILE + 1)) {
-                    Acc* a = &acc[w][hh[u] + 1][lane];
-                    if constexpr (NCH == 2) {
-                        float2 x0 = a[0], x1 = a[32];
-                        x0.x = fmaf(1.0f - ff[u], wc[u], x0.x);
-                        x0.y = fmaf(1.0f - ff[u], wp[u], x0.y);
-                        x1.x = fmaf(ff[u], wc[u], x1.x);
-                        x1.y = fmaf(ff[u], wp[u], x1.y);
-                        a[0] = x0;
-                        a[32] = x1;
+            stage_arrive<kFull, Sh::kThreads>(s);
+            ++batch;
+            fill = nseg = 0;
+            check = 0.f;
+            if (batch >= kStages) stage_sync<kEmpty, Sh::kThreads>(batch % kStages);  // the next stage is free
+        };
+        if constexpr (Sh::kProd > 32)
+            if (ptid < kStages) segs[ptid * (kBatchSegs + 1)].y = 0;
+#pragma unroll 1
+        for (axis = 0; axis < 2; ++axis) {
+#pragma unroll 1
+            for (int vb = c; vb < g.nv; vb += 32 * C) {
+                // one view per lane: its one or two intervals of candidate bins
+                const int v = vb + C * lane;
+                int l1 = 0, n1 = 0, l2 = 0, n2 = 0, win = 0;
+                float cx = 0.f, cy = 0.f;
+                if (v < g.nv) {
+                    const float4 V = __ldg(g.views + v);
+                    cx = axis ? V.y : V.x;  // along and across the sampled direction
+                    cy = axis ? V.x : V.y;
+                    win = window_bins(g, cx, cy, axis ? yc : xc, axis ? xc : yc, axis ? hy : hx, axis ? hx : hy);
+                    const CandRange cr = rect_candidates(g, V.x, V.y, xc, yc, hx, hy);
+                    int a1 = 0, b1 = g.nb - 1, a2 = 1, b2 = 0;  // a mixed layout: every bin, one interval
+                    if (!(V.w >= 0.f && fabsf(V.z) >= 1.f)) {
+                        win |= 1 << 30;
                     } else {
-                        a[0] = fmaf(1.0f - ff[u], wc[u], a[0]);
-                        a[32] = fmaf(ff[u], wc[u], a[32]);
+                        const int s1 = (int)fabsf(V.z) - 1, s2 = (int)V.w;
+                        if ((V.z < 0.f) == (axis != 0)) {
+                            b1 = s1 - 1;
+                            a2 = s2;
+                            b2 = g.nb - 1;
+                        } else {
+                            a1 = s1;
+                            b1 = s2 - 1;
+                        }
+                    }
+                    l1 = max(cr.lo, a1);
+                    n1 = max(0, min(cr.hi, b1) - l1 + 1);
+                    l2 = max(cr.lo, a2);
+                    n2 = max(0, min(cr.hi, b2) - l2 + 1);
+                }
+                for (unsigned todo = __ballot_sync(0xffffffffu, n1 > 0 || n2 > 0); todo; todo &= todo - 1) {
+                    const int src = __ffs(todo) - 1;
+                    const float vx = __shfl_sync(0xffffffffu, cx, src), vy = __shfl_sync(0xffffffffu, cy, src);
+                    const int vw = __shfl_sync(0xffffffffu, win, src), vwin = vw & 0xffff;
+                    const bool mixed = vw >> 30;
+                    const int4 iv = make_int4(__shfl_sync(0xffffffffu, l1, src), __shfl_sync(0xffffffffu, n1, src),
+                                              __shfl_sync(0xffffffffu, l2, src), __shfl_sync(0xffffffffu, n2, src));
+                    const unsigned row = (unsigned)(vb + C * src) * (unsigned)g.nb;
+#pragma unroll 1
+                    for (int part = 0; part < 2; ++part) {
+                        int k0 = part ? iv.z : iv.x, left = part ? iv.w : iv.y;
+                        while (left > 0) {
+                            // a segment that does not fit goes to the next batch, whole if it can
+                            if (nseg == kBatchSegs || (fill > 0 && left > CAP - fill)) publish(0);
+                            const int take = min(left, CAP - fill), s = batch % kStages;
+                            const bool my_turn = Sh::kProd == 32 || nseg % (Sh::kProd / 32) == ptid / 32;
+                            for (int r0 = 0; my_turn && r0 < take; r0 += kRays * 32) {
+                                // (the loads of these rays are in flight until the next ones' turn)
+                                flush();
+#pragma unroll
+                                for (int i = 0; i < kRays; ++i) {
+                                    const unsigned e = row + (unsigned)(k0 + min(r0 + lane + 32 * i, take - 1));
+                                    P[i] = __ldg(g.rays + e);
+                                    if constexpr (NCH == 2) {
+#pragma unroll
+                                        for (int q = 0; q < SG; ++q) {
+                                            const float2 sv = q < count ? ldg2(sn[q] + e) : make_float2(0.f, 0.f);
+                                            x[i][2 * q] = sv.x;
+                                            x[i][2 * q + 1] = sv.y;
+                                        }
+                                    } else {
+                                        x[i][0] = __ldg(sn[0] + e);
+                                        if (rw) x[i][0] *= __ldg(rw + d.sino_off + e);
+                                    }
+                                }
+                                p_at = fill + r0;
+                                p_n = take - r0;
+                                p_mixed = mixed;
+                            }
+                            const int n = min(vwin, take);
+                            if (ptid == 0)
+                                segs[s * (kBatchSegs + 1) + 1 + nseg] =
+                                    make_int4(__float_as_int(vx), __float_as_int(vy), (fill - k0) * 1024 + n,
+                                              fill | (fill + take - n) << 16);
+                            ++nseg;
+                            fill += take;
+                            k0 += take;
+                            left -= take;
+                        }
                     }
                 }
             }
+            publish(1);  // the axis' last batch (maybe without segments)
         }
-        __syncwarp();  // the stage is rewritten by the next chunk
+        static_assert(kStages == 2, "one batch is left unwaited for here");
+        stage_sync<kEmpty, Sh::kThreads>((batch - 1) % kStages);
+    } else {
+        // ---- gathering warps: 8 threads along a band of 32 sampled indices by 4 along the across direction ----
+        const int warp = tid / 32;
+        const int band = warp % BANDS, blk = 4 * (warp / BANDS) + lane / 8, along0 = kCols * (lane % 8);
+        int batch = 0;
+#pragma unroll 1
+        for (int axis = 0; axis < 2; ++axis) {
+            // this thread's pixels: sampled indices t .. t + kCols - 1 (columns for axis 0, rows for axis 1),
+            // across indices a .. a + kPix - 1
+            const int t = (axis ? tj : ti) + 32 * band + along0, a = (axis ? ti : tj) + kPix * blk;
+            const int n_along = axis ? ny : nx, n_across = axis ? nx : ny;
+            const bool idle = t - along0 >= n_along || a - kPix * (lane / 8) >= n_across;  // warp-uniform
+            // rays with a weight at them cross the rectangle of these corners (cm; past the image's edge: its edge)
+            const float ca = axis ? g.cx : g.cy, cl = axis ? g.cy : g.cx;
+            const float l0 = ((float)min(t, n_along - 1) - cl) * g.pix, l1 = ((float)min(t + kCols - 1, n_along - 1) - cl) * g.pix;
+            const float e0 = ((float)(min(a, n_across) - 1) - ca) * g.pix, e1 = ((float)min(a + kPix, n_across) - ca) * g.pix;
+            const float kk1 = axis ? g.k1 : -g.k1, gk0 = g.k0 - kBinEps, sod = g.sod, inv_du = g.inv_du;
+            const bool fan = g.kind != DECT_PARALLEL;
+            f32x2 acc[kCols][CH];
+#pragma unroll
+            for (int j = 0; j < kCols; ++j)
+#pragma unroll
+                for (int q = 0; q < CH; ++q) acc[j][q] = pack2(0.f, 0.f);
+            for (bool more = true; more;) {
+                const int st = batch % kStages;
+                stage_sync<kFull, Sh::kThreads>(st);
+                const int4* sg = segs + st * (kBatchSegs + 1);
+                const int head = sg[0].x, nseg = idle ? 0 : head & 0xffff;
+                const bool bad = (head >> 16) & 2;
+                more = !((head >> 16) & 1);
+                const Vec* bw = st_w + st * NV * CAP;
+                const int4* bp = st_pos + (st * BANDS + band) * CAP;
+                for (int s = 1; s <= nseg; ++s) {
+                    const int4 S = sg[s];
+                    const float cx = __int_as_float(S.x), cy = __int_as_float(S.y);
+                    // the lowest bin over the rectangle, from the two corners of its lower edge (bins rise or fall
+                    // along the across direction with the side of the source the rays come from): for a fan, with
+                    // (cx, cy) the view's (cos, sin) along and across, bin k1 (P . e) / (sod - P . n) + k0 with
+                    // P . e = +-(along cy - across cx), whose derivative across has the sign of +-(along - sod cx)
+                    float km;
+                    if (fan) {
+                        const float e = (l0 - sod * cx) * kk1 > 0.f ? e0 : e1;
+                        const float m = -e * cx, dn = fmaf(-e, cy, sod);
+                        const float ka = fmaf(l0, cy, m) * rcp_approx(fmaf(-l0, cx, dn));
+                        const float kb = fmaf(l1, cy, m) * rcp_approx(fmaf(-l1, cx, dn));
+                        km = fmaf(kk1, kk1 > 0.f ? fminf(ka, kb) : fmaxf(ka, kb), gk0);
+                    } else {
+                        const float m = fmaf(fminf(e0 * cy, e1 * cy), inv_du, gk0), cd = cx * inv_du;
+                        km = fminf(fmaf(l0, cd, m), fmaf(l1, cd, m));
+                    }
+                    // n rays from there on, within the segment (a ray outside the rectangle weighs zero at the
+                    // thread's pixels; the conversion saturates, so every index lies in the segment)
+                    const int n = S.z & 1023;
+                    const int i0 = min(max((int)((unsigned)__float2int_ru(km) + (unsigned)(S.z >> 10)), S.w & 0xffff), S.w >> 16);
+                    if (bad)
+                        gather_rays<CH, Sh::kVec, CAP, 1, true>(bp + i0, bw + i0, n, along0, kPix * blk, acc);
+                    else
+                        gather_rays<CH, Sh::kVec, CAP, Sh::kUnroll, false>(bp + i0, bw + i0, n, along0, kPix * blk, acc);
+                }
+                stage_arrive<kEmpty, Sh::kThreads>(st);
+                ++batch;
+            }
+            // the axis-0 sums into the tile, then the axis-1 sums on top of them
+            if (axis) bar_sync<kAxis, Sh::kGather>();
+            const int ct = 32 * band + along0;
+#pragma unroll
+            for (int q = 0; q < SG; ++q)
+#pragma unroll
+                for (int j = 0; j < kCols; ++j)
+#pragma unroll
+                    for (int p = 0; p < kPix; ++p) {
+                        const int al = ct + j, ac = kPix * blk + p;
+                        Acc* to = tile_acc + q * TILE * PITCH + (axis ? al * PITCH + ac : ac * PITCH + al);
+                        const float2 u = unpack2(acc[j][NCH * q]);
+                        if constexpr (NCH == 2) {
+                            const float2 v = unpack2(acc[j][NCH * q + 1]);
+                            float2 m = make_float2(p ? u.y : u.x, p ? v.y : v.x);
+                            if (axis) {
+                                const float2 o = *to;
+                                m.x = o.x + m.x;
+                                m.y = o.y + m.y;
+                            }
+                            *to = m;
+                        } else {
+                            const float m = p ? u.y : u.x;
+                            *to = axis ? *to + m : m;
+                        }
+                    }
+        }
     }
     __syncthreads();
     if constexpr (CLUSTER) {
@@ -328,13 +522,12 @@ __global__ void __launch_bounds__(SweepShape<TILE>::kThreads) k_bp_sweep(
             if (i < nx && j < ny) {
                 Acc sum{};
                 for (int k = 0; k < nrank; ++k) {
-                    Acc(*peer)[Sh::kRows][32] = cl.map_shared_rank(acc, k);
-                    const Acc a = peer[cc / 32][rr + 1][cc % 32], b = peer[Sh::kBands + rr / 32][cc + 1][rr % 32];
+                    const Acc a = cl.map_shared_rank(tile_acc, k)[rr * PITCH + cc];
                     if constexpr (NCH == 2) {
-                        sum.x += a.x + b.x;
-                        sum.y += a.y + b.y;
+                        sum.x += a.x;
+                        sum.y += a.y;
                     } else {
-                        sum += a + b;
+                        sum += a;
                     }
                 }
                 partial[d.img_off + (size_t)j * nx + i] = sum;
@@ -348,22 +541,7 @@ __global__ void __launch_bounds__(SweepShape<TILE>::kThreads) k_bp_sweep(
                 const int rr = px / TILE, cc = px % TILE;
                 const int i = ti + cc, j = tj + rr;
                 if (i < nx && j < ny) {
-                    Acc a, b;
-                    if constexpr (SG == 2) {
-                        const float4 a4 = acc4[cc / 32][rr + 1][cc % 32], b4 = acc4[Sh::kBands + rr / 32][cc + 1][rr % 32];
-                        a = q == 0 ? make_float2(a4.x, a4.y) : make_float2(a4.z, a4.w);
-                        b = q == 0 ? make_float2(b4.x, b4.y) : make_float2(b4.z, b4.w);
-                    } else {
-                        a = acc[cc / 32][rr + 1][cc % 32];
-                        b = acc[Sh::kBands + rr / 32][cc + 1][rr % 32];
-                    }
-                    Acc sum{};
-                    if constexpr (NCH == 2) {
-                        sum.x += a.x + b.x;
-                        sum.y += a.y + b.y;
-                    } else {
-                        sum += a + b;
-                    }
+                    const Acc sum = tile_acc[q * TILE * PITCH + rr * PITCH + cc];
                     partial[off + (size_t)j * nx + i] = sum;
                 }
             }
@@ -464,15 +642,12 @@ int sweep_tiles(int nx, int ny, int tile) { return ((nx + tile - 1) / tile) * ((
 int sweep_ctas_for_groups(int view_groups) { return view_groups; }
 int sweep_groups_per_cta() { return 1; }
 
-// the kernels' dynamic shared memory may exceed the default 48 KB (TILE 64); the attribute is per device
-static std::mutex g_slots_mu;
-static std::vector<int> g_slots[2];  // resident CTA slots of k_bp_sweep per device, TILE 32 and 64
-
+// the kernels' dynamic shared memory may exceed the default 48 KB; the attribute is per device
 template <class S2, int NCH, int TILE, bool CLUSTER, int SG>
 static cudaError_t sweep_attr1() {
-    auto* k = k_bp_sweep<S2, NCH, TILE, CLUSTER, SG>;
+    auto* k = k_bp_gather<S2, NCH, TILE, CLUSTER, SG>;
     cudaError_t e =
-        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sweep_acc_bytes<TILE, NCH, SG>());
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GatherShape<TILE, NCH, SG>::kBytes);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
     if (e == cudaSuccess && CLUSTER) e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     return e;
@@ -484,6 +659,8 @@ static cudaError_t sweep_attr() {
     if (e == cudaSuccess) e = sweep_attr1<S2, NCH, TILE, true, 1>();
     if constexpr (NCH == 2)
         if (e == cudaSuccess) e = sweep_attr1<S2, NCH, TILE, false, 2>();
+    if constexpr (NCH == 2 && TILE == 32)
+        if (e == cudaSuccess) e = sweep_attr1<S2, NCH, TILE, false, 4>();
     return e;
 }
 
@@ -496,28 +673,14 @@ cudaError_t sweep_init_attributes() {
     return e;
 }
 
-// CTA groups (view groups) per tile: the smallest C (up to 8) whose grid of tiles * C blocks fills the
-// resident slots best.
+// View groups per tile for a launch that is not autotuned: the smallest C (up to 8) whose tiles * C CTAs fill
+// whole multiples of 11 CTAs per SM (3 of the 64-pixel tiles) best: two to four times the resident ones, so that
+// the last ones to finish leave little of the chip idle.
 int sweep_groups(int tiles, int tile) {
-    int dev = 0;
+    int dev = 0, sms = 0;
     cudaGetDevice(&dev);
-    const int which = tile == 64 ? 1 : 0;
-    std::unique_lock<std::mutex> lk(g_slots_mu);
-    if ((int)g_slots[which].size() <= dev) g_slots[which].resize(dev + 1, 0);
-    if (!g_slots[which][dev]) {
-        int sms = 0, occ = 0;
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        sweep_init_attributes();
-        if (which)
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_bp_sweep<float2, 2, 64>, SweepShape<64>::kThreads,
-                                                          sweep_acc_bytes<64, 2>());
-        else
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_bp_sweep<float2, 2, 32>, SweepShape<32>::kThreads,
-                                                          sweep_acc_bytes<32, 2>());
-        g_slots[which][dev] = sms * (occ > 0 ? occ : 1);
-    }
-    const int slots = g_slots[which][dev];
-    lk.unlock();
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int slots = (sms > 0 ? sms : 1) * (tile == 64 ? 3 : 11);
     int best = 1;
     double best_fill = 0.0;
     for (int C = 1; C <= 8; ++C) {
@@ -537,14 +700,21 @@ static void sweep_t(const SliceDesc* dsl, const BlockMap& smap, int nsweep, int 
                     const int4* groups, const S2* sino, typename std::conditional<NCH == 2, float2, float>::type* partial,
                     int64_t stride, const float* rw, const float* scale, int* tile_count, cudaStream_t st) {
     if constexpr (NCH == 2) {
+        if constexpr (TILE == 32) {
+            if (sg == 4) {
+                k_bp_gather<S2, NCH, TILE, false, 4><<<nsweep, GatherShape<TILE, NCH, 4>::kThreads, GatherShape<TILE, NCH, 4>::kBytes, st>>>(
+                    dsl, smap, C, groups, sino, partial, stride, rw, scale, tile_count);
+                return;
+            }
+        }
         if (sg == 2) {
-            k_bp_sweep<S2, NCH, TILE, false, 2><<<nsweep, SweepShape<TILE>::kThreads, sweep_acc_bytes<TILE, NCH, 2>(), st>>>(
+            k_bp_gather<S2, NCH, TILE, false, 2><<<nsweep, GatherShape<TILE, NCH, 1>::kThreads, GatherShape<TILE, NCH, 2>::kBytes, st>>>(
                 dsl, smap, C, groups, sino, partial, stride, rw, scale, tile_count);
             return;
         }
     }
     if (!cluster || C == 1) {
-        k_bp_sweep<S2, NCH, TILE><<<nsweep, SweepShape<TILE>::kThreads, sweep_acc_bytes<TILE, NCH>(), st>>>(
+        k_bp_gather<S2, NCH, TILE><<<nsweep, GatherShape<TILE, NCH, 1>::kThreads, GatherShape<TILE, NCH, 1>::kBytes, st>>>(
             dsl, smap, C, nullptr, sino, partial, stride, rw, scale, tile_count);
         return;
     }
@@ -552,8 +722,8 @@ static void sweep_t(const SliceDesc* dsl, const BlockMap& smap, int nsweep, int 
     // so a cluster of C blocks is exactly one tile's view groups
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)nsweep);
-    cfg.blockDim = dim3(SweepShape<TILE>::kThreads);
-    cfg.dynamicSmemBytes = sweep_acc_bytes<TILE, NCH>();
+    cfg.blockDim = dim3(GatherShape<TILE, NCH, 1>::kThreads);
+    cfg.dynamicSmemBytes = GatherShape<TILE, NCH, 1>::kBytes;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -564,7 +734,7 @@ static void sweep_t(const SliceDesc* dsl, const BlockMap& smap, int nsweep, int 
     cfg.numAttrs = 1;
     const int4* no_groups = nullptr;
     int* no_count = nullptr;
-    cudaLaunchKernelEx(&cfg, k_bp_sweep<S2, NCH, TILE, true>, dsl, smap, C, no_groups, sino, partial, stride, rw,
+    cudaLaunchKernelEx(&cfg, k_bp_gather<S2, NCH, TILE, true>, dsl, smap, C, no_groups, sino, partial, stride, rw,
                        scale, no_count);
 }
 

@@ -155,19 +155,20 @@ void launch_project1(const SliceDesc* dsl, const BlockMap& map, int nblk, const 
                      const float2* ty, float* out, int views, cudaStream_t st);
 void launch_project(const SliceDesc* dsl, const BlockMap& map, int nblk, const int4* groups, const void* tx,
                     const void* ty, void* out, int prec, int views, cudaStream_t st);
-// backproject_sweep.cu: the solver's backprojector (two kernels: sweep into C partial images, then
+// backproject_sweep.cu: the solver's backprojector (two kernels: the gather into C partial images, then
 // the fixed-order sum of the partials with the epilogue; partial dots over the `pix` blocks)
 int sweep_ctas_for_groups(int view_groups);
 int sweep_groups_per_cta();
-// image tiles of the sweep for a TILE x TILE tile (32 or 64); the occupancy choice of view groups
+// image tiles for a TILE x TILE tile (32 or 64); the view groups of a launch that is not autotuned
 int sweep_tiles(int nx, int ny, int tile);
 int sweep_groups(int tiles, int tile);
-cudaError_t sweep_init_attributes();  // per device: dynamic shared memory of the 64-pixel tiles
+cudaError_t sweep_init_attributes();  // per device: the kernels' dynamic shared memory
 constexpr int kSweepTileDefault = 32;
 // cluster: the C view groups of a tile reduce on chip (thread-block cluster, distributed shared memory)
 // into partial image 0 (the finalize pass then reads one image, C = 1); otherwise C partial images.
-// sg = 2: the block map counts tiles of slice groups (groups: {slice, second slice or -1, -, -}) and a
-// CTA backprojects into both slices of its group (plain form only); sg = 1: the map counts slices.
+// sg = 2 or 4 (4: 32-pixel tiles): the block map counts tiles of slice groups (groups: up to sg slices of one
+// geometry, -1 past the group's size) and a CTA backprojects into every slice of its group (plain form only);
+// sg = 1: the map counts slices.
 // tile_count (plain form, C >= 2; nullptr otherwise): one zeroed counter per tile of the launch
 // (nsweep / C of them); the tile's last CTA sums the C partials into image 0 (the finalize pass then
 // reads one image, C = 1) and zeroes the counter again.
