@@ -280,9 +280,9 @@ typedef struct {
                                     0 plain CG; other values: DECT_EINVAL */
     int32_t use_graph;           /* 1: capture one iteration as a CUDA graph */
     int32_t bp_view_groups;      /* backprojector view groups per image tile, 1..16; -1 = chosen from the
-                                    occupancy (fill the GPU's resident slots); 0 = from the batch's size: 12 below
-                                    1024 tiles of 32 x 32 pixels, 6 from there on (fewer where the partial images
-                                    would not fit; reported in dect_stats). It fixes the order of a pixel's
+                                    occupancy (fill the GPU's resident slots); 0 = from the batch's tiles and views
+                                    (4 to 16; fewer where the partial images would not fit; reported in
+                                    dect_stats). It fixes the order of a pixel's
                                     partial sums: results are bitwise reproducible for a fixed value, and a
                                     slice solved alone or in a batch gives identical bits when the value is the
                                     same (it is the one launch-dependent choice of the batch). */

@@ -1147,6 +1147,28 @@ static dect_status enq_initialize(dect_admm* A, cudaStream_t st) {
 
 // ---- creation ------------------------------------------------------------------------------------
 
+// View groups per tile of a batch with `tiles` 32-pixel tiles over its slices (`paired` of them when slices of one
+// geometry are taken two at a time, 0 if none are) and `views` views per slice on average. Few tiles want many
+// groups to fill the chip, but a group of less than about 6 views pays more for its start than it computes;
+// medium batches of few views take as many groups as give 11 CTAs per SM (6 of paired slices); large ones fill it
+// with any count and take fewer partial images. Between 4 and 16 groups the backprojector's time differs by a few
+// percent (512^2 alone: 0.71 to 0.76 ms per iteration, 8 of them: 2.57 to 2.67).
+static int default_view_groups(int tiles, int paired, int views) {
+    if (tiles < 100) return views >= 150 ? 16 : (paired && tiles >= 75) ? 10 : views >= 75 ? 12 : 10;
+    if (paired && tiles < 160) return 10;
+    const int units = paired ? paired : tiles, slots = paired ? 6 * 152 : 11 * 152;
+    if (4 * units <= slots && views < 390) {
+        int C = 4;
+        for (int c : {6, 8, 10, 12, 16})
+            if (units * c <= slots) C = c;
+        return C;
+    }
+    if (tiles < 480) return 12;
+    if (tiles < 640) return views > 810 ? 16 : 12;
+    if (tiles < 800) return views > 800 ? 12 : 8;
+    return tiles < 1500 ? 8 : 6;
+}
+
 // Sweep block map for C CTA groups per TILE x TILE tile (prefix over slices, or over slice pairs for sg = 2)
 static void sweep_prefix(const dect_admm* A, int C, int tile, int sg, std::vector<int>& h) {
     h.assign(1, 0);
@@ -1496,16 +1518,20 @@ extern "C" dect_status dect_admm_create(dect_geom* const* geoms, int32_t B, cons
         } else if (P->bp_view_groups < 0) {
             A->sweep_C = sweep_groups(total, tile0);  // occupancy choice, not timed
         } else {
-            // by the batch's tiles: 12 below 1024 of them, so that a lone small or medium slice fills the chip
-            // (512^2: 0.71 ms per iteration at 10 to 16 groups, 0.76 at 7), 6 from there on (8 slices of 512^2: 2.62
-            // at 6, 2.67 at 4 and 8), as far as the partial images fit in 1/16 of the free memory and 4 GiB. Not
-            // timed: it fixes the order of a pixel's sums, so the same batch gives the same bits on every run.
+            // from the batch's shape, as far as the partial images fit in 1/16 of the free memory and 4 GiB.
+            // Not timed: it fixes the order of a pixel's sums, so the same batch gives the same bits on every run.
             size_t free_b = 0, total_b = 0;
             cudaMemGetInfo(&free_b, &total_b);
             const double budget = std::min(4.0 * (1 << 30), (double)free_b / 16.0);
             int tiles32 = 0;
-            for (int b = 0; b < B; ++b) tiles32 += sweep_tiles(geoms[b]->desc.nx, geoms[b]->desc.ny, 32);
-            A->sweep_C = tiles32 < 1024 ? 12 : 6;
+            int64_t views = 0;
+            for (int b = 0; b < B; ++b) {
+                tiles32 += sweep_tiles(geoms[b]->desc.nx, geoms[b]->desc.ny, 32);
+                views += geoms[b]->desc.n_views;
+            }
+            int paired = 0;  // tiles when the slices of one geometry are taken in pairs
+            for (const int4& pr : A->sgroups[0]) paired += sweep_tiles(geoms[pr.x]->desc.nx, geoms[pr.x]->desc.ny, 32);
+            A->sweep_C = default_view_groups(tiles32, sg_ok && paired < tiles32 ? paired : 0, (int)(views / B));
             while (A->sweep_C > 1 && (double)A->sweep_C * pix * sizeof(float2) > budget) --A->sweep_C;
             tune.push_back(A->sweep_C);  // the launch shapes that give the same bits are timed at this C
         }
