@@ -128,7 +128,8 @@ struct dect_spectra {
     double4_32a* w64 = nullptr;  // [2][ne]: {S_h, S_l, S_h f_KN, S_h f_p}, {S_l f_KN, S_l f_p, 0, 0}
     double abar_low = 1.0;  // sum_E S_l f_KN (unit-sum S_l)
     int n_both = 0, n_end = 0, tail_high = 1;  // supports of the spectra (see SpecDev)
-    SpecDev dev() const { return SpecDev{ne, t1, t2, w64, w64 + ne, n_both, n_end, tail_high}; }
+    float kc_max = 0.f, kp_max = 0.f;
+    SpecDev dev() const { return SpecDev{ne, t1, t2, w64, w64 + ne, n_both, n_end, tail_high, kc_max, kp_max}; }
 };
 
 extern "C" const char* dect_version(void) { return "dect 0.1 sm_103a"; }
@@ -307,6 +308,10 @@ extern "C" dect_status dect_spectra_create(int32_t ne, const double* S_h, const 
     dect_spectra* s = new dect_spectra();
     s->ne = ne;
     s->abar_low = abar;
+    for (const float4& t : t1) {
+        s->kc_max = std::max(s->kc_max, std::fabs(t.x));
+        s->kp_max = std::max(s->kp_max, std::fabs(t.y));
+    }
     int last_h = 0, last_l = 0;  // one past the last non-zero bin of each spectrum
     for (int e = 0; e < ne; ++e) {
         if (S_h[e] > 0.0) last_h = e + 1;

@@ -115,6 +115,7 @@ struct SpecDev {
     const double4_32a* w1;
     const double4_32a* w2;
     int n_both, n_end, tail_high;
+    float kc_max, kp_max;  // largest |k_kn| and |k_p| of t1
 };
 
 // Epilogue modes of the backprojector.

@@ -42,6 +42,27 @@ __device__ __forceinline__ void block_partials(float (&v)[N], double* __restrict
     }
 }
 
+// The same for a block whose threads hold R values each in place of a block R times as large: set k of thread t
+// stands for thread t + k blockDim.x, and the sums are formed in that block's order (the same bits).
+template <int R, int N>
+__device__ __forceinline__ void block_partials_rows(float (&v)[R][N], double* __restrict__ out) {
+    __shared__ double redf[N][32];
+    const int w = threadIdx.x / 32, nw = blockDim.x / 32;
+#pragma unroll
+    for (int k = 0; k < R; ++k) {
+        for (int q = 0; q < N; ++q)
+            for (int o = 16; o > 0; o >>= 1) v[k][q] += __shfl_down_sync(0xffffffffu, v[k][q], o);
+        if ((threadIdx.x & 31) == 0)
+            for (int q = 0; q < N; ++q) redf[q][w + k * nw] = (double)v[k][q];
+    }
+    __syncthreads();
+    if (threadIdx.x < N) {
+        double t = 0.0;
+        for (int k = 0; k < R * nw; ++k) t += redf[threadIdx.x][k];
+        out[N * (size_t)blockIdx.x + threadIdx.x] = t;
+    }
+}
+
 // Sum of partial slots [prefix[s], prefix[s+1]) of width N, by one block (fixed order).
 template <int N>
 __device__ void slice_sum(const double* __restrict__ part, const int* __restrict__ prefix, int s, double (&out)[N]) {
