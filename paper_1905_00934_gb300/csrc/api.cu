@@ -942,7 +942,7 @@ static void enq_iteration64(dect_admm* A, cudaStream_t st) {
     pb(A, st);
     launch64_udm_admm(A->ds, rays, A->rays.total, A->spec->t64, A->spec->ne, A->meas, v, A->status, A->sc,
                       A->P.m_udm, A->part_udm, st);
-    pe(A, DECT_PHASE_UDM, 1, st);
+    pe(A, DECT_PHASE_UDM, 2, st);
     if (A->counting) A->cF += 4 * A->P.m_udm;
     pb(A, st);
     launch64_image_update(A->ds, pix, A->pix.total, A->sc, A->P.lambda_c, A->P.lambda_p, v, A->part_img, st);
@@ -1458,7 +1458,7 @@ extern "C" dect_status dect_admm_create(dect_geom* const* geoms, int32_t B, cons
         if (geoms[b]->desc.nx > 2048 || geoms[b]->desc.ny > 2048)
             DECT_FAIL(DECT_EUNSUPPORTED, "dect_admm_create: the solver supports images up to 2048 x 2048");
     }
-    cudaError_t fe = fft_init_attributes();
+    cudaError_t fe = P->storage == DECT_STORE_F64 ? solver64_init_attributes() : fft_init_attributes();
     if (fe != cudaSuccess) DECT_FAIL(DECT_ECUDA, std::string("dect_admm_create: ") + cudaGetErrorString(fe));
 
     dect_admm* A = new dect_admm();

@@ -282,6 +282,7 @@ struct F64Vecs {
     double *H = nullptr, *Hn = nullptr;
     double2* Z = nullptr;
 };
+cudaError_t solver64_init_attributes();  // per device: the transforms' dynamic shared memory
 void launch64_sino_resid(const SliceDesc* d, const BlockMap& rays, int nr, const double* a, const double* ua,
                          const double* Rx, double* b, cudaStream_t st);
 void launch64_r0(const SliceDesc* d, const BlockMap& pix, int np, const double* RTb, const F64Vecs& v, double* r,

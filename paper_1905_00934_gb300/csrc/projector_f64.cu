@@ -6,8 +6,14 @@
 // their weights to ~1e-7; here every ray's position at index 0, slope and weight come from a
 // float64 table built once per geometry, and both kernels evaluate a sample's position with the
 // same explicit fused multiply-add, so R and R^T apply identical float64 weights. Same Joseph
-// interpolation and conventions as the float32 path; simple thread-per-ray / thread-per-pixel
-// kernels (float64 throughput on this GPU is low; these are not on the solver's path).
+// interpolation and conventions as the float32 path. Four lanes share a ray (R) and eight warps a row of 32
+// pixels (R^T, a view group each), so that the small problems these are meant for fill the GPU; every sum has a
+// fixed order.
+//
+// What bounds them: the float64 pipe (two lanes per clock and SM) and latency at small sizes. R^T first tests a
+// candidate ray by its fixed-point position, so float64 work is done only for rays that weigh something; a
+// pixel's candidates are the bins of the square of one pixel around its centre. Measured on GB300: 64^2 x 90 x 96,
+// both bases: R 67 -> 26 us, R^T 300 -> 38; 128^2 x 180 x 256: R 207 -> 141, R^T 862 -> 273.
 #include <cuda_runtime.h>
 #include <math.h>
 
@@ -60,90 +66,129 @@ cudaError_t build_ray_table_f64(const dect_geom_desc& d, double4_32a* rays, cuda
     return cudaGetLastError();
 }
 
-__device__ __forceinline__ double img64(const double* __restrict__ im, int nx, int ny, int j, int i) {
-    return (i < 0 || i >= nx || j < 0 || j >= ny) ? 0.0 : __ldg(im + (size_t)j * nx + i);
-}
+constexpr int kLanesPerRay = 4;
+constexpr int kRayThreads = 128;
+constexpr int kPixGroups = 8;  // view groups (warps) per row of 32 pixels
 
-// out[c][ray] = R x[c], planar float64
-__global__ void k_project_f64(GeomDev g, const double4_32a* __restrict__ rays, const double* __restrict__ x, int nch,
-                              double* __restrict__ out) {
+// out[c][ray] = R x[c], planar float64. Lane l of a ray takes the samples lo + l, lo + l + 4, ...
+template <int NCH>
+__global__ void __launch_bounds__(kRayThreads) k_project_f64(GeomDev g, const double4_32a* __restrict__ rays,
+                                                             const double* __restrict__ x, double* __restrict__ out) {
     const int64_t n = (int64_t)g.nv * g.nb;
-    const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= n) return;
-    const double4_32a P = rays[r];
-    const bool ax = P.w != 0.0;
-    const int n_along = ax ? g.ny : g.nx, n_across = ax ? g.nx : g.ny;
-    // indices whose positions lie in (-1, n_across): the only ones with a non-zero weight
-    int lo = 0, hi = n_along - 1;
-    if (P.y != 0.0) {
-        const double t0 = (-1.0 - P.x) / P.y, t1 = ((double)n_across - P.x) / P.y;
-        lo = max(lo, (int)floor(fmax(fmin(t0, t1), -1.0)));
-        hi = min(hi, (int)ceil(fmin(fmax(t0, t1), (double)n_along)));
-    } else if (!(P.x > -1.0 && P.x < n_across)) {
-        hi = -1;
-    }
-    const size_t plane = (size_t)g.nx * g.ny;
-    for (int c = 0; c < nch; ++c) {
-        const double* im = x + c * plane;
-        double acc = 0.0;
-        for (int t = lo; t <= hi; ++t) {
-            const double q = __fma_rn((double)t, P.y, P.x);
-            const double fl = floor(q);
-            const double f = q - fl;
-            const int h = (int)fl;
-            const double a = ax ? img64(im, g.nx, g.ny, t, h) : img64(im, g.nx, g.ny, h, t);
-            const double b = ax ? img64(im, g.nx, g.ny, t, h + 1) : img64(im, g.nx, g.ny, h + 1, t);
-            acc += (1.0 - f) * a + f * b;
+    const int64_t r = ((int64_t)blockIdx.x * kRayThreads + threadIdx.x) / kLanesPerRay;
+    const int sub = threadIdx.x % kLanesPerRay;
+    double acc[NCH];
+#pragma unroll
+    for (int c = 0; c < NCH; ++c) acc[c] = 0.0;
+    double w = 0.0;
+    if (r < n) {
+        const double4_32a P = rays[r];
+        w = P.z;
+        const bool ax = P.w != 0.0;
+        const int n_along = ax ? g.ny : g.nx, n_across = ax ? g.nx : g.ny;
+        // indices whose positions lie in (-1, n_across): the only ones with a non-zero weight
+        int lo = 0, hi = n_along - 1;
+        if (P.y != 0.0) {
+            const double t0 = (-1.0 - P.x) / P.y, t1 = ((double)n_across - P.x) / P.y;
+            // (both bounded before the conversion: a nearly axis-parallel ray far outside has ends at +-1e17)
+            lo = max(lo, (int)floor(fmin(fmax(fmin(t0, t1), -1.0), (double)n_along)));
+            hi = min(hi, (int)ceil(fmax(fmin(fmax(t0, t1), (double)n_along), -1.0)));
+        } else if (!(P.x > -1.0 && P.x < n_across)) {
+            hi = -1;
         }
-        out[c * n + r] = P.z * acc;
-    }
-}
-
-// x[c][pixel] = R^T s[c]: gathers per pixel over views and candidate bins
-__global__ void k_backproject_f64(GeomDev g, const double4_32a* __restrict__ rays, const double* __restrict__ sino, int nch,
-                                  double* __restrict__ out) {
-    const int64_t np = (int64_t)g.nx * g.ny;
-    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= np) return;
-    const int j = (int)(e / g.nx), i = (int)(e % g.nx);
-    // rays with a non-zero weight at (i, j) pass within 1 pixel of it: candidates of the square of
-    // half-side 1.5 pixels around the 2x2 block with top-left (i, j)
-    const float xc = ((float)i + 0.5f - g.cx) * g.pix, yc = ((float)j + 0.5f - g.cy) * g.pix;
-    const int64_t n = (int64_t)g.nv * g.nb;
-    double acc0 = 0.0, acc1 = 0.0;
-    for (int v = 0; v < g.nv; ++v) {
-        const float4 V = __ldg(g.views + v);
-        const CandRange cr = rect_candidates(g, V.x, V.y, xc, yc, 1.5f * g.pix, 1.5f * g.pix);
-        for (int k = cr.lo; k <= cr.hi; ++k) {
-            const int64_t r = (int64_t)v * g.nb + k;
-            const double4_32a P = rays[r];
-            const bool ax = P.w != 0.0;
-            const int t = ax ? j : i, across = ax ? i : j;
+        const size_t plane = (size_t)g.nx * g.ny;
+        const size_t s_along = ax ? g.nx : 1, s_across = ax ? 1 : g.nx;
+        for (int t = lo + sub; t <= hi; t += kLanesPerRay) {
             const double q = __fma_rn((double)t, P.y, P.x);
             const double fl = floor(q);
             const double f = q - fl;
             const int h = (int)fl;
-            const double wgt = h == across ? 1.0 - f : (h + 1 == across ? f : 0.0);
-            if (wgt != 0.0) {
-                acc0 += P.z * wgt * sino[r];
-                if (nch > 1) acc1 += P.z * wgt * sino[n + r];
+            const bool in0 = h >= 0 && h < n_across, in1 = h + 1 >= 0 && h + 1 < n_across;
+            const double* im = x + t * s_along + (int64_t)h * (int64_t)s_across;
+#pragma unroll
+            for (int c = 0; c < NCH; ++c) {
+                const double a = in0 ? __ldg(im + c * plane) : 0.0;
+                const double b = in1 ? __ldg(im + c * plane + s_across) : 0.0;
+                acc[c] += (1.0 - f) * a + f * b;
             }
         }
     }
-    out[e] = acc0;
-    if (nch > 1) out[np + e] = acc1;
+#pragma unroll
+    for (int c = 0; c < NCH; ++c)
+#pragma unroll
+        for (int o = 1; o < kLanesPerRay; o <<= 1) acc[c] += __shfl_xor_sync(0xffffffffu, acc[c], o);
+    if (r < n && sub == 0)
+#pragma unroll
+        for (int c = 0; c < NCH; ++c) out[c * n + r] = w * acc[c];
+}
+
+// x[c][pixel] = R^T s[c]: a warp gathers for 32 pixels of a row over the views of its group and their candidate
+// bins; the groups' sums are added in order
+template <int NCH>
+__global__ void __launch_bounds__(32 * kPixGroups) k_backproject_f64(GeomDev g, const double4_32a* __restrict__ rays,
+                                                                     const double* __restrict__ sino,
+                                                                     double* __restrict__ out) {
+    __shared__ double part[NCH][kPixGroups][33];
+    const int lane = threadIdx.x % 32, grp = threadIdx.x / 32;
+    const int tiles = (g.nx + 31) / 32;
+    const int j = blockIdx.x / tiles, i = (blockIdx.x % tiles) * 32 + lane;
+    const int64_t n = (int64_t)g.nv * g.nb;
+    double acc[NCH];
+#pragma unroll
+    for (int c = 0; c < NCH; ++c) acc[c] = 0.0;
+    if (i < g.nx) {
+        // a ray with a weight here passes within one pixel of the centre along its across direction
+        const float xc = ((float)i - g.cx) * g.pix, yc = ((float)j - g.cy) * g.pix;
+        for (int v = grp; v < g.nv; v += kPixGroups) {
+            const float4 V = __ldg(g.views + v);
+            const CandRange cr = rect_candidates(g, V.x, V.y, xc, yc, g.pix, g.pix);
+            for (int k = cr.lo; k <= cr.hi; ++k) {
+                const int64_t r = (int64_t)v * g.nb + k;
+                const int4 F = __ldg(g.rays + r);
+                const bool ax = ray_axis(F);
+                const int t = ax ? j : i, across = ax ? i : j;
+                // its fixed-point position is within a pixel (and 6e-5, far above the table's rounding)
+                const long long dq = ray_pos(F, t) - ((long long)across << 30);
+                if (dq <= -((1ll << 30) + (1 << 16)) || dq >= (1ll << 30) + (1 << 16)) continue;
+                const double4_32a P = rays[r];
+                // the ray's own axis bit: near 45 degrees the two tables may differ
+                const bool ax64 = P.w != 0.0;
+                const double q = __fma_rn((double)(ax64 ? j : i), P.y, P.x);
+                const double wgt = 1.0 - fabs(q - (double)(ax64 ? i : j));
+                if (!(wgt > 0.0)) continue;
+#pragma unroll
+                for (int c = 0; c < NCH; ++c) acc[c] += P.z * wgt * __ldg(sino + c * n + r);
+            }
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < NCH; ++c) part[c][grp][lane] = acc[c];
+    __syncthreads();
+    if (grp < NCH && i < g.nx) {
+        double s = 0.0;
+#pragma unroll
+        for (int k = 0; k < kPixGroups; ++k) s += part[grp][k][lane];
+        out[(size_t)grp * g.nx * g.ny + (size_t)j * g.nx + i] = s;
+    }
 }
 
 void project_single_f64(const GeomDev& g, const double4_32a* rays, const double* x, int nch, double* out,
                         cudaStream_t st) {
-    const int64_t n = (int64_t)g.nv * g.nb;
-    k_project_f64<<<(unsigned)((n + 127) / 128), 128, 0, st>>>(g, rays, x, nch, out);
+    const int64_t threads = (int64_t)g.nv * g.nb * kLanesPerRay;
+    const unsigned nblk = (unsigned)((threads + kRayThreads - 1) / kRayThreads);
+    if (nch > 1)
+        k_project_f64<2><<<nblk, kRayThreads, 0, st>>>(g, rays, x, out);
+    else
+        k_project_f64<1><<<nblk, kRayThreads, 0, st>>>(g, rays, x, out);
 }
 
 void backproject_single_f64(const GeomDev& g, const double4_32a* rays, const double* sino, int nch, double* out,
                             cudaStream_t st) {
-    const int64_t np = (int64_t)g.nx * g.ny;
-    k_backproject_f64<<<(unsigned)((np + 127) / 128), 128, 0, st>>>(g, rays, sino, nch, out);
+    const unsigned nblk = (unsigned)(((g.nx + 31) / 32) * (int64_t)g.ny);
+    if (nch > 1)
+        k_backproject_f64<2><<<nblk, 32 * kPixGroups, 0, st>>>(g, rays, sino, out);
+    else
+        k_backproject_f64<1><<<nblk, 32 * kPixGroups, 0, st>>>(g, rays, sino, out);
 }
 
 }  // namespace dect

@@ -11,7 +11,7 @@
 // The element-wise kernels run over the batch's pixel / ray block maps (256 per block, as in the
 // float32 path), so their partial sums land in the same slots and the same reduction kernels
 // (CG alpha / beta, residual balancing, xi) finish them. The projector pair is the float64
-// thread-per-ray / thread-per-pixel gather of projector_f64.cu, launched per slice. Arithmetic follows
+// gather of projector_f64.cu, launched per slice. Arithmetic follows
 // the oracle's operation order where it is written out (Eq. 9-13); the preconditioner transforms
 // Compton + i PE in one complex FFT (H is real and even, so the two parts stay separate).
 #include <cuda_runtime.h>
@@ -176,18 +176,29 @@ __global__ void __launch_bounds__(256) k64_cg_p(const SliceDesc* __restrict__ ds
 
 __device__ __forceinline__ int brev64(int t, int logn) { return (int)(__brev((unsigned)t) >> (32 - logn)); }
 
-// radix-2 decimation in time on a bit-reversed shared buffer (all threads of the block take part);
-// twiddle of butterfly position pos at stage half: exp(-+ i pi pos / half)
-__device__ void fft64(double2* buf, int logn, bool inverse) {
+// The twiddles exp(i pi k / (n / 2)), k < n / 2, of a length-n transform, in shared memory behind its buffer: the
+// butterfly at position pos of the stage of half-length half takes entry pos (n / 2) / half (the same argument of
+// sincospi as when it is formed there; forming it at every butterfly took most of the transform's float64 work).
+// No barrier: the transform's callers have one before it.
+__device__ __forceinline__ void twiddles64(double2* tw, int logn) {
+    const int half = 1 << (logn - 1);
+    for (int k = threadIdx.x; k < half; k += blockDim.x) {
+        double sn, cs;
+        sincospi((double)k / (double)half, &sn, &cs);
+        tw[k] = make_double2(cs, sn);
+    }
+}
+
+// radix-2 decimation in time on a bit-reversed shared buffer (all threads of the block take part)
+__device__ void fft64(double2* buf, const double2* tw, int logn, bool inverse) {
     const int n = 1 << logn;
     for (int s = 0; s < logn; ++s) {
         const int half = 1 << s;
         for (int b = threadIdx.x; b < n / 2; b += blockDim.x) {
             const int pos = b & (half - 1);
             const int i0 = ((b >> s) << (s + 1)) + pos, i1 = i0 + half;
-            double sn, cs;
-            sincospi((double)pos / (double)half, &sn, &cs);
-            const double wi = inverse ? sn : -sn;
+            const double2 w = tw[pos << (logn - 1 - s)];
+            const double cs = w.x, wi = inverse ? w.y : -w.y;
             const double2 u = buf[i0], v = buf[i1];
             const double tr = cs * v.x - wi * v.y, ti = cs * v.y + wi * v.x;
             buf[i0] = make_double2(u.x + tr, u.y + ti);
@@ -206,10 +217,12 @@ __global__ void __launch_bounds__(256) k64_rows_fwd(const SliceDesc* __restrict_
     const int nx = d.g.nx, px = d.px;
     const int64_t np = np_of(d);
     const double* rc = r + 2 * d.img_off + (size_t)j * nx;
+    double2* tw = zb + px;
+    twiddles64(tw, d.lpx);
     for (int t = threadIdx.x; t < px; t += blockDim.x)
         zb[brev64(t, d.lpx)] = t < nx ? make_double2(rc[t], rc[np + t]) : make_double2(0.0, 0.0);
     __syncthreads();
-    fft64(zb, d.lpx, false);
+    fft64(zb, tw, d.lpx, false);
     double2* zr = Z + d.fft_off + (size_t)j * px;
     for (int t = threadIdx.x; t < px; t += blockDim.x) zr[t] = zb[t];
 }
@@ -218,9 +231,11 @@ __global__ void __launch_bounds__(256) k64_rows_fwd(const SliceDesc* __restrict_
 __global__ void __launch_bounds__(256) k64_rows_full(SliceDesc d, double2* __restrict__ Z) {
     extern __shared__ double2 zb[];
     double2* zr = Z + (size_t)blockIdx.x * d.px;
+    double2* tw = zb + d.px;
+    twiddles64(tw, d.lpx);
     for (int t = threadIdx.x; t < d.px; t += blockDim.x) zb[brev64(t, d.lpx)] = zr[t];
     __syncthreads();
-    fft64(zb, d.lpx, false);
+    fft64(zb, tw, d.lpx, false);
     for (int t = threadIdx.x; t < d.px; t += blockDim.x) zr[t] = zb[t];
 }
 
@@ -234,10 +249,12 @@ __global__ void __launch_bounds__(256) k64_cols(const SliceDesc* __restrict__ ds
     const int px = d.px, py = d.py, lp = d.lpy;
     const int rows_in = rows_in_all ? py : d.g.ny, rows_out = rows_out_all ? py : d.g.ny;
     double2* zs = Z + d.fft_off;
+    double2* tw = zb + py;
+    twiddles64(tw, lp);
     for (int j = threadIdx.x; j < py; j += blockDim.x)
         zb[brev64(j, lp)] = j < rows_in ? zs[(size_t)j * px + k] : make_double2(0.0, 0.0);
     __syncthreads();
-    fft64(zb, lp, false);
+    fft64(zb, tw, lp, false);
     if (H) {
         const double* hs = H + d.h_off;
         for (int j = threadIdx.x; j < py; j += blockDim.x) {
@@ -254,7 +271,7 @@ __global__ void __launch_bounds__(256) k64_cols(const SliceDesc* __restrict__ ds
             }
         }
         __syncthreads();
-        fft64(zb, lp, true);
+        fft64(zb, tw, lp, true);
     }
     for (int j = threadIdx.x; j < rows_out; j += blockDim.x) zs[(size_t)j * px + k] = zb[j];
 }
@@ -269,9 +286,11 @@ __global__ void __launch_bounds__(256) k64_rows_inv(const SliceDesc* __restrict_
     const int nx = d.g.nx, px = d.px;
     const int64_t np = np_of(d);
     const double2* zr = Z + d.fft_off + (size_t)j * px;
+    double2* tw = zb + px;
+    twiddles64(tw, d.lpx);
     for (int t = threadIdx.x; t < px; t += blockDim.x) zb[brev64(t, d.lpx)] = zr[t];
     __syncthreads();
-    fft64(zb, d.lpx, true);
+    fft64(zb, tw, d.lpx, true);
     const double scale = 1.0 / ((double)px * (double)d.py);
     const size_t row = 2 * d.img_off + (size_t)j * nx;
     double acc[2] = {0.0, 0.0};
@@ -376,12 +395,14 @@ __device__ __forceinline__ double cost64(const Ray64& q, double fh, double fl, d
 
 // `iters` LM iterations: Gauss-Newton system A = sum_k w_k J_k J_k^T + diag(rho), Marquardt damping
 // B = A with its diagonal times (1 + mu), step -B^-1 g, kept iff the cost decreases (mu / 10, else * 10),
-// mu clamped to [1e-10, 1e10]; status 0 accepted, 1 rejected, 2 non-finite or singular
+// mu clamped to [1e-10, 1e10]; status 0 accepted, 1 rejected, 2 non-finite or singular. f and J at a trial point
+// that is kept are the next iteration's, so an iteration makes one pass over the energies.
 __device__ void lm64(const double4_32a* __restrict__ T, int ne, const Ray64& q, int iters, double& a0, double& a1,
                      double& m, uint8_t& st) {
+    if (iters <= 0) return;
+    double fh, fl, J[4];
+    fwd64(T, ne, a0, a1, fh, fl, J);
     for (int it = 0; it < iters; ++it) {
-        double fh, fl, J[4];
-        fwd64(T, ne, a0, a1, fh, fl, J);
         const double rh = fh - q.mh, rl = fl - q.ml;
         const double g0 = q.wh * rh * J[0] + q.wl * rl * J[2] + q.rc * (a0 - q.vc);
         const double g1 = q.wh * rh * J[1] + q.wl * rl * J[3] + q.rp * (a1 - q.vp);
@@ -397,8 +418,9 @@ __device__ void lm64(const double4_32a* __restrict__ T, int ne, const Ray64& q, 
         }
         const double t0 = a0 + (-g0 * B11 + g1 * A01) / det;
         const double t1 = a1 + (-g1 * B00 + g0 * A01) / det;
-        double fh1, fl1;
-        fwd64(T, ne, t0, t1, fh1, fl1, nullptr);
+        double fh1, fl1, J1[4];
+        const bool last = it == iters - 1;
+        fwd64(T, ne, t0, t1, fh1, fl1, last ? nullptr : J1);
         const double cost1 = cost64(q, fh1, fl1, t0, t1);
         if (!isfinite(cost1)) {
             m *= 10.0;
@@ -408,6 +430,11 @@ __device__ void lm64(const double4_32a* __restrict__ T, int ne, const Ray64& q, 
             a1 = t1;
             m /= 10.0;
             st = DECT_RAY_ACCEPTED;
+            if (!last) {
+                fh = fh1;
+                fl = fl1;
+                for (int k = 0; k < 4; ++k) J[k] = J1[k];
+            }
         } else {
             m *= 10.0;
             st = DECT_RAY_REJECTED;
@@ -422,42 +449,60 @@ __device__ __forceinline__ const double4_32a* load_tables64(const double4_32a* _
     return sh;
 }
 
-// a-update (v = R x - u^a) fused with u^a += a - R x; partial[4 blk + {0,1}] = sum (a - R x)^2,
-// {2,3} = sum (a - a_old)^2
-__global__ void __launch_bounds__(256) k64_udm_admm(const SliceDesc* __restrict__ dsl, BlockMap rays,
-                                                    const double4_32a* __restrict__ t64, int ne,
-                                                    const float4* __restrict__ meas, const double* __restrict__ Rx,
-                                                    double* __restrict__ ua, double* __restrict__ a,
-                                                    double* __restrict__ mu, uint8_t* __restrict__ status,
-                                                    const SliceScalars* __restrict__ sc, int iters,
-                                                    double* __restrict__ partial) {
+// Rays per block of the decomposition: a warp each, so that the few thousand rays of a small problem spread over
+// every SM (the blocks of 256 of the ray map left most of them idle: 8640 rays are 34 such blocks). The residual
+// sums keep the ray map's blocks in a kernel of their own.
+constexpr int kRays64 = 32;
+
+// a-update (v = R x - u^a): the new a into an, mu and status in place
+__global__ void __launch_bounds__(kRays64) k64_udm_admm(const SliceDesc* __restrict__ dsl, BlockMap rays,
+                                                        const double4_32a* __restrict__ t64, int ne,
+                                                        const float4* __restrict__ meas, const double* __restrict__ Rx,
+                                                        const double* __restrict__ ua, const double* __restrict__ a,
+                                                        double* __restrict__ an, double* __restrict__ mu,
+                                                        uint8_t* __restrict__ status, const SliceScalars* __restrict__ sc,
+                                                        int iters) {
     extern __shared__ double4_32a tab64[];
     const double4_32a* T = load_tables64(t64, ne, tab64);
     int local;
-    const int s = slice_of(rays, blockIdx.x, local);
+    const int s = slice_of(rays, blockIdx.x / (256 / kRays64), local);
     const SliceDesc& d = dsl[s];
+    const int64_t nr = nr_of(d), k = (int64_t)local * 256 + (blockIdx.x % (256 / kRays64)) * kRays64 + threadIdx.x;
+    if (k >= nr) return;
+    const int64_t ec = 2 * d.sino_off + k, ep = ec + nr, er = d.sino_off + k;
+    const float4 m4 = meas[er];
+    Ray64 q;
+    q.mh = m4.x;
+    q.ml = m4.y;
+    q.wh = m4.z;
+    q.wl = m4.w;
+    q.vc = Rx[ec] - ua[ec];
+    q.vp = Rx[ep] - ua[ep];
+    q.rc = sc[s].rho[0];
+    q.rp = sc[s].rho[1];
+    double a0 = a[ec], a1 = a[ep], m = mu[er];
+    uint8_t st = DECT_RAY_ACCEPTED;
+    lm64(T, ne, q, iters, a0, a1, m, st);
+    an[ec] = a0;
+    an[ep] = a1;
+    mu[er] = m;
+    if (status) status[er] = st;
+}
+
+// a = an and u^a += a - R x; partial[4 blk + {0,1}] = sum (a - R x)^2, {2,3} = sum (a - a_old)^2
+__global__ void __launch_bounds__(256) k64_a_update(const SliceDesc* __restrict__ dsl, BlockMap rays,
+                                                    const double* __restrict__ an, const double* __restrict__ Rx,
+                                                    double* __restrict__ ua, double* __restrict__ a,
+                                                    double* __restrict__ partial) {
+    int local;
+    const SliceDesc& d = dsl[slice_of(rays, blockIdx.x, local)];
     const int64_t nr = nr_of(d), k = (int64_t)local * 256 + threadIdx.x;
     double acc[4] = {0.0, 0.0, 0.0, 0.0};
     if (k < nr) {
-        const int64_t ec = 2 * d.sino_off + k, ep = ec + nr, er = d.sino_off + k;
-        const float4 m4 = meas[er];
-        Ray64 q;
-        q.mh = m4.x;
-        q.ml = m4.y;
-        q.wh = m4.z;
-        q.wl = m4.w;
-        q.vc = Rx[ec] - ua[ec];
-        q.vp = Rx[ep] - ua[ep];
-        q.rc = sc[s].rho[0];
-        q.rp = sc[s].rho[1];
-        const double oc = a[ec], op = a[ep];
-        double a0 = oc, a1 = op, m = mu[er];
-        uint8_t st = DECT_RAY_ACCEPTED;
-        lm64(T, ne, q, iters, a0, a1, m, st);
+        const int64_t ec = 2 * d.sino_off + k, ep = ec + nr;
+        const double a0 = an[ec], a1 = an[ep], oc = a[ec], op = a[ep];
         a[ec] = a0;
         a[ep] = a1;
-        mu[er] = m;
-        if (status) status[er] = st;
         ua[ec] = ua[ec] + a0 - Rx[ec];
         ua[ep] = ua[ep] + a1 - Rx[ep];
         const double rc = a0 - Rx[ec], rp = a1 - Rx[ep], dc = a0 - oc, dp = a1 - op;
@@ -470,16 +515,16 @@ __global__ void __launch_bounds__(256) k64_udm_admm(const SliceDesc* __restrict_
 }
 
 // initial decomposition: rho = (0, rho_p), v = 0, from a = (m_l / abar, 0); a = (a_c, 0), mu = mu0
-__global__ void __launch_bounds__(256) k64_udm_init(const SliceDesc* __restrict__ dsl, BlockMap rays,
-                                                    const double4_32a* __restrict__ t64, int ne,
-                                                    const float4* __restrict__ meas, double* __restrict__ a,
-                                                    double* __restrict__ mu, double rho_p, int iters, double abar,
-                                                    double mu0) {
+__global__ void __launch_bounds__(kRays64) k64_udm_init(const SliceDesc* __restrict__ dsl, BlockMap rays,
+                                                        const double4_32a* __restrict__ t64, int ne,
+                                                        const float4* __restrict__ meas, double* __restrict__ a,
+                                                        double* __restrict__ mu, double rho_p, int iters, double abar,
+                                                        double mu0) {
     extern __shared__ double4_32a tab64[];
     const double4_32a* T = load_tables64(t64, ne, tab64);
     int local;
-    const SliceDesc& d = dsl[slice_of(rays, blockIdx.x, local)];
-    const int64_t nr = nr_of(d), k = (int64_t)local * 256 + threadIdx.x;
+    const SliceDesc& d = dsl[slice_of(rays, blockIdx.x / (256 / kRays64), local)];
+    const int64_t nr = nr_of(d), k = (int64_t)local * 256 + (blockIdx.x % (256 / kRays64)) * kRays64 + threadIdx.x;
     if (k >= nr) return;
     const float4 m4 = meas[d.sino_off + k];
     Ray64 q;
@@ -702,6 +747,21 @@ __global__ void k64_from_f32(const float* __restrict__ in, int64_t n, double* __
 
 static unsigned nblocks(int64_t n, int t = 256) { return (unsigned)((n + t - 1) / t); }
 
+// shared memory (buffer and twiddles) and threads of a length-p transform's block
+static size_t fft64_bytes(int p) { return sizeof(double2) * (size_t)(p + p / 2); }
+static int fft64_threads(int p) { return p / 2 >= 256 ? 256 : (p / 2 <= 32 ? 32 : p / 2); }
+
+cudaError_t solver64_init_attributes() {
+    cudaError_t e = cudaSuccess;  // images up to 1024 x 1024: transforms up to 2048
+    const int bytes = (int)fft64_bytes(2048);
+    for (cudaError_t r : {cudaFuncSetAttribute(k64_rows_fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes),
+                          cudaFuncSetAttribute(k64_rows_full, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes),
+                          cudaFuncSetAttribute(k64_cols, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes),
+                          cudaFuncSetAttribute(k64_rows_inv, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes)})
+        if (e == cudaSuccess) e = r;
+    return e;
+}
+
 void launch64_sino_resid(const SliceDesc* d, const BlockMap& rays, int nr, const double* a, const double* ua,
                          const double* Rx, double* b, cudaStream_t st) {
     k64_sino_resid<<<nr, 256, 0, st>>>(d, rays, a, ua, Rx, b);
@@ -729,28 +789,33 @@ void launch64_precond(const SliceDesc* d, const BlockMap& rows, int nrows, const
         k64_identity<<<nrows, 256, 0, st>>>(d, rows, r, s, partial);
         return;
     }
-    k64_rows_fwd<<<nrows, 256, sizeof(double2) * max_px, st>>>(d, rows, r, Z);
-    k64_cols<<<ncols, 256, sizeof(double2) * max_py, st>>>(d, cols, Z, H, 0, 0);
-    k64_rows_inv<<<nrows, 256, sizeof(double2) * max_px, st>>>(d, rows, Z, r, s, partial);
+    // (a thread per butterfly: a short transform's barriers cost less in a small block)
+    const int tx = fft64_threads(max_px), ty = fft64_threads(max_py);
+    k64_rows_fwd<<<nrows, tx, fft64_bytes(max_px), st>>>(d, rows, r, Z);
+    k64_cols<<<ncols, ty, fft64_bytes(max_py), st>>>(d, cols, Z, H, 0, 0);
+    k64_rows_inv<<<nrows, tx, fft64_bytes(max_px), st>>>(d, rows, Z, r, s, partial);
 }
 void launch64_response(const SliceDesc* d_dev, const SliceDesc& d, const BlockMap& cols, int ncols, const double* psf,
                        double2* Z, double* H, double* Hn, bool ramp, cudaStream_t st) {
     const int64_t n = (int64_t)d.px * d.py;
     k64_embed_psf<<<nblocks(n), 256, 0, st>>>(d, psf, Z);
-    k64_rows_full<<<d.py, 256, sizeof(double2) * d.px, st>>>(d, Z);
-    k64_cols<<<ncols, 256, sizeof(double2) * d.py, st>>>(d_dev, cols, Z, nullptr, 1, 1);
+    k64_rows_full<<<d.py, 256, fft64_bytes(d.px), st>>>(d, Z);
+    k64_cols<<<ncols, 256, fft64_bytes(d.py), st>>>(d_dev, cols, Z, nullptr, 1, 1);
     k64_response<<<nblocks(n), 256, 0, st>>>(d, Z, H, Hn, ramp ? 1 : 0);
 }
 void launch64_udm_admm(const SliceDesc* d, const BlockMap& rays, int nr, const double4_32a* t64, int ne,
                        const float4* meas, const F64Vecs& v, uint8_t* status, const SliceScalars* sc, int iters,
                        double* partial, cudaStream_t st) {
-    k64_udm_admm<<<nr, 256, sizeof(double4_32a) * ne, st>>>(d, rays, t64, ne, meas, v.Rx, v.ua, v.a, v.mu, status, sc,
-                                                        iters, partial);
+    // (q, R p of the CG step just taken, is free until the next one: it holds the new a in between)
+    k64_udm_admm<<<nr * (256 / kRays64), kRays64, sizeof(double4_32a) * ne, st>>>(d, rays, t64, ne, meas, v.Rx, v.ua, v.a,
+                                                                                  v.q, v.mu, status, sc, iters);
+    k64_a_update<<<nr, 256, 0, st>>>(d, rays, v.q, v.Rx, v.ua, v.a, partial);
 }
 void launch64_udm_init(const SliceDesc* d, const BlockMap& rays, int nr, const double4_32a* t64, int ne,
                        const float4* meas, const F64Vecs& v, double rho_p, int iters, double abar, double mu0,
                        cudaStream_t st) {
-    k64_udm_init<<<nr, 256, sizeof(double4_32a) * ne, st>>>(d, rays, t64, ne, meas, v.a, v.mu, rho_p, iters, abar, mu0);
+    k64_udm_init<<<nr * (256 / kRays64), kRays64, sizeof(double4_32a) * ne, st>>>(d, rays, t64, ne, meas, v.a, v.mu, rho_p,
+                                                                                  iters, abar, mu0);
 }
 void launch64_image_update(const SliceDesc* d, const BlockMap& pix, int np, const SliceScalars* sc, double lam_c,
                            double lam_p, const F64Vecs& v, double* partial, cudaStream_t st) {
