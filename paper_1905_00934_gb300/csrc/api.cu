@@ -549,6 +549,7 @@ struct dect_admm {
     const int* rs_prefix() const { return P.precondition ? prows.d : rows.d; }
     int n_groups = 0;                // projector groups: consecutive slices of one geometry (proj_group_size())
     std::vector<int2> group_shape;   // {views, bins} per projector group
+    int group_max() const { return n_groups < B ? proj_group_size() : 1; }  // the most slices a group may have
     int proj_views = 2;              // views per projector CTA (2, 4 or 8; does not change results)
     int4* d_groups = nullptr;        // {slice, further slices or -1} per group
     int sweep_C = 1;                 // CTA groups (partial images) per backprojector tile
@@ -679,7 +680,7 @@ static void enq_project(dect_admm* A, const float2* img, void* out, cudaStream_t
     launch_textures(A->ds, A->tx.map(B), A->tx.total, A->ty.map(B), A->ty.total, img, A->txb, A->tyb, A->prec, st);
     pe(A, DECT_PHASE_TEXTURE, 2, st);
     pb(A, st);
-    launch_project(A->ds, A->ptile.map(A->n_groups), A->ptile.total, A->d_groups, A->txb, A->tyb, out, A->prec,
+    launch_project(A->ds, A->ptile.map(A->n_groups), A->ptile.total, A->d_groups, A->group_max(), A->txb, A->tyb, out, A->prec,
                    A->proj_views, st);
     pe(A, DECT_PHASE_PROJECT, 1, st);
     if (A->counting) A->cR += 2;
@@ -791,7 +792,7 @@ static void enq_lm_step(dect_admm* A, int b, cudaStream_t st) {
         launch_textures1(A->ds, A->tx.map(B), A->tx.total, A->ty.map(B), A->ty.total, A->lm_p, A->tx1, A->ty1, st);
         pe(A, DECT_PHASE_TEXTURE, 2, st);
         pb(A, st);
-        launch_project1(A->ds, A->ptile.map(A->n_groups), A->ptile.total, A->d_groups, A->tx1, A->ty1, A->lm_q,
+        launch_project1(A->ds, A->ptile.map(A->n_groups), A->ptile.total, A->d_groups, A->group_max(), A->tx1, A->ty1, A->lm_q,
                         A->proj_views, st);
         pe(A, DECT_PHASE_PROJECT, 1, st);
         pb(A, st);
@@ -1207,7 +1208,7 @@ static cudaError_t autotune_projector(dect_admm* A) {
         ptile_prefix(A, views, h);
         e = cudaMemcpy(A->ptile.d, h.data(), sizeof(int) * h.size(), cudaMemcpyHostToDevice);
         const BlockMap m{A->ptile.d, A->n_groups};
-        auto run = [&]() { launch_project(A->ds, m, h.back(), A->d_groups, A->txb, A->tyb, A->q, A->prec, views, st); };
+        auto run = [&]() { launch_project(A->ds, m, h.back(), A->d_groups, A->group_max(), A->txb, A->tyb, A->q, A->prec, views, st); };
         run();  // warm-up
         e = cudaGetLastError();
         if (e == cudaSuccess) e = cudaEventRecord(e0, st);

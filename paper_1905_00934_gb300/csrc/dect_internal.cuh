@@ -152,9 +152,10 @@ void launch_textures1(const SliceDesc* dsl, const BlockMap& mx, int nbx, const B
 int proj_tiles(int nv, int nb, int views);
 int proj_default_views();
 int proj_group_size();
-void launch_project1(const SliceDesc* dsl, const BlockMap& map, int nblk, const int4* groups, const float2* tx,
-                     const float2* ty, float* out, int views, cudaStream_t st);
-void launch_project(const SliceDesc* dsl, const BlockMap& map, int nblk, const int4* groups, const void* tx,
+// (group: the most slices any group of the launch has)
+void launch_project1(const SliceDesc* dsl, const BlockMap& map, int nblk, const int4* groups, int group,
+                     const float2* tx, const float2* ty, float* out, int views, cudaStream_t st);
+void launch_project(const SliceDesc* dsl, const BlockMap& map, int nblk, const int4* groups, int group, const void* tx,
                     const void* ty, void* out, int prec, int views, cudaStream_t st);
 // backproject_sweep.cu: the solver's backprojector (two kernels: the gather into C partial images, then
 // the fixed-order sum of the partials with the epilogue; partial dots over the `pix` blocks)

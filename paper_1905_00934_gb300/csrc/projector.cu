@@ -199,9 +199,7 @@ __global__ void k_pack_planar(const float* __restrict__ in, int nch, int64_t n, 
 
 // Launch shape of the forward projector (compile-time; the defaults are the measured best on GB300):
 // samples whose texel loads are issued together per lane, views (warps) per CTA, the CTAs per SM the
-// register allocation must allow, slices of one geometry per CTA (1, 2 or 4), and whether the
-// single-slice sum's positions advance incrementally or are recomputed from the index at every sample
-// (both give the same integers, so the same results; the grouped sum always steps incrementally).
+// register allocation must allow, slices of one geometry per CTA (1, 2 or 4) where a geometry has several.
 #ifndef DECT_PROJ_BATCH
 #define DECT_PROJ_BATCH 8
 #endif
@@ -213,9 +211,6 @@ __global__ void k_pack_planar(const float* __restrict__ in, int nch, int64_t n, 
 #endif
 #ifndef DECT_PROJ_GROUP
 #define DECT_PROJ_GROUP 2
-#endif
-#ifndef DECT_PROJ_INCR
-#define DECT_PROJ_INCR 0
 #endif
 constexpr int kProjBatch = DECT_PROJ_BATCH;
 
@@ -253,79 +248,6 @@ __device__ __forceinline__ f32x2 lerp2(float f, const float4 v) {
     return fma2(pack2(f, f), sub2(pack2(v.z, v.w), lo), lo);
 }
 
-// Sum over a ray's samples of the interpolated {c, p} (unweighted), with the warp stepping in lock
-// step: every lane visits the same sampled index t, from the warp's lowest first index to its highest
-// last one, so at each step the lanes (neighbouring rays) read neighbouring texels of one texture row
-// and their loads coalesce. A lane outside its own [lo, hi] reads texel 0 of its texture, which is
-// always zero padding (the pair of rows or columns -2, -1 of column or row 0), and adds an exact zero,
-// so each ray's sum takes the same terms in the same order as a walk over its own range alone.
-// Every lane of the warp must call this (valid = false for lanes without a ray).
-template <class TX>
-__device__ __forceinline__ float2 ray_sum_sync(const int4 P, bool valid, const GeomDev& g, const TX* __restrict__ tx,
-                                               const TX* __restrict__ ty) {
-    const bool ax = ray_axis(P);
-    const int n_across = ax ? g.nx : g.ny;
-    const TX* __restrict__ tex = ax ? ty : tx;
-    const int ld = n_across + 3;
-    int lo = 1, hi = 0;
-    if (valid) trimmed_range(P, g, lo, hi);
-    const bool any = lo <= hi;
-    const int t0 = __reduce_min_sync(0xffffffffu, any ? lo : 0x7fffffff);
-    const int t1 = __reduce_max_sync(0xffffffffu, any ? hi : -1);
-    // {c, p} sums as one packed pair: each element's terms and order are those of two scalar sums
-    f32x2 acc = pack2(0.f, 0.f);
-    if (t0 > t1) return unpack2(acc);  // no lane of the warp samples the image (warp-uniform)
-    // from here 0 <= t0 <= t1 < max(nx, ny): the bounds below cannot overflow
-    const long long step = ray_step(P), q0 = ray_q0(P);
-    int t = t0;
-#if DECT_PROJ_INCR
-    // positions and texel rows advance by exact integer steps; a lane samples while (t - lo), modulo 2^32
-    // (it wraps through 0 exactly when t reaches lo), is <= hi - lo. A lane without samples starts at
-    // 2^31 with len 0: its rel stays in [2^31, 2^31 + 4104) over at most 4096 + 8 steps, never <= 0.
-    long long q = q0 + (long long)t0 * step;
-    int base = t0 * ld + 2;  // texel (t, floor + 2) is tex[base + floor(q)]
-    unsigned rel = any ? (unsigned)(t0 - lo) : 0x80000000u;
-    const unsigned len = any ? (unsigned)(hi - lo) : 0u;
-    for (; t <= t1 - (kProjBatch - 1); t += kProjBatch) {
-        float4 v[kProjBatch];
-        float f[kProjBatch];
-#pragma unroll
-        for (int u = 0; u < kProjBatch; ++u) {
-            v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (rel + (unsigned)u <= len) v[u] = ldtex(tex + (base + pos_floor(q)));
-            f[u] = frac_of(q);
-            q += step;
-            base += ld;
-        }
-        rel += kProjBatch;
-#pragma unroll
-        for (int u = 0; u < kProjBatch; ++u) acc = add2(acc, lerp2(f[u], v[u]));
-    }
-#else
-    for (; t <= t1 - (kProjBatch - 1); t += kProjBatch) {
-        float4 v[kProjBatch];
-        float f[kProjBatch];
-#pragma unroll
-        for (int u = 0; u < kProjBatch; ++u) {
-            const int tt = t + u;
-            const long long qu = q0 + (long long)tt * step;
-            // a lane outside its range reads texel 0, which is zero padding (rows or columns -2 and -1)
-            const int idx = (tt >= lo && tt <= hi) ? tt * ld + 2 + pos_floor(qu) : 0;
-            v[u] = ldtex(tex + idx);
-            f[u] = frac_of(qu);
-        }
-#pragma unroll
-        for (int u = 0; u < kProjBatch; ++u) acc = add2(acc, lerp2(f[u], v[u]));
-    }
-#endif
-    for (; t <= t1; ++t) {
-        const long long q1 = q0 + (long long)t * step;
-        const float4 v = ldtex(tex + ((t >= lo && t <= hi) ? t * ld + 2 + pos_floor(q1) : 0));
-        acc = add2(acc, lerp2(frac_of(q1), v));
-    }
-    return unpack2(acc);
-}
-
 // A CTA takes a tile of V consecutive views x 32 consecutive bins, one warp per view: the rays of
 // neighbouring views through the same bins cross nearly the same texels, so the tile's warps share them
 // in L1. V = 2, 4 or 8 is timed by the solver at creation (a ray's sum does not depend on its tile, so
@@ -347,45 +269,72 @@ __device__ __forceinline__ bool proj_ray(int local, int nv, int nb, int& v, int&
     return v < nv && k < nb;
 }
 
-// The same lock-step sum for the rays of one geometry through up to G slices' images at once (slices
-// of one scan share the geometry): positions, ranges and texel indices are formed once per sample and
-// only the texel loads and the accumulation are per slice. Each slice's sum takes the same terms in the
-// same order as ray_sum_sync on that slice alone. count (<= G) is uniform over the CTA.
+// Sum over a ray's samples of the interpolated {c, p} (unweighted) of up to G slices' images at once, with the
+// warp stepping in lock step: every lane visits the same sampled index t, from the warp's lowest first index to
+// its highest last one, so at each step the lanes (neighbouring rays) read neighbouring texels of one texture row
+// and their loads coalesce. A lane outside its own [lo, hi] reads texel 0 of its texture, which is
+// always zero padding (the pair of rows or columns -2, -1 of column or row 0), and adds an exact zero,
+// so each ray's sum takes the same terms in the same order as a walk over its own range alone, whatever G.
+// Over the indices that every lane with samples has (nearly all of them inside the image) the range test is left
+// out: it was 4 of the 18 instructions of a sample. Measured on GB300, 512 x 512 x 720 x 1024, both bases: one slice
+// 209 -> 165 us (issue was the bound; with G = 1 the group's loops go too), 8 slices in pairs 1.132 -> 1.102 ms,
+// where the texel loads bind: L1 serves 16 bytes per sample and slice at 90 % of its wavefront rate.
+// The slices of one scan share the geometry: positions, ranges and texel indices are formed once per sample and
+// only the texel loads and the accumulation are per slice. A position advances shifted left by 2, so that its
+// floor is the high word. Every lane of the warp must call this (valid = false for lanes without a ray); count
+// (<= G) is uniform over the CTA.
 template <class TX, int G>
 __device__ __forceinline__ void ray_sum_group(const int4 P, bool valid, const GeomDev& g, const TX* const (&txs)[G],
                                               const TX* const (&tys)[G], int count, float2 (&acc)[G]) {
     const bool ax = ray_axis(P);
     const int n_across = ax ? g.nx : g.ny;
-    const int ld = n_across + 3;
+    int ld = n_across + 3;
     int lo = 1, hi = 0;
     if (valid) trimmed_range(P, g, lo, hi);
     const bool any = lo <= hi;
     const int t0 = __reduce_min_sync(0xffffffffu, any ? lo : 0x7fffffff);
     const int t1 = __reduce_max_sync(0xffffffffu, any ? hi : -1);
+    // [c0, c1]: the indices inside every sampling lane's range
+    const int c0 = __reduce_max_sync(0xffffffffu, any ? lo : -1);
+    const int c1 = __reduce_min_sync(0xffffffffu, any ? hi : 0x7fffffff);
     f32x2 acc2[G];  // {c, p} sums per slice as packed pairs
 #pragma unroll
     for (int k = 0; k < G; ++k) acc2[k] = pack2(0.f, 0.f);
     if (t0 <= t1) {  // some lane of the warp samples the image (warp-uniform)
         // from here 0 <= t0 <= t1 < max(nx, ny): the bounds below cannot overflow
-        const long long step = ray_step(P), q0 = ray_q0(P);
         const TX* tex[G];
 #pragma unroll
         for (int k = 0; k < G; ++k) tex[k] = ax ? tys[k] : txs[k];
+        // position and texel row of sample t, stepped exactly: q = q0 + t step, base = t ld + 2; a lane without
+        // samples stays at texel 0
+        const long long q0 = any ? (ray_q0(P) + (long long)t0 * ray_step(P)) << 2 : 0, step = any ? ray_step(P) << 2 : 0;
+        if (!any) ld = 0;
+        int fl = (int)(q0 >> 32), base = any ? t0 * ld + 2 : 0;
+        unsigned fr = (unsigned)q0;
+        const int sfl = (int)(step >> 32);
+        const unsigned sfr = (unsigned)step;
+        auto advance = [&](int& idx, float& f) {
+            idx = base + fl;
+            f = __uint_as_float(0x3f800000u | (fr >> 9)) - 1.0f;
+            asm("add.cc.u32 %0, %0, %2; addc.s32 %1, %1, %3;" : "+r"(fr), "+r"(fl) : "r"(sfr), "r"(sfl));
+            base += ld;
+        };
         int t = t0;
-        // position and texel row of sample t, stepped exactly: q = q0 + t step, base = t ld + 2
-        long long q = q0 + (long long)t0 * step;
-        int base = t0 * ld + 2;
-        for (; t <= t1 - (kProjBatch - 1); t += kProjBatch) {
+        while (t <= t1 - (kProjBatch - 1)) {
             int idx[kProjBatch];
             float f[kProjBatch];
+            if (t >= c0 && t + (kProjBatch - 1) <= c1) {
 #pragma unroll
-            for (int u = 0; u < kProjBatch; ++u) {
-                const int tt = t + u;
-                idx[u] = (tt >= lo && tt <= hi) ? base + pos_floor(q) : 0;  // texel 0: zero padding
-                f[u] = frac_of(q);
-                q += step;
-                base += ld;
+                for (int u = 0; u < kProjBatch; ++u) advance(idx[u], f[u]);
+            } else {
+#pragma unroll
+                for (int u = 0; u < kProjBatch; ++u) {
+                    const int tt = t + u;
+                    advance(idx[u], f[u]);
+                    if (tt < lo || tt > hi) idx[u] = 0;  // texel 0: zero padding
+                }
             }
+            t += kProjBatch;
 #pragma unroll
             for (int k = 0; k < G; ++k) {
                 if (k >= count) break;
@@ -396,9 +345,11 @@ __device__ __forceinline__ void ray_sum_group(const int4 P, bool valid, const Ge
                 for (int u = 0; u < kProjBatch; ++u) acc2[k] = add2(acc2[k], lerp2(f[u], v[u]));
             }
         }
-        for (; t <= t1; ++t, q += step, base += ld) {
-            const int i1 = (t >= lo && t <= hi) ? base + pos_floor(q) : 0;
-            const float f = frac_of(q);
+        for (; t <= t1; ++t) {
+            int i1;
+            float f;
+            advance(i1, f);
+            if (t < lo || t > hi) i1 = 0;
 #pragma unroll
             for (int k = 0; k < G; ++k) {
                 if (k >= count) break;
@@ -413,7 +364,8 @@ __device__ __forceinline__ void ray_sum_group(const int4 P, bool valid, const Ge
 // One CTA per (geometry group, tile): group gi holds up to kProjGroup slices of one geometry (their
 // indices in groups[gi], -1 past the group's size); the block map counts tiles per group.
 // (the register budget allows DECT_PROJ_MINB 64-thread CTAs per SM, the same warps for every V)
-template <class S2, class TX, int V>
+// G: the most slices a group of the launch has (1: no two slices share a geometry).
+template <class S2, class TX, int V, int G>
 __global__ void __launch_bounds__(32 * V, DECT_PROJ_MINB * 2 / V) k_project(const SliceDesc* __restrict__ dsl,
                                                                           BlockMap map, const int4* __restrict__ groups,
                                                                           const TX* __restrict__ tx,
@@ -422,29 +374,29 @@ __global__ void __launch_bounds__(32 * V, DECT_PROJ_MINB * 2 / V) k_project(cons
     const int gi = slice_of(map, blockIdx.x, local);
     const int4 gs = __ldg(groups + gi);
     const int all[4] = {gs.x, gs.y, gs.z, gs.w};
-    int sl[kProjGroup];
+    int sl[G];
 #pragma unroll
-    for (int q = 0; q < kProjGroup; ++q) sl[q] = all[q];
+    for (int q = 0; q < G; ++q) sl[q] = all[q];
     const int count = 1 + (gs.y >= 0) + (gs.z >= 0) + (gs.w >= 0);
     const SliceDesc& d = dsl[sl[0]];
     int v, k;
     const bool valid = proj_ray<V>(local, d.g.nv, d.g.nb, v, k);
     const int64_t r = (int64_t)v * d.g.nb + k;
     const int4 P = valid ? __ldg(d.g.rays + r) : make_int4(0, 0, 0, 0);
-    const TX* txs[kProjGroup];
-    const TX* tys[kProjGroup];
+    const TX* txs[G];
+    const TX* tys[G];
 #pragma unroll
-    for (int q = 0; q < kProjGroup; ++q) {
+    for (int q = 0; q < G; ++q) {
         const SliceDesc& dq = dsl[q < count ? sl[q] : sl[0]];
         txs[q] = tx + dq.tx_off;
         tys[q] = ty + dq.ty_off;
     }
-    float2 acc[kProjGroup];
-    ray_sum_group<TX, kProjGroup>(P, valid, d.g, txs, tys, count, acc);
+    float2 acc[G];
+    ray_sum_group<TX, G>(P, valid, d.g, txs, tys, count, acc);
     const float w = ray_w(P);
     if (!valid) return;
 #pragma unroll
-    for (int q = 0; q < kProjGroup; ++q)
+    for (int q = 0; q < G; ++q)
         if (q < count) st2(out + dsl[sl[q]].sino_off + r, make_float2(w * acc[q].x, w * acc[q].y));
 }
 
@@ -456,38 +408,50 @@ __global__ void __launch_bounds__(32 * kProjViews, DECT_PROJ_MINB) k_project_pla
     const bool valid = proj_ray<kProjViews>(blockIdx.x, d.g.nv, d.g.nb, v, k);
     const int64_t r = (int64_t)v * d.g.nb + k;
     const int4 P = valid ? __ldg(d.g.rays + r) : make_int4(0, 0, 0, 0);
-    const float2 acc = ray_sum_sync(P, valid, d.g, tx, ty);
+    const float4* const txs[1] = {tx};
+    const float4* const tys[1] = {ty};
+    float2 acc[1];
+    ray_sum_group<float4, 1>(P, valid, d.g, txs, tys, 1, acc);
     const float w = ray_w(P);
     if (!valid) return;
-    out[r] = w * acc.x;
-    if (nch > 1) out[n + r] = w * acc.y;
+    out[r] = w * acc[0].x;
+    if (nch > 1) out[n + r] = w * acc[0].y;
+}
+
+template <class S2, class TX, int G>
+static void project_g(const SliceDesc* dsl, const BlockMap& map, int nblk, const int4* groups, const TX* tx,
+                      const TX* ty, S2* out, int views, cudaStream_t st) {
+    if (views == 8)
+        k_project<S2, TX, 8, G><<<nblk, 256, 0, st>>>(dsl, map, groups, tx, ty, out);
+    else if (views == 4)
+        k_project<S2, TX, 4, G><<<nblk, 128, 0, st>>>(dsl, map, groups, tx, ty, out);
+    else
+        k_project<S2, TX, 2, G><<<nblk, 64, 0, st>>>(dsl, map, groups, tx, ty, out);
 }
 
 template <class S2, class TX>
-static void project_t(const SliceDesc* dsl, const BlockMap& map, int nblk, const int4* groups, const TX* tx,
+static void project_t(const SliceDesc* dsl, const BlockMap& map, int nblk, const int4* groups, int group, const TX* tx,
                       const TX* ty, S2* out, int views, cudaStream_t st) {
-    if (views == 8)
-        k_project<S2, TX, 8><<<nblk, 256, 0, st>>>(dsl, map, groups, tx, ty, out);
-    else if (views == 4)
-        k_project<S2, TX, 4><<<nblk, 128, 0, st>>>(dsl, map, groups, tx, ty, out);
+    if (group > 1)
+        project_g<S2, TX, kProjGroup>(dsl, map, nblk, groups, tx, ty, out, views, st);
     else
-        k_project<S2, TX, 2><<<nblk, 64, 0, st>>>(dsl, map, groups, tx, ty, out);
+        project_g<S2, TX, 1>(dsl, map, nblk, groups, tx, ty, out, views, st);
 }
 
-void launch_project(const SliceDesc* dsl, const BlockMap& map, int nblk, const int4* groups, const void* tx,
+void launch_project(const SliceDesc* dsl, const BlockMap& map, int nblk, const int4* groups, int group, const void* tx,
                     const void* ty, void* out, int prec, int views, cudaStream_t st) {
     if (prec == PREC_F16)
-        project_t(dsl, map, nblk, groups, (const TexH*)tx, (const TexH*)ty, (__half2*)out, views, st);
+        project_t(dsl, map, nblk, groups, group, (const TexH*)tx, (const TexH*)ty, (__half2*)out, views, st);
     else if (prec == PREC_BF16)
-        project_t(dsl, map, nblk, groups, (const TexB*)tx, (const TexB*)ty, (__nv_bfloat162*)out, views, st);
+        project_t(dsl, map, nblk, groups, group, (const TexB*)tx, (const TexB*)ty, (__nv_bfloat162*)out, views, st);
     else
-        project_t(dsl, map, nblk, groups, (const float4*)tx, (const float4*)ty, (float2*)out, views, st);
+        project_t(dsl, map, nblk, groups, group, (const float4*)tx, (const float4*)ty, (float2*)out, views, st);
 }
 
 // single channel: float out, float2 texels
-void launch_project1(const SliceDesc* dsl, const BlockMap& map, int nblk, const int4* groups, const float2* tx,
-                     const float2* ty, float* out, int views, cudaStream_t st) {
-    project_t(dsl, map, nblk, groups, tx, ty, out, views, st);
+void launch_project1(const SliceDesc* dsl, const BlockMap& map, int nblk, const int4* groups, int group,
+                     const float2* tx, const float2* ty, float* out, int views, cudaStream_t st) {
+    project_t(dsl, map, nblk, groups, group, tx, ty, out, views, st);
 }
 
 int proj_group_size() { return kProjGroup; }
