@@ -18,8 +18,6 @@ namespace dect {
 static thread_local std::string g_err;
 void set_error(const std::string& m) { g_err = m; }
 
-void project_single(const SliceDesc& sd, const float* img, int nch, float2* scratch, float4* tx, float4* ty,
-                    float* out, cudaStream_t st);
 void launch_identity_precond(const SliceDesc* d, const BlockMap& rows, int nrows, const float2* r, float2* s,
                              double* partial, cudaStream_t st);
 }  // namespace dect
@@ -68,16 +66,16 @@ struct dect_geom {
     int4* rays = nullptr;
     float4* views = nullptr;
     // workspace of dect_project / dect_backproject (allocated on first use)
-    float2* ws_img = nullptr;
     float4* ws_tx = nullptr;
     float4* ws_ty = nullptr;
-    float2* ws_sino = nullptr;
-    // R^T workspace: descriptor with zero offsets, block-map prefixes {0, sweep CTAs, 0, pixel blocks},
-    // ws_C partial images
+    // R^T workspace: descriptor with zero offsets, block-map prefixes {0, sweep CTAs, 0, pixel blocks} for ws_C view
+    // groups (dect_backproject) and behind them for ws_Cr (the point responses of the solvers'
+    // preconditioners), as many partial images as the larger count
     SliceDesc* ws_desc = nullptr;
     int* ws_maps = nullptr;
     float2* ws_partial = nullptr;
-    int ws_C = 1;
+    int ws_C = 1, ws_Cr = 1;
+    bool ws_ready = false;
     double4_32a* rays64 = nullptr;  // float64 ray table (DECT_F64 calls; built on first use)
     // dect_fbp: per-view constants, fan pre-weights, filtered sinograms [2][V][Nb] (built on first use)
     float4* fbp_tab = nullptr;
@@ -193,10 +191,8 @@ extern "C" void dect_geometry_destroy(dect_geom* g) {
     if (!g) return;
     cudaFree(g->rays);
     cudaFree(g->views);
-    cudaFree(g->ws_img);
     cudaFree(g->ws_tx);
     cudaFree(g->ws_ty);
-    cudaFree(g->ws_sino);
     cudaFree(g->ws_desc);
     cudaFree(g->ws_maps);
     cudaFree(g->ws_partial);
@@ -208,22 +204,23 @@ extern "C" void dect_geometry_destroy(dect_geom* g) {
 }
 
 static dect_status geom_workspace(dect_geom* g) {
-    if (g->ws_img) return DECT_OK;
+    if (g->ws_ready) return DECT_OK;
     const auto& d = g->desc;
-    CUDA_TRY(dalloc(&g->ws_img, (size_t)g->n_pix()));
-    CUDA_TRY(dalloc(&g->ws_tx, (size_t)d.nx * (d.ny + 3)));
-    CUDA_TRY(dalloc(&g->ws_ty, (size_t)d.ny * (d.nx + 3)));
-    CUDA_TRY(dalloc(&g->ws_sino, (size_t)g->n_rays()));
-    CUDA_TRY(sweep_init_attributes());  // per device: the geometry's device is the current one
     const int tiles = sweep_tiles(d.nx, d.ny, kSweepTileDefault);
-    g->ws_C = sweep_groups(tiles, kSweepTileDefault);
-    CUDA_TRY(dalloc(&g->ws_partial, (size_t)g->ws_C * g->n_pix()));
-    CUDA_TRY(dalloc(&g->ws_desc, 1));
-    CUDA_TRY(dalloc(&g->ws_maps, 4));
+    g->ws_C = sweep_groups_single(tiles, d.n_views);
+    g->ws_Cr = sweep_groups(tiles, kSweepTileDefault);
+    if (!g->ws_tx) CUDA_TRY(dalloc(&g->ws_tx, (size_t)d.nx * (d.ny + 3)));
+    if (!g->ws_ty) CUDA_TRY(dalloc(&g->ws_ty, (size_t)d.ny * (d.nx + 3)));
+    CUDA_TRY(sweep_init_attributes());  // per device: the geometry's device is the current one
+    if (!g->ws_partial) CUDA_TRY(dalloc(&g->ws_partial, (size_t)std::max(g->ws_C, g->ws_Cr) * g->n_pix()));
+    if (!g->ws_desc) CUDA_TRY(dalloc(&g->ws_desc, 1));
+    if (!g->ws_maps) CUDA_TRY(dalloc(&g->ws_maps, 8));
     const SliceDesc sd = g->single();
-    const int maps[4] = {0, tiles * g->ws_C, 0, (int)((g->n_pix() + kPixPerBlock - 1) / kPixPerBlock)};
+    const int pix = (int)((g->n_pix() + kPixPerBlock - 1) / kPixPerBlock);
+    const int maps[8] = {0, tiles * g->ws_C, 0, pix, 0, tiles * g->ws_Cr, 0, pix};
     CUDA_TRY(cudaMemcpy(g->ws_desc, &sd, sizeof(SliceDesc), cudaMemcpyHostToDevice));
     CUDA_TRY(cudaMemcpy(g->ws_maps, maps, sizeof(maps), cudaMemcpyHostToDevice));
+    g->ws_ready = true;
     return DECT_OK;
 }
 
@@ -249,7 +246,7 @@ extern "C" dect_status dect_project(dect_geom* g, int32_t nch, int32_t dtype, co
     }
     dect_status st = geom_workspace(g);
     if (st != DECT_OK) return st;
-    project_single(g->single(), (const float*)x, nch, g->ws_img, g->ws_tx, g->ws_ty, (float*)sino, as_stream(stream));
+    project_single(g->single(), (const float*)x, nch, g->ws_tx, g->ws_ty, (float*)sino, as_stream(stream));
     CUDA_TRY(cudaGetLastError());
     return DECT_OK;
 }
@@ -270,8 +267,8 @@ extern "C" dect_status dect_backproject(dect_geom* g, int32_t nch, int32_t dtype
     }
     dect_status st = geom_workspace(g);
     if (st != DECT_OK) return st;
-    backproject_single(g->single(), g->ws_desc, g->ws_maps, g->ws_C, kSweepTileDefault, (const float*)sino, nch,
-                       g->ws_sino, g->ws_partial, (float*)x, as_stream(stream));
+    backproject_single(g->single(), g->ws_desc, g->ws_maps, g->ws_C, (const float*)sino, nch,
+                       g->ws_partial, (float*)x, as_stream(stream));
     CUDA_TRY(cudaGetLastError());
     return DECT_OK;
 }
@@ -1363,8 +1360,8 @@ static dect_status compute_responses(dect_admm* A) {
         dect_geom* g = A->geoms[b];
         dect_status ws = geom_workspace(g);
         if (ws != DECT_OK) return ws;
-        project_single(sd, A->stage, 2, g->ws_img, g->ws_tx, g->ws_ty, A->stage + 2 * np, st);
-        backproject_single(sd, g->ws_desc, g->ws_maps, g->ws_C, kSweepTileDefault, A->stage + 2 * np, 2, g->ws_sino,
+        project_single(sd, A->stage, 2, g->ws_tx, g->ws_ty, A->stage + 2 * np, st);
+        backproject_single(sd, g->ws_desc, g->ws_maps + 4, g->ws_Cr, A->stage + 2 * np, 2,
                            g->ws_partial, A->stage, st);
         launch_interleave(A->stage, np, A->r + sd.img_off, st);
         // one-slice descriptor and column map

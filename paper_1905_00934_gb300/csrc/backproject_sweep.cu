@@ -101,6 +101,18 @@ __device__ __forceinline__ void stage_arrive(int s) {
     if (s) bar_arrive<ID + 1, THREADS>(); else bar_arrive<ID, THREADS>();
 }
 
+// a planar sinogram of two channels, the second n_views n_bins elements behind the first
+struct PlanarPair {
+    float v;
+};
+__device__ __forceinline__ float2 load_pair(const PlanarPair* p, unsigned e, unsigned n) {
+    return make_float2(__ldg(&p[e].v), __ldg(&p[e + (size_t)n].v));
+}
+template <class S2>
+__device__ __forceinline__ float2 load_pair(const S2* p, unsigned e, unsigned) {
+    return ldg2(p + e);
+}
+
 template <int N>
 struct VecF;
 template <>
@@ -191,7 +203,7 @@ __device__ __forceinline__ int window_bins(const GeomDev& g, float cx, float cy,
     return (int)fminf(fmaf(w, 1.0005f, 2.f * kBinEps), 1022.f) + 1;
 }
 
-// NCH = 2: sinogram S2 pairs {c, p}, float2 partial images. NCH = 1: float sinogram and partial images,
+// NCH = 2: sinogram S2 pairs {c, p} (or PlanarPair), float2 partial images. NCH = 1: float sinogram and partial images,
 // optionally multiplied per ray by rw[ray] and per slice by scale[slice] as the rays are staged (the weighted R^T
 // of a Gauss-Newton operator).
 // CLUSTER: the C CTAs of a tile (consecutive blocks) form a thread-block cluster and add their tiles through
@@ -251,6 +263,7 @@ __global__ void __launch_bounds__(GatherShape<TILE, NCH, SG>::kThreads, GatherSh
 #pragma unroll
         for (int q = 0; q < SG; ++q) sn[q] = sino + dsl[sl[q]].sino_off;
         const float sscale = (NCH == 1 && scale) ? __ldg(scale + sl[0]) : 1.0f;
+        const unsigned n_rays = (unsigned)g.nv * (unsigned)g.nb;
         // the tile's rectangle (clipped to the image) widened by one pixel: a ray with a weight at one of its
         // pixels passes through it (inside the image's one-pixel margin, in front of a fan source)
         const int te = min(ti + TILE, nx) - 1, tf = min(tj + TILE, ny) - 1;
@@ -390,7 +403,7 @@ __global__ void __launch_bounds__(GatherShape<TILE, NCH, SG>::kThreads, GatherSh
                                     if constexpr (NCH == 2) {
 #pragma unroll
                                         for (int q = 0; q < SG; ++q) {
-                                            const float2 sv = q < count ? ldg2(sn[q] + e) : make_float2(0.f, 0.f);
+                                            const float2 sv = q < count ? load_pair(sn[q], e, n_rays) : make_float2(0.f, 0.f);
                                             x[i][2 * q] = sv.x;
                                             x[i][2 * q + 1] = sv.y;
                                         }
@@ -667,7 +680,7 @@ static cudaError_t sweep_attr() {
 cudaError_t sweep_init_attributes() {
     cudaError_t e = cudaSuccess;
     for (cudaError_t r : {sweep_attr<float2, 2, 32>(), sweep_attr<__half2, 2, 32>(), sweep_attr<__nv_bfloat162, 2, 32>(),
-                          sweep_attr<float, 1, 32>(), sweep_attr<float2, 2, 64>(), sweep_attr<__half2, 2, 64>(),
+                          sweep_attr<float, 1, 32>(), sweep_attr1<PlanarPair, 2, 32, false, 1>(), sweep_attr<float2, 2, 64>(), sweep_attr<__half2, 2, 64>(),
                           sweep_attr<__nv_bfloat162, 2, 64>(), sweep_attr<float, 1, 64>()})
         if (e == cudaSuccess) e = r;
     return e;
@@ -794,15 +807,42 @@ void launch_bp_finalize(int mode, const SliceDesc* dsl, const BlockMap& pix, int
     }
 }
 
-void backproject_single(const SliceDesc& sd, const SliceDesc* d_dev, const int* maps, int C, int tile, const float* sino,
-                        int nch, float2* packed, float2* partial, float* out, cudaStream_t st) {
-    const int64_t nr = (int64_t)sd.g.nv * sd.g.nb, np = (int64_t)sd.g.nx * sd.g.ny;
-    launch_pack_planar(sino, nch, nr, packed, st);
+// out[pixel] = sum of the C single-channel partial images, in order (one slice)
+__global__ void __launch_bounds__(256) k_sum_partials(int64_t np, int C, const float* __restrict__ partial,
+                                                      float* __restrict__ out) {
+    const int64_t e = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    if (e >= np) return;
+    float s = 0.f;
+    for (int c = 0; c < C; ++c) s += __ldg(partial + c * np + e);
+    out[e] = s;
+}
+
+void backproject_single(const SliceDesc& sd, const SliceDesc* d_dev, const int* maps, int C, const float* sino, int nch,
+                        float2* partial, float* out, cudaStream_t st) {
+    const int64_t np = (int64_t)sd.g.nx * sd.g.ny;
     const BlockMap smap{maps, 1}, pmap{maps + 2, 1};
-    launch_bp_sweep(d_dev, smap, sweep_tiles(sd.g.nx, sd.g.ny, tile) * C, C, tile, false, 1, nullptr, packed, partial,
-                    np, PREC_F32, nullptr, st);
-    k_bp_finalize<BP_PLAIN><<<(unsigned)((np + 255) / 256), fin_threads(BP_PLAIN), 0, st>>>(d_dev, pmap, C, partial, np, nullptr,
-                                                                         BpEpilogue{}, out, nch);
+    const int nblk = sweep_tiles(sd.g.nx, sd.g.ny, 32) * C;
+    if (nch > 1) {
+        using Sh = GatherShape<32, 2, 1>;
+        k_bp_gather<PlanarPair, 2, 32><<<nblk, Sh::kThreads, Sh::kBytes, st>>>(
+            d_dev, smap, C, nullptr, (const PlanarPair*)sino, partial, np, nullptr, nullptr, nullptr);
+        k_bp_finalize<BP_PLAIN><<<(unsigned)((np + 255) / 256), fin_threads(BP_PLAIN), 0, st>>>(
+            d_dev, pmap, C, partial, np, nullptr, BpEpilogue{}, out, nch);
+    } else {
+        using Sh = GatherShape<32, 1, 1>;
+        k_bp_gather<float, 1, 32><<<nblk, Sh::kThreads, Sh::kBytes, st>>>(d_dev, smap, C, nullptr, sino, (float*)partial,
+                                                                          np, nullptr, nullptr, nullptr);
+        k_sum_partials<<<(unsigned)((np + 255) / 256), 256, 0, st>>>(np, C, (const float*)partial, out);
+    }
+}
+
+// About 6000 CTAs (eight waves) at most, 11 groups at most and four views each at least. Measured per call and
+// pair of bases: 512^2 (256 tiles) 395 us at 6 groups, 368 at 11, 372 at 16; 256^2: 95, 83, 87; 93^2: 31, 30, 31.
+int sweep_groups_single(int tiles, int nv) {
+    int C = 6000 / (tiles > 0 ? tiles : 1);
+    C = C > 11 ? 11 : (C < 2 ? 2 : C);
+    const int by_views = (nv + 3) / 4;
+    return C < by_views ? C : by_views;
 }
 
 }  // namespace dect

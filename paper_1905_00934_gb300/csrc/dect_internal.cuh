@@ -185,12 +185,13 @@ void launch_bp_finalize(int mode, const SliceDesc* dsl, const BlockMap& pix, int
                         int64_t stride, float2* out, const BpEpilogue& ep, cudaStream_t st);
 // Single-slice planar R^T (dect_backproject): sino [nch][nv][nb] -> out [nch][ny][nx]. d_dev is the
 // slice's descriptor on the device with zero offsets; maps holds the sweep and pixel-block prefixes
-// {0, sweep_tiles * C, 0, pixel blocks}; packed holds nv*nb float2, partial C*nx*ny float2.
-void backproject_single(const SliceDesc& sd, const SliceDesc* d_dev, const int* maps, int C, int tile, const float* sino,
-                        int nch, float2* packed, float2* partial, float* out, cudaStream_t st);
-void project_single(const SliceDesc& sd, const float* img, int nch, float2* scratch, float4* tx, float4* ty,
-                    float* out, cudaStream_t st);
-void launch_pack_planar(const float* in, int nch, int64_t n, float2* out, cudaStream_t st);
+// {0, sweep_tiles * C, 0, pixel blocks}; partial C*nx*ny float2.
+void backproject_single(const SliceDesc& sd, const SliceDesc* d_dev, const int* maps, int C, const float* sino, int nch,
+                        float2* partial, float* out, cudaStream_t st);
+// view groups of a single R^T call on a slice with `tiles` tiles and nv views
+int sweep_groups_single(int tiles, int nv);
+void project_single(const SliceDesc& sd, const float* img, int nch, float4* tx, float4* ty, float* out,
+                    cudaStream_t st);
 int texture_x_blocks(int nx, int ny);
 int texture_y_blocks(int nx, int ny);
 constexpr int kRaysPerBlock = 256;

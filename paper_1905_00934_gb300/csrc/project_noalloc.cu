@@ -85,9 +85,7 @@ extern "C" dect_status dect_project_noalloc(const dect_geom* g, int32_t nch, con
     }
     float4* tx = reinterpret_cast<float4*>(base);
     float4* ty = tx + (size_t)d->nx * (d->ny + 3);
-    float2* img = reinterpret_cast<float2*>(ty + (size_t)d->ny * (d->nx + 3));
-    dect::project_single(dect::geom_single_of(g), x_dev, nch, img, tx, ty, sino_dev,
-                         reinterpret_cast<cudaStream_t>(stream));
+    dect::project_single(dect::geom_single_of(g), x_dev, nch, tx, ty, sino_dev, reinterpret_cast<cudaStream_t>(stream));
     e = cudaGetLastError();
     if (e != cudaSuccess) {
         dect::set_error(std::string("dect_project_noalloc: ") + cudaGetErrorString(e));

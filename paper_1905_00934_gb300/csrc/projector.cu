@@ -187,13 +187,6 @@ void launch_textures1(const SliceDesc* dsl, const BlockMap& mx, int nbx, const B
     k_texture_y<float2, float><<<nby, 256, 0, st>>>(dsl, my, img, ty);
 }
 
-// planar input (1 or 2 channels) -> interleaved float2 image
-__global__ void k_pack_planar(const float* __restrict__ in, int nch, int64_t n, float2* __restrict__ out) {
-    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= n) return;
-    out[e] = make_float2(__ldg(in + e), nch > 1 ? __ldg(in + n + e) : 0.0f);
-}
-
 // ---------------------------------------------------------------------------------------------
 // forward projector
 
@@ -400,22 +393,24 @@ __global__ void __launch_bounds__(32 * V, DECT_PROJ_MINB * 2 / V) k_project(cons
         if (q < count) st2(out + dsl[sl[q]].sino_off + r, make_float2(w * acc[q].x, w * acc[q].y));
 }
 
-__global__ void __launch_bounds__(32 * kProjViews, DECT_PROJ_MINB) k_project_planar(SliceDesc d, const float4* __restrict__ tx,
-                                                                    const float4* __restrict__ ty,
-                                                                    float* __restrict__ out, int nch) {
+// one slice, planar output; TX = float4 texels of two channels or float2 texels of one
+template <class TX>
+__global__ void __launch_bounds__(32 * kProjViews, DECT_PROJ_MINB) k_project_planar(SliceDesc d, const TX* __restrict__ tx,
+                                                                    const TX* __restrict__ ty,
+                                                                    float* __restrict__ out) {
     const int64_t n = (int64_t)d.g.nv * d.g.nb;
     int v, k;
     const bool valid = proj_ray<kProjViews>(blockIdx.x, d.g.nv, d.g.nb, v, k);
     const int64_t r = (int64_t)v * d.g.nb + k;
     const int4 P = valid ? __ldg(d.g.rays + r) : make_int4(0, 0, 0, 0);
-    const float4* const txs[1] = {tx};
-    const float4* const tys[1] = {ty};
+    const TX* const txs[1] = {tx};
+    const TX* const tys[1] = {ty};
     float2 acc[1];
-    ray_sum_group<float4, 1>(P, valid, d.g, txs, tys, 1, acc);
+    ray_sum_group<TX, 1>(P, valid, d.g, txs, tys, 1, acc);
     const float w = ray_w(P);
     if (!valid) return;
     out[r] = w * acc[0].x;
-    if (nch > 1) out[n + r] = w * acc[0].y;
+    if (sizeof(TX) == sizeof(float4)) out[n + r] = w * acc[0].y;
 }
 
 template <class S2, class TX, int G>
@@ -459,53 +454,62 @@ int proj_group_size() { return kProjGroup; }
 // ---------------------------------------------------------------------------------------------
 // single-slice planar entry points (dect_project / dect_backproject)
 
-__global__ void k_texture_x_single(SliceDesc d, const float2* __restrict__ img, float4* __restrict__ tx) {
-    // same as k_texture_x for one slice without a block map
-    __shared__ float2 tile[33][33];
+// image value at (j, i) of a planar image, zero outside
+__device__ __forceinline__ void planar_at(const float* __restrict__ img, int nx, int ny, int j, int i, float2& o) {
+    const size_t e = (size_t)j * nx + i;
+    o = (j < 0 || j >= ny || i < 0 || i >= nx) ? make_float2(0.f, 0.f)
+                                               : make_float2(__ldg(img + e), __ldg(img + (size_t)nx * ny + e));
+}
+__device__ __forceinline__ void planar_at(const float* __restrict__ img, int nx, int ny, int j, int i, float& o) {
+    o = (j < 0 || j >= ny || i < 0 || i >= nx) ? 0.f : __ldg(img + (size_t)j * nx + i);
+}
+
+// Both pair textures of one planar image in one launch (the first nbx blocks write TX as k_texture_x does, the
+// others TY); IM = float2 (two channels) with TX = float4, or float with float2
+template <class TX, class IM>
+__global__ void __launch_bounds__(256) k_textures_planar(SliceDesc d, int nbx, const float* __restrict__ img,
+                                                         TX* __restrict__ tx, TX* __restrict__ ty) {
+    __shared__ IM tile[33][33];
     const int nx = d.g.nx, ny = d.g.ny;
+    if ((int)blockIdx.x >= nbx) {
+        const int ld = nx + 3;
+        const int64_t e = (int64_t)(blockIdx.x - nbx) * blockDim.x + threadIdx.x;
+        if (e >= (int64_t)ny * ld) return;
+        const int j = (int)(e / ld), ii = (int)(e % ld);
+        IM a, b;
+        planar_at(img, nx, ny, j, ii - 2, a);
+        planar_at(img, nx, ny, j, ii - 1, b);
+        sttex(ty + e, a, b);
+        return;
+    }
     const int tiles_i = (nx + 31) / 32;
     const int jt = (blockIdx.x / tiles_i) * 32, it = (blockIdx.x % tiles_i) * 32;
-    for (int e = threadIdx.x; e < 33 * 32; e += blockDim.x) {
-        const int rr = e / 32, cc = e % 32;
-        tile[rr][cc] = img_at(img, nx, ny, jt - 2 + rr, it + cc);
-    }
+    for (int e = threadIdx.x; e < 33 * 32; e += blockDim.x) planar_at(img, nx, ny, jt - 2 + e / 32, it + e % 32, tile[e / 32][e % 32]);
     __syncthreads();
     const int ld = ny + 3;
     for (int e = threadIdx.x; e < 32 * 32; e += blockDim.x) {
         const int ci = e / 32, cj = e % 32;
         const int i = it + ci, jj = jt + cj;
-        if (i < nx && jj < ld) {
-            const float2 a = tile[cj][ci], b = tile[cj + 1][ci];
-            tx[(size_t)i * ld + jj] = make_float4(a.x, a.y, b.x, b.y);
-        }
+        if (i < nx && jj < ld) sttex(tx + (size_t)i * ld + jj, tile[cj][ci], tile[cj + 1][ci]);
     }
 }
 
-__global__ void k_texture_y_single(SliceDesc d, const float2* __restrict__ img, float4* __restrict__ ty) {
-    const int nx = d.g.nx, ny = d.g.ny, ld = nx + 3;
-    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= (int64_t)ny * ld) return;
-    const int j = (int)(e / ld), ii = (int)(e % ld);
-    const float2 a = img_at(img, nx, ny, j, ii - 2), b = img_at(img, nx, ny, j, ii - 1);
-    ty[e] = make_float4(a.x, a.y, b.x, b.y);
-}
-
-// `scratch` must hold nx*ny float2
 // The buffers passed here are the slice's own (already offset), so the descriptor's offsets are
-// cleared before the kernels see it.
-void project_single(const SliceDesc& sd_in, const float* img, int nch, float2* scratch, float4* tx, float4* ty,
-                    float* out, cudaStream_t st) {
+// cleared before the kernels see it. One channel takes texels of half the size.
+void project_single(const SliceDesc& sd_in, const float* img, int nch, float4* tx, float4* ty, float* out,
+                    cudaStream_t st) {
     SliceDesc sd = sd_in;
     sd.img_off = sd.sino_off = sd.tx_off = sd.ty_off = sd.fft_off = sd.h_off = 0;
-    const int64_t np = (int64_t)sd.g.nx * sd.g.ny;
-    k_pack_planar<<<(unsigned)((np + 255) / 256), 256, 0, st>>>(img, nch, np, scratch);
-    k_texture_x_single<<<tx_blocks(sd.g.nx, sd.g.ny), 256, 0, st>>>(sd, scratch, tx);
-    k_texture_y_single<<<ty_blocks(sd.g.nx, sd.g.ny), 256, 0, st>>>(sd, scratch, ty);
-    k_project_planar<<<proj_tiles(sd.g.nv, sd.g.nb, kProjViews), 32 * kProjViews, 0, st>>>(sd, tx, ty, out, nch);
-}
-
-void launch_pack_planar(const float* in, int nch, int64_t n, float2* out, cudaStream_t st) {
-    k_pack_planar<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(in, nch, n, out);
+    const int nbx = tx_blocks(sd.g.nx, sd.g.ny), nb = nbx + ty_blocks(sd.g.nx, sd.g.ny);
+    const int tiles = proj_tiles(sd.g.nv, sd.g.nb, kProjViews);
+    if (nch > 1) {
+        k_textures_planar<float4, float2><<<nb, 256, 0, st>>>(sd, nbx, img, tx, ty);
+        k_project_planar<float4><<<tiles, 32 * kProjViews, 0, st>>>(sd, tx, ty, out);
+    } else {
+        float2 *tx1 = (float2*)tx, *ty1 = (float2*)ty;
+        k_textures_planar<float2, float><<<nb, 256, 0, st>>>(sd, nbx, img, tx1, ty1);
+        k_project_planar<float2><<<tiles, 32 * kProjViews, 0, st>>>(sd, tx1, ty1, out);
+    }
 }
 
 int texture_x_blocks(int nx, int ny) { return tx_blocks(nx, ny); }
