@@ -77,9 +77,10 @@ struct dect_geom {
     int ws_C = 1, ws_Cr = 1;
     bool ws_ready = false;
     double4_32a* rays64 = nullptr;  // float64 ray table (DECT_F64 calls; built on first use)
-    // dect_fbp: per-view constants, fan pre-weights, filtered sinograms [2][V][Nb] (built on first use)
+    // dect_fbp: per-view constants, fan pre-weights, filtered rows (built on first use)
     float4* fbp_tab = nullptr;
-    float* fbp_prew = nullptr;
+    float* fbp_prew = nullptr;  // pre-weights (fan)
+    float* fbp_ramp = nullptr;  // the ramp filter's odd taps
     float* fbp_q = nullptr;
 
     int64_t n_rays() const { return (int64_t)desc.n_views * desc.n_bins; }
@@ -199,6 +200,7 @@ extern "C" void dect_geometry_destroy(dect_geom* g) {
     cudaFree(g->rays64);
     cudaFree(g->fbp_tab);
     cudaFree(g->fbp_prew);
+    cudaFree(g->fbp_ramp);
     cudaFree(g->fbp_q);
     delete g;
 }
@@ -401,16 +403,26 @@ static dect_status fbp_prepare(dect_geom* g, FbpDev& f) {
             e = dalloc(&pw, w.size());
             if (e == cudaSuccess) e = cudaMemcpy(pw, w.data(), sizeof(float) * w.size(), cudaMemcpyHostToDevice);
         }
+        std::vector<float> taps((d.n_bins + 1) / 2);
+        for (size_t j = 0; j < taps.size(); ++j) {
+            const double m = 2.0 * (double)j + 1.0;
+            taps[j] = (float)(1.0 / (M_PI * M_PI * m * m));
+        }
+        float* ramp = nullptr;
+        if (e == cudaSuccess) e = dalloc(&ramp, taps.size());
+        if (e == cudaSuccess) e = cudaMemcpy(ramp, taps.data(), sizeof(float) * taps.size(), cudaMemcpyHostToDevice);
         float* q = nullptr;
-        if (e == cudaSuccess) e = dalloc(&q, (size_t)2 * g->n_rays());
+        if (e == cudaSuccess) e = dalloc(&q, fbp_q_floats(d.n_views, d.n_bins));
         if (e != cudaSuccess) {
             cudaFree(dt);
             cudaFree(pw);
+            cudaFree(ramp);
             cudaFree(q);
             CUDA_TRY(e);
         }
         g->fbp_tab = dt;
         g->fbp_prew = pw;
+        g->fbp_ramp = ramp;
         g->fbp_q = q;
     }
     f.nx = d.nx;
@@ -428,6 +440,7 @@ static dect_status fbp_prepare(dect_geom* g, FbpDev& f) {
     f.scale = (float)((fan ? 2.0 * M_PI : M_PI) / d.n_views);
     f.tab = g->fbp_tab;
     f.prew = g->fbp_prew;
+    f.ramp = g->fbp_ramp;
     return DECT_OK;
 }
 

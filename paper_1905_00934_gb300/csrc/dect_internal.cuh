@@ -331,7 +331,10 @@ struct FbpDev {
     float gain, scale;   // filter gain (1/du, or 1/(2 du SOD/SDD)); backprojection factor (pi/V, 2 pi/V)
     const float4* tab;   // [nv]: parallel {c/du, s/du, k0, 0}; fan {c, s, 0, 0}
     const float* prew;   // [nb] fan pre-weight SOD / sqrt(SOD^2 + s^2), or null
+    const float* ramp;   // [(nb + 1) / 2] odd taps 1 / (pi^2 (2j + 1)^2)
 };
+// q: fbp_q_floats(n_views, n_bins) floats of scratch for the filtered rows
+size_t fbp_q_floats(int nv, int nb);
 void launch_fbp(const FbpDev& f, int nch, const float* sino, float* q, float* x, bool clamp, cudaStream_t st);
 void launch_cdm_start(int64_t n, const float* m_l, float inv_abar, float mu0, float* a_c, float* a_p, float* mu,
                       float* zero, cudaStream_t st);
