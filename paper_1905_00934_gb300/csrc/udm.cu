@@ -6,9 +6,10 @@
 // and f_h, f_l at the trial point a + delta enter, the 4 evaluations of f of Table 1; the
 // sums at a trial point that is kept are the next iteration's sums at a, so an iteration
 // makes one pass over the energies (one exp2 and eight FMAs per bin), not two.
-// What bounds it: issue (73 % active; the exponentials take 25 % of their unit). Measured on GB300, 737280 rays
-// of 121 bins: 10 iterations 878 -> 479 us (one pass per iteration, two rays per thread, the bare exponential
-// where nothing underflows); one iteration inside the solver, 8 slices: 0.739 -> 0.641 ms.
+// What bounds it: issue and the FMA pipe (a packed pair takes it for two cycles). Measured on GB300, 737280 rays
+// of 121 bins: 10 iterations 878 -> 453 us (one pass per iteration, two rays per thread and five CTAs, the bare
+// exponential where nothing underflows, no per-bin tests there, no division to choose the logarithm); one iteration
+// inside the solver, 8 slices: 0.739 -> 0.545 ms.
 // Energy
 // sums are float32 (compensated). Residuals come from the ratio of a spectral
 // sum to the measured transmission t = e^{-m}: f - m = -log(s / t), from
@@ -61,7 +62,10 @@ __device__ __forceinline__ void kahan_add(float& sum, float& comp, float v) {
 // longer one (the high spectrum if tail_high) in [n_both, n_end), neither from n_end on. Zero-weight
 // terms are exact zeros, so skipping them leaves every sum bit for bit as it was; the compensated
 // additions still run once per block of 8 bins over all ne bins, so the blocking is unchanged too.
-// Blocks that lie wholly in one range run an unrolled body without per-bin tests.
+// Blocks that lie wholly in one range run an unrolled body without per-bin tests. So does every other block where
+// the exponentials are the bare instruction's, hence finite: zero weights then add zeros (the tables in shared memory
+// end in zeros up to a multiple of 8 bins).
+__host__ __device__ constexpr int padded(int ne) { return (ne + 7) & ~7; }
 
 // 2^x. FAST: the bare instruction, for x above the range that underflows (in_fast_range), where it is what exp2f
 // returns; exp2f's scaling for the rest costs three more instructions per bin.
@@ -148,7 +152,7 @@ __device__ __forceinline__ void sums_jac(const float4* __restrict__ t1, const fl
         float bh[R], bl[R];
 #pragma unroll
         for (int k = 0; k < R; ++k) bh[k] = bl[k] = 0.f;
-        if (e0 + 8 <= sp.n_both) {
+        if (FAST ? e0 < sp.n_both : e0 + 8 <= sp.n_both) {
             // both spectra: the sum pairs {b_h, b_l}, {s_hc, s_hp}, {s_lc, s_lp} advance as packed float32
             // pairs, each sum taking bin_jac<3>'s terms in its order (the same bits, half the instructions)
             f32x2 bhl[R], sh2[R], sl2[R];
@@ -181,7 +185,7 @@ __device__ __forceinline__ void sums_jac(const float4* __restrict__ t1, const fl
                 o.slc[k] = z.x;
                 o.slp[k] = z.y;
             }
-        } else if (e0 >= sp.n_both && e0 + 8 <= sp.n_end) {
+        } else if (FAST ? e0 < sp.n_end : e0 >= sp.n_both && e0 + 8 <= sp.n_end) {
             if (sp.tail_high) {
 #pragma unroll
                 for (int u = 0; u < 8; ++u) {
@@ -199,7 +203,7 @@ __device__ __forceinline__ void sums_jac(const float4* __restrict__ t1, const fl
                         bin_jac<2, FAST>(a, b, ac[k], ap[k], bh[k], bl[k], o.shc[k], o.shp[k], o.slc[k], o.slp[k]);
                 }
             }
-        } else {
+        } else if (!FAST) {
             const int e1 = min(e0 + 8, sp.n_end);
             for (int e = e0; e < e1; ++e) {
                 const float4 a = t1[e], b = t2[e];
@@ -232,14 +236,14 @@ __device__ __forceinline__ void sums_val(const float4* __restrict__ t1, const Sp
         float bh[R], bl[R];
 #pragma unroll
         for (int k = 0; k < R; ++k) bh[k] = bl[k] = 0.f;
-        if (e0 + 8 <= sp.n_both) {
+        if (EXP == EXP_FAST ? e0 < sp.n_both : e0 + 8 <= sp.n_both) {
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
                 const float4 a = t1[e0 + u];
 #pragma unroll
                 for (int k = 0; k < R; ++k) bin_val<3, EXP>(a, ac[k], ap[k], bh[k], bl[k]);
             }
-        } else if (e0 >= sp.n_both && e0 + 8 <= sp.n_end) {
+        } else if (EXP == EXP_FAST ? e0 < sp.n_end : e0 >= sp.n_both && e0 + 8 <= sp.n_end) {
             if (sp.tail_high) {
 #pragma unroll
                 for (int u = 0; u < 8; ++u) {
@@ -255,7 +259,7 @@ __device__ __forceinline__ void sums_val(const float4* __restrict__ t1, const Sp
                     for (int k = 0; k < R; ++k) bin_val<2, EXP>(a, ac[k], ap[k], bh[k], bl[k]);
                 }
             }
-        } else {
+        } else if (EXP != EXP_FAST) {
             const int e1 = min(e0 + 8, sp.n_end);
             for (int e = e0; e < e1; ++e) {
                 const float4 a = t1[e];
@@ -322,12 +326,13 @@ __device__ __forceinline__ void spectral_sums_jac(const float4* __restrict__ t1,
     slp = o.slp[0];
 }
 
-// -log(a / b) for positive a, b: from the relative difference when the ratio is within [1/2, 2] (then
+// -log(a / b) for positive a, b: from the relative difference when the ratio is within (1/2, 2) (then
 // a - b is exact and log1p keeps its accuracy), from the ratio itself otherwise (photon-starved
-// rays whose model sum is orders of magnitude off the measurement, large trial steps)
+// rays whose model sum is orders of magnitude off the measurement, large trial steps). The test takes no division:
+// 2a > b exactly when the rounded a / b exceeds 1/2 (the ratio is then at least 1/2 + 2^-25, above the halfway point
+// to the next number), a < 2b when it is below 2, and doubling is exact.
 __device__ __forceinline__ float neg_log_ratio(float a, float b) {
-    const float q = a / b;
-    return (q > 0.5f && q < 2.0f) ? -log1pf((a - b) / b) : -logf(q);
+    return (a + a > b && a < b + b) ? -log1pf((a - b) / b) : -logf(a / b);
 }
 
 // a * b - c * d with one rounding of the result (the rounding error of c * d is recovered by an fma)
@@ -530,27 +535,30 @@ __device__ void lm_ray64(const float4* __restrict__ t1, const double4_32a* __res
 }
 
 __device__ __forceinline__ void load_tables(const SpecDev& sp, float4* t1, float4* t2) {
-    for (int e = threadIdx.x; e < sp.ne; e += blockDim.x) {
-        t1[e] = __ldg(sp.t1 + e);
-        t2[e] = __ldg(sp.t2 + e);
+    for (int e = threadIdx.x; e < padded(sp.ne); e += blockDim.x) {
+        const bool in = e < sp.ne;
+        t1[e] = in ? __ldg(sp.t1 + e) : make_float4(0.f, 0.f, 0.f, 0.f);
+        t2[e] = in ? __ldg(sp.t2 + e) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
     __syncthreads();
 }
 
+// CTAs per SM that two rays per thread leave room for: holds the registers at 102 (126 otherwise; four, five, six CTAs:
+// 10 iterations of 737280 rays 468 / 453 / 477 us, one in the solver 0.600 / 0.545 / 0.597 ms)
+constexpr int kUdmCtas = 5;
+
 // ADMM a-update fused with the a-block of the dual update (Eq. 11) and the a-block residual sums:
 // partial[4*blk + {0,1}] = sum (a - Rx)^2 (c, p); partial[4*blk + {2,3}] = sum (a - a_old)^2.
 template <class S2, bool F64, int R>
-__global__ void __launch_bounds__(kRaysPerBlock / R) k_udm_admm(const SliceDesc* __restrict__ dsl, BlockMap map, SpecDev sp,
-                                                            const float4* __restrict__ meas,
-                                                            const S2* __restrict__ Rx, S2* __restrict__ ua,
-                                                            S2* __restrict__ a, float* __restrict__ mu,
-                                                            uint8_t* __restrict__ status,
-                                                            const SliceScalars* __restrict__ sc, int iters,
-                                                            double* __restrict__ partial) {
+__global__ void __launch_bounds__(kRaysPerBlock / R, R == 2 ? kUdmCtas : 4)
+    k_udm_admm(const SliceDesc* __restrict__ dsl, BlockMap map, SpecDev sp, const float4* __restrict__ meas,
+               const S2* __restrict__ Rx, S2* __restrict__ ua, S2* __restrict__ a, float* __restrict__ mu,
+               uint8_t* __restrict__ status, const SliceScalars* __restrict__ sc, int iters,
+               double* __restrict__ partial) {
     extern __shared__ float4 tabs[];
     float4* t1 = tabs;
-    float4* t2 = tabs + sp.ne;
-    double4_32a* w1 = reinterpret_cast<double4_32a*>(tabs + 2 * sp.ne);
+    float4* t2 = tabs + padded(sp.ne);
+    double4_32a* w1 = reinterpret_cast<double4_32a*>(tabs + 2 * padded(sp.ne));
     double4_32a* w2 = w1 + sp.ne;
     if (F64)
         for (int e = threadIdx.x; e < sp.ne; e += blockDim.x) {
@@ -616,13 +624,12 @@ __global__ void __launch_bounds__(kRaysPerBlock / R) k_udm_admm(const SliceDesc*
 
 // Initial decomposition: rho = (0, rho_p), v = 0, from a = (m_l / abar, 0), mu = mu0.
 template <class S2, int R>
-__global__ void __launch_bounds__(kRaysPerBlock / R) k_udm_init(const SliceDesc* __restrict__ dsl, BlockMap map, SpecDev sp,
-                                                            const float4* __restrict__ meas, S2* __restrict__ a,
-                                                            float* __restrict__ mu, double rho_p, int iters,
-                                                            float abar, float mu0) {
+__global__ void __launch_bounds__(kRaysPerBlock / R, R == 2 ? kUdmCtas : 4)
+    k_udm_init(const SliceDesc* __restrict__ dsl, BlockMap map, SpecDev sp, const float4* __restrict__ meas,
+               S2* __restrict__ a, float* __restrict__ mu, double rho_p, int iters, float abar, float mu0) {
     extern __shared__ float4 tabs[];
     float4* t1 = tabs;
-    float4* t2 = tabs + sp.ne;
+    float4* t2 = tabs + padded(sp.ne);
     load_tables(sp, t1, t2);
     int local;
     const int s = slice_of(map, blockIdx.x, local);
@@ -655,15 +662,14 @@ __global__ void __launch_bounds__(kRaysPerBlock / R) k_udm_init(const SliceDesc*
 
 // Public per-ray entry point (planar float arrays).
 template <int R>
-__global__ void __launch_bounds__(kRaysPerBlock / R) k_udm_rays(SpecDev sp, int64_t n, const float* __restrict__ mh,
-                                                            const float* __restrict__ ml, const float* __restrict__ wh,
-                                                            const float* __restrict__ wl, const float* __restrict__ vc,
-                                                            const float* __restrict__ vp, double rho_c, double rho_p,
-                                                            int iters, float* ac, float* ap, float* mu,
-                                                            uint8_t* __restrict__ status) {
+__global__ void __launch_bounds__(kRaysPerBlock / R, R == 2 ? kUdmCtas : 4)
+    k_udm_rays(SpecDev sp, int64_t n, const float* __restrict__ mh, const float* __restrict__ ml,
+               const float* __restrict__ wh, const float* __restrict__ wl, const float* __restrict__ vc,
+               const float* __restrict__ vp, double rho_c, double rho_p, int iters, float* ac, float* ap, float* mu,
+               uint8_t* __restrict__ status) {
     extern __shared__ float4 tabs[];
     float4* t1 = tabs;
-    float4* t2 = tabs + sp.ne;
+    float4* t2 = tabs + padded(sp.ne);
     load_tables(sp, t1, t2);
     const int64_t r0 = (int64_t)blockIdx.x * kRaysPerBlock + threadIdx.x;
     RayIn in[R];
@@ -707,7 +713,7 @@ __global__ void __launch_bounds__(kRaysPerBlock) k_lm_rays(const SliceDesc* __re
                                                            float* __restrict__ Rd) {
     extern __shared__ float4 tabs[];
     float4* t1 = tabs;
-    float4* t2 = tabs + sp.ne;
+    float4* t2 = tabs + padded(sp.ne);
     load_tables(sp, t1, t2);
     int local;
     const int s = slice_of(map, blockIdx.x, local);
@@ -737,7 +743,7 @@ __global__ void __launch_bounds__(kRaysPerBlock) k_lm_trial(const SliceDesc* __r
                                                             double* __restrict__ partial) {
     extern __shared__ float4 tabs[];
     float4* t1 = tabs;
-    float4* t2 = tabs + sp.ne;
+    float4* t2 = tabs + padded(sp.ne);
     load_tables(sp, t1, t2);
     int local;
     const int s = slice_of(map, blockIdx.x, local);
@@ -761,7 +767,7 @@ __global__ void __launch_bounds__(kRaysPerBlock) k_lm_trial(const SliceDesc* __r
     block_partials<1>(acc, partial);
 }
 
-static size_t tab_bytes(const SpecDev& sp) { return 2 * sizeof(float4) * (size_t)sp.ne; }
+static size_t tab_bytes(const SpecDev& sp) { return 2 * sizeof(float4) * (size_t)padded(sp.ne); }
 // ---- Eq. 4's data term, per ray -------------------------------------------------------------------
 
 // partial[blk] = sum over the block's rays of 1/2 (w_h r_h^2 + w_l r_l^2), r = f(q) - m at the
@@ -773,7 +779,7 @@ __global__ void __launch_bounds__(kRaysPerBlock) k_objective_rays(const SliceDes
                                                                   double* __restrict__ partial) {
     extern __shared__ float4 tabs[];
     float4* t1 = tabs;
-    float4* t2 = tabs + sp.ne;
+    float4* t2 = tabs + padded(sp.ne);
     load_tables(sp, t1, t2);
     int local;
     const SliceDesc& d = dsl[slice_of(map, blockIdx.x, local)];
@@ -816,12 +822,20 @@ __global__ void __launch_bounds__(kRaysPerBlock) k_forward_model_f32(SpecDev sp,
                                                                      float* __restrict__ op) {
     extern __shared__ float4 tabs[];
     float4* t1 = tabs;
-    float4* t2 = tabs + sp.ne;
+    float4* t2 = tabs + padded(sp.ne);
     load_tables(sp, t1, t2);
     const int64_t r = (int64_t)blockIdx.x * kRaysPerBlock + threadIdx.x;
     if (r >= n) return;
+    const float a[1] = {__ldg(ac + r)}, p[1] = {__ldg(ap + r)};
+    if (!jac && !oc) {  // (half of the sums, the same bits)
+        float sh[1], sl[1];
+        spectral_sums<1>(t1, sp, a, p, sh, sl);
+        if (fh) fh[r] = (float)(-log((double)sh[0]));
+        if (fl) fl[r] = (float)(-log((double)sl[0]));
+        return;
+    }
     float sh, sl, shc, shp, slc, slp;
-    spectral_sums_jac(t1, t2, sp, __ldg(ac + r), __ldg(ap + r), sh, sl, shc, shp, slc, slp);
+    spectral_sums_jac(t1, t2, sp, a[0], p[0], sh, sl, shc, shp, slc, slp);
     const double ish = 1.0 / (double)sh, isl = 1.0 / (double)sl;
     const double j0 = shc * ish, j1 = shp * ish, j2 = slc * isl, j3 = slp * isl;
     if (fh) fh[r] = (float)(-log((double)sh));

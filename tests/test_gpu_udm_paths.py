@@ -43,3 +43,31 @@ def test_long_calls_equal_short_calls_bit_for_bit(cuda_dev, n, iters):
         pstatus[sl] = cs
     for t, p in zip(state + [status], part + [pstatus]):
         assert torch.equal(t.view(torch.uint8), p.view(torch.uint8))
+
+
+@pytest.mark.parametrize("n_both, n_end, ne", [(1, 1, 2), (3, 5, 8), (7, 9, 17), (8, 16, 17), (9, 15, 24), (16, 16, 23),
+                                               (20, 22, 30)])
+@pytest.mark.parametrize("tail_high", [True, False])
+def test_padded_bins_equal_tested_bins_bit_for_bit(cuda_dev, n_both, n_end, ne, tail_high):
+    from paper_1905_00934_gb300 import Spectra
+
+    rng = np.random.default_rng(ne)
+    s = [rng.uniform(0.1, 1.0, ne) * (np.arange(ne) < (n_end if long else n_both)) for long in (tail_high, not tail_high)]
+    f_kn, f_p = rng.uniform(0.1, 0.3, ne), rng.uniform(0.05, 2.0, ne)
+    n = 5000
+    m = rng.uniform(0.0, 4.0, (2, n))
+    a = [rng.uniform(0.0, 4.0, n), rng.uniform(0.0, 0.5, n)]
+
+    def run(f_last):
+        # a bin that neither spectrum has: a large coefficient there takes every ray off the padded path
+        f_kn[ne - 1] = f_last
+        spec = Spectra(s[0], s[1], f_kn, f_p)
+        dev = lambda x: torch.tensor(x, dtype=torch.float32, device=cuda_dev)
+        state = [dev(a[0]), dev(a[1]), torch.full((n,), 1e-3, device=cuda_dev)]
+        status = torch.zeros(n, dtype=torch.uint8, device=cuda_dev)
+        spec.decompose(dev(m[0]), dev(m[1]), dev(np.exp(-m[0])), dev(np.exp(-m[1])), dev(a[0]), dev(a[1]), 1e-3, 1e-3,
+                       3, *state, status)
+        return torch.stack(state).view(torch.int32), status
+
+    for x, y in zip(run(0.2), run(1e6)):
+        assert torch.equal(x, y)
