@@ -64,17 +64,45 @@ __global__ void __launch_bounds__(256) k_alpha(const double* __restrict__ part, 
     }
 }
 
-// x += alpha p, r -= alpha A p (unless last) over the image blocks; R x += alpha q over the ray blocks
-template <class S2>
+// x += alpha p, r -= alpha A p (unless last) over the image blocks; R x += alpha q over the ray blocks.
+// SUMS: each block forms its slice's rs = <r, M^-1 r> and alpha itself, as k_rs_reduce and k_alpha do from the same
+// slots, and the slice's first block stores them. Two launches less per step, which is what small batches spend
+// their time on; the float64 sums of every block are what large ones could not hide (cg_small_batch).
+template <class S2, bool SUMS>
 __global__ void __launch_bounds__(256) k_cg_update(const SliceDesc* __restrict__ dsl, BlockMap pix, int nblk_pix,
-                                                   BlockMap rays, const SliceScalars* __restrict__ sc,
+                                                   BlockMap rays, SliceScalars* __restrict__ sc,
+                                                   const double* __restrict__ part_pap,
+                                                   const double* __restrict__ part_rs,
+                                                   const int* __restrict__ rows_prefix,
                                                    float2* __restrict__ x, const float2* __restrict__ p,
                                                    float2* __restrict__ r, const float2* __restrict__ Ap,
                                                    S2* __restrict__ Rx, const S2* __restrict__ q, int last) {
     int local;
     const bool img = (int)blockIdx.x < nblk_pix;
     const int sb = img ? slice_of(pix, blockIdx.x, local) : slice_of(rays, blockIdx.x - nblk_pix, local);
-    const float2 al = make_float2(sc[sb].alpha_f[0], sc[sb].alpha_f[1]);
+    float2 al;
+    if constexpr (SUMS) {
+        __shared__ float sal[2];
+        double v[4];  // <p, A p>, rs
+        slice_sum_pair_small(part_pap, pix.prefix, part_rs, rows_prefix, sb, v);
+        if (threadIdx.x == 0) {
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                const double a = v[c] > 0.0 ? v[2 + c] / v[c] : 0.0;
+                sal[c] = (float)a;
+                if (img && local == 0) {
+                    sc[sb].rs[c] = v[2 + c];
+                    sc[sb].pAp[c] = v[c];
+                    sc[sb].alpha[c] = a;
+                    sc[sb].alpha_f[c] = (float)a;
+                }
+            }
+        }
+        __syncthreads();
+        al = make_float2(sal[0], sal[1]);
+    } else {
+        al = make_float2(sc[sb].alpha_f[0], sc[sb].alpha_f[1]);
+    }
     if (img) {
         const int s = sb;
         const SliceDesc& d = dsl[s];
@@ -113,13 +141,36 @@ __global__ void __launch_bounds__(256) k_cg_update(const SliceDesc* __restrict__
     }
 }
 
-// p = s + beta p
+// p = s + beta p. SUMS: beta from the new rs, formed from its slots as k_rs_reduce does, over the rs that the last
+// k_cg_update stored (the next one stores the new rs).
+template <bool SUMS>
 __global__ void __launch_bounds__(256) k_cg_p(const SliceDesc* __restrict__ dsl, BlockMap pix,
-                                              const SliceScalars* __restrict__ sc, const float2* __restrict__ sv,
+                                              SliceScalars* __restrict__ sc, const double* __restrict__ part_rs,
+                                              const int* __restrict__ rows_prefix, const float2* __restrict__ sv,
                                               float2* __restrict__ p) {
     int local;
     const int s = slice_of(pix, blockIdx.x, local);
-    const float2 be = make_float2(sc[s].beta_f[0], sc[s].beta_f[1]);
+    float2 be;
+    if constexpr (SUMS) {
+        __shared__ float sbe[2];
+        double v[4];
+        slice_sum_pair_small(part_rs, rows_prefix, part_rs, rows_prefix, s, v);
+        if (threadIdx.x == 0) {
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                const double old = sc[s].rs[c], b = old > 0.0 ? v[c] / old : 0.0;
+                sbe[c] = (float)b;
+                if (local == 0) {
+                    sc[s].beta[c] = b;
+                    sc[s].beta_f[c] = (float)b;
+                }
+            }
+        }
+        __syncthreads();
+        be = make_float2(sbe[0], sbe[1]);
+    } else {
+        be = make_float2(sc[s].beta_f[0], sc[s].beta_f[1]);
+    }
     const SliceDesc& d = dsl[s];
     const int64_t k = (int64_t)local * 256 + threadIdx.x;
     if (k >= (int64_t)d.g.nx * d.g.ny) return;
@@ -505,15 +556,25 @@ void launch_rs_reduce(const double* part, const int* rows_prefix, SliceScalars* 
 void launch_alpha(const double* part, const int* bp_prefix, SliceScalars* sc, int B, cudaStream_t st) {
     k_alpha<<<B, 256, 0, st>>>(part, bp_prefix, sc);
 }
-void launch_cg_update(const SliceDesc* d, const BlockMap& pix, int np, const BlockMap& rays, int nr,
-                      const SliceScalars* sc, float2* x, const float2* p, float2* r, const float2* Ap, void* Rx,
-                      const void* q, int last, int prec, cudaStream_t st) {
-    DISPATCH_S2(prec, (k_cg_update<S2><<<np + nr, 256, 0, st>>>(d, pix, np, rays, sc, x, p, r, Ap, (S2*)Rx,
-                                                                 (const S2*)q, last)));
+void launch_cg_update(const SliceDesc* d, const BlockMap& pix, int np, const BlockMap& rays, int nr, SliceScalars* sc,
+                      const double* part_pap, const double* part_rs, const int* rows_prefix, bool sums, float2* x,
+                      const float2* p, float2* r, const float2* Ap, void* Rx, const void* q, int last, int prec,
+                      cudaStream_t st) {
+    if (sums)
+        DISPATCH_S2(prec, (k_cg_update<S2, true><<<np + nr, 256, 0, st>>>(
+                              d, pix, np, rays, sc, part_pap, part_rs, rows_prefix, x, p, r, Ap, (S2*)Rx, (const S2*)q,
+                              last)));
+    else
+        DISPATCH_S2(prec, (k_cg_update<S2, false><<<np + nr, 256, 0, st>>>(
+                              d, pix, np, rays, sc, part_pap, part_rs, rows_prefix, x, p, r, Ap, (S2*)Rx, (const S2*)q,
+                              last)));
 }
-void launch_cg_p(const SliceDesc* d, const BlockMap& pix, int np, const SliceScalars* sc, const float2* s, float2* p,
-                 cudaStream_t st) {
-    k_cg_p<<<np, 256, 0, st>>>(d, pix, sc, s, p);
+void launch_cg_p(const SliceDesc* d, const BlockMap& pix, int np, SliceScalars* sc, const double* part_rs,
+                 const int* rows_prefix, bool sums, const float2* s, float2* p, cudaStream_t st) {
+    if (sums)
+        k_cg_p<true><<<np, 256, 0, st>>>(d, pix, sc, part_rs, rows_prefix, s, p);
+    else
+        k_cg_p<false><<<np, 256, 0, st>>>(d, pix, sc, part_rs, rows_prefix, s, p);
 }
 void launch_image_update(const SliceDesc* d, const BlockMap& pix, int np, const SliceScalars* sc, double lam_c,
                          double lam_p, const float2* x, float4* y, float4* uy, float2* z, float2* uz, double* partial,

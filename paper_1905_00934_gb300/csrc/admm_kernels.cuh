@@ -10,11 +10,14 @@ void launch_sino_resid(const SliceDesc* d, const BlockMap& rays, int nr, const v
                        const void* Rx, void* b, int prec, cudaStream_t st);
 void launch_rs_reduce(const double* part, const int* rows_prefix, SliceScalars* sc, int B, int first, cudaStream_t st);
 void launch_alpha(const double* part, const int* bp_prefix, SliceScalars* sc, int B, cudaStream_t st);
-void launch_cg_update(const SliceDesc* d, const BlockMap& pix, int np, const BlockMap& rays, int nr,
-                      const SliceScalars* sc, float2* x, const float2* p, float2* r, const float2* Ap, void* Rx,
-                      const void* q, int last, int prec, cudaStream_t st);
-void launch_cg_p(const SliceDesc* d, const BlockMap& pix, int np, const SliceScalars* sc, const float2* s, float2* p,
-                 cudaStream_t st);
+// sums: the kernels form alpha, beta and rs from the slots themselves (at most 256 per slice), and launch_rs_reduce and
+// launch_alpha are left out; otherwise the three arguments before it are not read
+void launch_cg_update(const SliceDesc* d, const BlockMap& pix, int np, const BlockMap& rays, int nr, SliceScalars* sc,
+                      const double* part_pap, const double* part_rs, const int* rows_prefix, bool sums, float2* x,
+                      const float2* p, float2* r, const float2* Ap, void* Rx, const void* q, int last, int prec,
+                      cudaStream_t st);
+void launch_cg_p(const SliceDesc* d, const BlockMap& pix, int np, SliceScalars* sc, const double* part_rs,
+                 const int* rows_prefix, bool sums, const float2* s, float2* p, cudaStream_t st);
 void launch_image_update(const SliceDesc* d, const BlockMap& pix, int np, const SliceScalars* sc, double lam_c,
                          double lam_p, const float2* x, float4* y, float4* uy, float2* z, float2* uz, double* partial,
                          cudaStream_t st);

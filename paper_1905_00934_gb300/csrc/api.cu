@@ -688,7 +688,7 @@ static void enq_project(dect_admm* A, const float2* img, void* out, cudaStream_t
     const int B = A->B;
     pb(A, st);
     launch_textures(A->ds, A->tx.map(B), A->tx.total, A->ty.map(B), A->ty.total, img, A->txb, A->tyb, A->prec, st);
-    pe(A, DECT_PHASE_TEXTURE, 2, st);
+    pe(A, DECT_PHASE_TEXTURE, 1, st);
     pb(A, st);
     launch_project(A->ds, A->ptile.map(A->n_groups), A->ptile.total, A->d_groups, A->group_max(), A->txb, A->tyb, out, A->prec,
                    A->proj_views, st);
@@ -710,9 +710,22 @@ static void enq_precond(dect_admm* A, const float* H, const float2* r, float2* s
     }
 }
 
+// Whether the update kernels of a CG step form the step's scalars themselves: each of their blocks then adds up to 256
+// slots in float64, which six blocks per SM hide behind the two launches that it saves. Measured (13 CG steps within
+// a reconstruction): 64^2 x 90 x 96, 50 blocks 1157 -> 1065 us, four slices 1400 -> 1308, 16 slices (800 blocks) 2265
+// -> 2200; 128^2 x 180 x 256, 244 blocks 1499 -> 1421; 256^2 x 360 x 512, 976 blocks 2753 and 2759.
+static bool cg_small_batch(const dect_admm* A) {
+    if (A->pix.total + A->rays.total > 6 * 152) return false;
+    const std::vector<int>& rows = A->P.precondition ? A->prows.h : A->rows.h;
+    for (int b = 0; b < A->B; ++b)
+        if (A->pix.h[b + 1] - A->pix.h[b] > 256 || rows[b + 1] - rows[b] > 256) return false;
+    return true;
+}
+
 // Eq. 12: n PCG steps, warm-started from x, R x carried
 static void enq_pcg(dect_admm* A, int n, bool with_grad, const float* H, cudaStream_t st) {
     const int B = A->B;
+    const bool sums = cg_small_batch(A);
     BpEpilogue ep{};
     ep.x = A->x;
     ep.y = A->y;
@@ -734,9 +747,11 @@ static void enq_pcg(dect_admm* A, int n, bool with_grad, const float* H, cudaStr
     pe(A, DECT_PHASE_BP_FINALIZE, 1, st);
     if (A->counting) A->cRT += 2;
     enq_precond(A, H, A->r, A->p, st);
-    pb(A, st);
-    launch_rs_reduce(A->part_rs, A->rs_prefix(), A->sc, B, 1, st);
-    pe(A, DECT_PHASE_REDUCE, 1, st);
+    if (!sums) {
+        pb(A, st);
+        launch_rs_reduce(A->part_rs, A->rs_prefix(), A->sc, B, 1, st);
+        pe(A, DECT_PHASE_REDUCE, 1, st);
+    }
     for (int it = 0; it < n; ++it) {
         enq_project(A, A->p, A->q, st);
         pb(A, st);
@@ -748,21 +763,26 @@ static void enq_pcg(dect_admm* A, int n, bool with_grad, const float* H, cudaStr
                            A->bp_partial, A->n_img, A->Ap, ep, st);
         pe(A, DECT_PHASE_BP_FINALIZE, 1, st);
         if (A->counting) A->cRT += 2;
-        pb(A, st);
-        launch_alpha(A->part_pap, A->pix.d, A->sc, B, st);
-        pe(A, DECT_PHASE_REDUCE, 1, st);
+        if (!sums) {
+            pb(A, st);
+            launch_alpha(A->part_pap, A->pix.d, A->sc, B, st);
+            pe(A, DECT_PHASE_REDUCE, 1, st);
+        }
         const int last = it == n - 1;
         pb(A, st);
-        launch_cg_update(A->ds, A->pix.map(B), A->pix.total, A->rays.map(B), A->rays.total, A->sc, A->x, A->p, A->r,
-                         A->Ap, A->Rx, A->q, last, A->prec, st);
+        launch_cg_update(A->ds, A->pix.map(B), A->pix.total, A->rays.map(B), A->rays.total, A->sc,
+                         A->part_pap, A->part_rs, A->rs_prefix(), sums, A->x, A->p, A->r, A->Ap, A->Rx, A->q, last,
+                         A->prec, st);
         pe(A, DECT_PHASE_UPDATE, 1, st);
         if (!last) {
             enq_precond(A, H, A->r, A->s, st);
+            if (!sums) {
+                pb(A, st);
+                launch_rs_reduce(A->part_rs, A->rs_prefix(), A->sc, B, 0, st);
+                pe(A, DECT_PHASE_REDUCE, 1, st);
+            }
             pb(A, st);
-            launch_rs_reduce(A->part_rs, A->rs_prefix(), A->sc, B, 0, st);
-            pe(A, DECT_PHASE_REDUCE, 1, st);
-            pb(A, st);
-            launch_cg_p(A->ds, A->pix.map(B), A->pix.total, A->sc, A->s, A->p, st);
+            launch_cg_p(A->ds, A->pix.map(B), A->pix.total, A->sc, A->part_rs, A->rs_prefix(), sums, A->s, A->p, st);
             pe(A, DECT_PHASE_UPDATE, 1, st);
         }
     }
@@ -800,7 +820,7 @@ static void enq_lm_step(dect_admm* A, int b, cudaStream_t st) {
         const int last = k == n - 1;
         pb(A, st);
         launch_textures1(A->ds, A->tx.map(B), A->tx.total, A->ty.map(B), A->ty.total, A->lm_p, A->tx1, A->ty1, st);
-        pe(A, DECT_PHASE_TEXTURE, 2, st);
+        pe(A, DECT_PHASE_TEXTURE, 1, st);
         pb(A, st);
         launch_project1(A->ds, A->ptile.map(A->n_groups), A->ptile.total, A->d_groups, A->group_max(), A->tx1, A->ty1, A->lm_q,
                         A->proj_views, st);

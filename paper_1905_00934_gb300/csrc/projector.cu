@@ -119,14 +119,26 @@ __device__ __forceinline__ IM img_at(const IM* __restrict__ img, int nx, int ny,
     return __ldg(img + (size_t)j * nx + i);
 }
 
-// TX[i][jj] from a 32 (jj) x 32 (i) tile; rows jj-2 .. jj+29 staged in shared memory.
+// Both pair textures of a batch in one launch. The first nbx blocks: TX[i][jj] from a 32 (jj) x 32 (i) tile, rows
+// jj-2 .. jj+29 staged in shared memory; the others: TY[j][ii], one entry per thread. (One launch for both: a
+// reconstruction of one 64 x 64 slice, 14 projections, takes 1165 -> 1157 us.)
 template <class TX, class IM = float2>
-__global__ void __launch_bounds__(256) k_texture_x(const SliceDesc* __restrict__ dsl, BlockMap map,
-                                                   const IM* __restrict__ img, TX* __restrict__ tx) {
+__global__ void __launch_bounds__(256) k_textures(const SliceDesc* __restrict__ dsl, BlockMap mx, int nbx, BlockMap my,
+                                                  const IM* __restrict__ img, TX* __restrict__ tx,
+                                                  TX* __restrict__ ty) {
     __shared__ IM tile[33][33];
     int local;
-    const int s = slice_of(map, blockIdx.x, local);
-    const SliceDesc& d = dsl[s];
+    if ((int)blockIdx.x >= nbx) {
+        const SliceDesc& d = dsl[slice_of(my, blockIdx.x - nbx, local)];
+        const int nx = d.g.nx, ny = d.g.ny, ld = nx + 3;
+        const int64_t e = (int64_t)local * blockDim.x + threadIdx.x;
+        if (e >= (int64_t)ny * ld) return;
+        const int j = (int)(e / ld), ii = (int)(e % ld);
+        const IM* im = img + d.img_off;
+        sttex(ty + d.ty_off + e, img_at(im, nx, ny, j, ii - 2), img_at(im, nx, ny, j, ii - 1));
+        return;
+    }
+    const SliceDesc& d = dsl[slice_of(mx, blockIdx.x, local)];
     const int nx = d.g.nx, ny = d.g.ny;
     const int tiles_i = (nx + 31) / 32;
     const int jt = (local / tiles_i) * 32, it = (local % tiles_i) * 32;
@@ -146,21 +158,6 @@ __global__ void __launch_bounds__(256) k_texture_x(const SliceDesc* __restrict__
     }
 }
 
-// TY[j][ii], one entry per thread.
-template <class TX, class IM = float2>
-__global__ void __launch_bounds__(256) k_texture_y(const SliceDesc* __restrict__ dsl, BlockMap map,
-                                                   const IM* __restrict__ img, TX* __restrict__ ty) {
-    int local;
-    const int s = slice_of(map, blockIdx.x, local);
-    const SliceDesc& d = dsl[s];
-    const int nx = d.g.nx, ny = d.g.ny, ld = nx + 3;
-    const int64_t e = (int64_t)local * blockDim.x + threadIdx.x;
-    if (e >= (int64_t)ny * ld) return;
-    const int j = (int)(e / ld), ii = (int)(e % ld);
-    const IM* im = img + d.img_off;
-    sttex(ty + d.ty_off + e, img_at(im, nx, ny, j, ii - 2), img_at(im, nx, ny, j, ii - 1));
-}
-
 static int tx_blocks(int nx, int ny) { return ((nx + 31) / 32) * ((ny + 3 + 31) / 32); }
 static int ty_blocks(int nx, int ny) { return (int)(((int64_t)ny * (nx + 3) + 255) / 256); }
 
@@ -168,14 +165,11 @@ static int ty_blocks(int nx, int ny) { return (int)(((int64_t)ny * (nx + 3) + 25
 void launch_textures(const SliceDesc* dsl, const BlockMap& mx, int nbx, const BlockMap& my, int nby,
                      const float2* img, void* tx, void* ty, int prec, cudaStream_t st) {
     if (prec == PREC_F16) {
-        k_texture_x<TexH><<<nbx, 256, 0, st>>>(dsl, mx, img, (TexH*)tx);
-        k_texture_y<TexH><<<nby, 256, 0, st>>>(dsl, my, img, (TexH*)ty);
+        k_textures<TexH><<<nbx + nby, 256, 0, st>>>(dsl, mx, nbx, my, img, (TexH*)tx, (TexH*)ty);
     } else if (prec == PREC_BF16) {
-        k_texture_x<TexB><<<nbx, 256, 0, st>>>(dsl, mx, img, (TexB*)tx);
-        k_texture_y<TexB><<<nby, 256, 0, st>>>(dsl, my, img, (TexB*)ty);
+        k_textures<TexB><<<nbx + nby, 256, 0, st>>>(dsl, mx, nbx, my, img, (TexB*)tx, (TexB*)ty);
     } else {
-        k_texture_x<float4><<<nbx, 256, 0, st>>>(dsl, mx, img, (float4*)tx);
-        k_texture_y<float4><<<nby, 256, 0, st>>>(dsl, my, img, (float4*)ty);
+        k_textures<float4><<<nbx + nby, 256, 0, st>>>(dsl, mx, nbx, my, img, (float4*)tx, (float4*)ty);
     }
 }
 
@@ -183,8 +177,7 @@ void launch_textures(const SliceDesc* dsl, const BlockMap& mx, int nbx, const Bl
 // per-basis projections.
 void launch_textures1(const SliceDesc* dsl, const BlockMap& mx, int nbx, const BlockMap& my, int nby,
                       const float* img, float2* tx, float2* ty, cudaStream_t st) {
-    k_texture_x<float2, float><<<nbx, 256, 0, st>>>(dsl, mx, img, tx);
-    k_texture_y<float2, float><<<nby, 256, 0, st>>>(dsl, my, img, ty);
+    k_textures<float2, float><<<nbx + nby, 256, 0, st>>>(dsl, mx, nbx, my, img, tx, ty);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -464,7 +457,7 @@ __device__ __forceinline__ void planar_at(const float* __restrict__ img, int nx,
     o = (j < 0 || j >= ny || i < 0 || i >= nx) ? 0.f : __ldg(img + (size_t)j * nx + i);
 }
 
-// Both pair textures of one planar image in one launch (the first nbx blocks write TX as k_texture_x does, the
+// Both pair textures of one planar image in one launch (the first nbx blocks write TX as k_textures does, the
 // others TY); IM = float2 (two channels) with TX = float4, or float with float2
 template <class TX, class IM>
 __global__ void __launch_bounds__(256) k_textures_planar(SliceDesc d, int nbx, const float* __restrict__ img,

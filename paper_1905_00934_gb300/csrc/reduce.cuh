@@ -85,4 +85,38 @@ __device__ void slice_sum(const double* __restrict__ part, const int* __restrict
     __syncthreads();
 }
 
+// slice_sum's sums of at most 256 slots by a block of 256 threads, for two sets of slots at once (out[0 .. 1] of part0,
+// out[2 .. 3] of part1; valid in warp 0): the steps that would only add the zeros of absent slots are left out
+// (float64 is slow), so the sums have slice_sum's bits.
+__device__ __forceinline__ void slice_sum_pair_small(const double* __restrict__ part0, const int* __restrict__ prefix0,
+                                                     const double* __restrict__ part1,
+                                                     const int* __restrict__ prefix1, int s, double (&out)[4]) {
+    __shared__ double red[4][256];
+    const int t = threadIdx.x, b0 = prefix0[s], b1 = prefix1[s];
+    const int n0 = prefix0[s + 1] - b0, n1 = prefix1[s + 1] - b1, n = max(n0, n1);
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        out[q] = t < n0 ? part0[2 * (size_t)(b0 + t) + q] : 0.0;
+        out[2 + q] = t < n1 ? part1[2 * (size_t)(b1 + t) + q] : 0.0;
+    }
+    if (n > 32) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) red[q][t] = out[q];
+        __syncthreads();
+        for (int h = n > 128 ? 128 : (n > 64 ? 64 : 32); h >= 32; h >>= 1) {
+            if (t < h)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) red[q][t] += red[q][t + h];
+            __syncthreads();
+        }
+        if (t < 32)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) out[q] = red[q][t];
+    }
+    if (t < 32)
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            for (int h = 16; h > 0; h >>= 1) out[q] += __shfl_down_sync(0xffffffffu, out[q], h);
+}
+
 }  // namespace dect
