@@ -393,15 +393,63 @@ __device__ __forceinline__ double cost64(const Ray64& q, double fh, double fl, d
     return 0.5 * (q.wh * rh * rh + q.wl * rl * rl) + 0.5 * (q.rc * (ac - q.vc) * (ac - q.vc) + q.rp * (ap - q.vp) * (ap - q.vp));
 }
 
+// The decomposition's tables in shared memory: t = {S_h, S_l, f_KN, f_p}, w = {S_h f_KN, S_h f_p, S_l f_KN, S_l f_p}
+// (a product in the loop would be formed for every ray and bin); both: one past the last bin that both spectra reach,
+// beyond which only the high one (high) or the low one is summed
+struct Tables64 {
+    const double4_32a *t, *w;
+    int ne, both;
+    bool high;
+};
+
+// fwd64 with the products taken from the table and without the shorter spectrum's sums past its end, where they add
+// zeros: the same bits where the exponentials are finite; where one is not, neither is one of f_h, f_l, as in fwd64.
+__device__ __forceinline__ void lm_sums64(const Tables64& T, double ac, double ap, bool jac, double& fh, double& fl,
+                                          double (&J)[4]) {
+    double sh = 0.0, sl = 0.0, shc = 0.0, shp = 0.0, slc = 0.0, slp = 0.0;
+    auto bins = [&](int e0, int e1, bool high, bool low) {
+        for (int e = e0; e < e1; ++e) {
+            const double4_32a t4 = T.t[e];
+            const double t = exp(-t4.z * ac - t4.w * ap);
+            if (high) sh += t4.x * t;
+            if (low) sl += t4.y * t;
+            if (jac) {
+                const double4_32a w4 = T.w[e];
+                if (high) {
+                    shc += w4.x * t;
+                    shp += w4.y * t;
+                }
+                if (low) {
+                    slc += w4.z * t;
+                    slp += w4.w * t;
+                }
+            }
+        }
+    };
+    bins(0, T.both, true, true);
+    if (T.high)
+        bins(T.both, T.ne, true, false);
+    else
+        bins(T.both, T.ne, false, true);
+    fh = -log(sh);
+    fl = -log(sl);
+    if (jac) {
+        J[0] = shc / sh;
+        J[1] = shp / sh;
+        J[2] = slc / sl;
+        J[3] = slp / sl;
+    }
+}
+
 // `iters` LM iterations: Gauss-Newton system A = sum_k w_k J_k J_k^T + diag(rho), Marquardt damping
 // B = A with its diagonal times (1 + mu), step -B^-1 g, kept iff the cost decreases (mu / 10, else * 10),
 // mu clamped to [1e-10, 1e10]; status 0 accepted, 1 rejected, 2 non-finite or singular. f and J at a trial point
 // that is kept are the next iteration's, so an iteration makes one pass over the energies.
-__device__ void lm64(const double4_32a* __restrict__ T, int ne, const Ray64& q, int iters, double& a0, double& a1,
+__device__ void lm64(const Tables64& T, const Ray64& q, int iters, double& a0, double& a1,
                      double& m, uint8_t& st) {
     if (iters <= 0) return;
     double fh, fl, J[4];
-    fwd64(T, ne, a0, a1, fh, fl, J);
+    lm_sums64(T, a0, a1, true, fh, fl, J);
     for (int it = 0; it < iters; ++it) {
         const double rh = fh - q.mh, rl = fl - q.ml;
         const double g0 = q.wh * rh * J[0] + q.wl * rl * J[2] + q.rc * (a0 - q.vc);
@@ -420,7 +468,7 @@ __device__ void lm64(const double4_32a* __restrict__ T, int ne, const Ray64& q, 
         const double t1 = a1 + (-g1 * B00 + g0 * A01) / det;
         double fh1, fl1, J1[4];
         const bool last = it == iters - 1;
-        fwd64(T, ne, t0, t1, fh1, fl1, last ? nullptr : J1);
+        lm_sums64(T, t0, t1, !last, fh1, fl1, J1);
         const double cost1 = cost64(q, fh1, fl1, t0, t1);
         if (!isfinite(cost1)) {
             m *= 10.0;
@@ -454,6 +502,23 @@ __device__ __forceinline__ const double4_32a* load_tables64(const double4_32a* _
 // sums keep the ray map's blocks in a kernel of their own.
 constexpr int kRays64 = 32;
 
+// The tables by a warp's block (sh: 2 ne entries)
+__device__ __forceinline__ Tables64 load_lm_tables64(const double4_32a* __restrict__ t64, int ne, double4_32a* sh) {
+    static_assert(kRays64 == 32, "the supports are a warp's maxima");
+    int n_h = 0, n_l = 0;
+    for (int e = threadIdx.x; e < ne; e += kRays64) {
+        const double4_32a t = t64[e];
+        sh[e] = t;
+        sh[ne + e] = make_double4_32a(t.x * t.z, t.x * t.w, t.y * t.z, t.y * t.w);
+        if (t.x > 0.0) n_h = e + 1;
+        if (t.y > 0.0) n_l = e + 1;
+    }
+    n_h = __reduce_max_sync(0xffffffffu, n_h);
+    n_l = __reduce_max_sync(0xffffffffu, n_l);
+    __syncthreads();
+    return Tables64{sh, sh + ne, ne, min(n_h, n_l), n_h >= n_l};
+}
+
 // a-update (v = R x - u^a): the new a into an, mu and status in place
 __global__ void __launch_bounds__(kRays64) k64_udm_admm(const SliceDesc* __restrict__ dsl, BlockMap rays,
                                                         const double4_32a* __restrict__ t64, int ne,
@@ -463,7 +528,7 @@ __global__ void __launch_bounds__(kRays64) k64_udm_admm(const SliceDesc* __restr
                                                         uint8_t* __restrict__ status, const SliceScalars* __restrict__ sc,
                                                         int iters) {
     extern __shared__ double4_32a tab64[];
-    const double4_32a* T = load_tables64(t64, ne, tab64);
+    const Tables64 T = load_lm_tables64(t64, ne, tab64);
     int local;
     const int s = slice_of(rays, blockIdx.x / (256 / kRays64), local);
     const SliceDesc& d = dsl[s];
@@ -482,7 +547,7 @@ __global__ void __launch_bounds__(kRays64) k64_udm_admm(const SliceDesc* __restr
     q.rp = sc[s].rho[1];
     double a0 = a[ec], a1 = a[ep], m = mu[er];
     uint8_t st = DECT_RAY_ACCEPTED;
-    lm64(T, ne, q, iters, a0, a1, m, st);
+    lm64(T, q, iters, a0, a1, m, st);
     an[ec] = a0;
     an[ep] = a1;
     mu[er] = m;
@@ -521,7 +586,7 @@ __global__ void __launch_bounds__(kRays64) k64_udm_init(const SliceDesc* __restr
                                                         double* __restrict__ mu, double rho_p, int iters, double abar,
                                                         double mu0) {
     extern __shared__ double4_32a tab64[];
-    const double4_32a* T = load_tables64(t64, ne, tab64);
+    const Tables64 T = load_lm_tables64(t64, ne, tab64);
     int local;
     const SliceDesc& d = dsl[slice_of(rays, blockIdx.x / (256 / kRays64), local)];
     const int64_t nr = nr_of(d), k = (int64_t)local * 256 + (blockIdx.x % (256 / kRays64)) * kRays64 + threadIdx.x;
@@ -537,7 +602,7 @@ __global__ void __launch_bounds__(kRays64) k64_udm_init(const SliceDesc* __restr
     q.rp = rho_p;
     double a0 = (double)m4.y / abar, a1 = 0.0, m = mu0;
     uint8_t st = DECT_RAY_ACCEPTED;
-    lm64(T, ne, q, iters, a0, a1, m, st);
+    lm64(T, q, iters, a0, a1, m, st);
     a[2 * d.sino_off + k] = a0;
     a[2 * d.sino_off + nr + k] = 0.0;
     mu[d.sino_off + k] = mu0;
@@ -807,15 +872,15 @@ void launch64_udm_admm(const SliceDesc* d, const BlockMap& rays, int nr, const d
                        const float4* meas, const F64Vecs& v, uint8_t* status, const SliceScalars* sc, int iters,
                        double* partial, cudaStream_t st) {
     // (q, R p of the CG step just taken, is free until the next one: it holds the new a in between)
-    k64_udm_admm<<<nr * (256 / kRays64), kRays64, sizeof(double4_32a) * ne, st>>>(d, rays, t64, ne, meas, v.Rx, v.ua, v.a,
-                                                                                  v.q, v.mu, status, sc, iters);
+    k64_udm_admm<<<nr * (256 / kRays64), kRays64, 2 * sizeof(double4_32a) * ne, st>>>(
+        d, rays, t64, ne, meas, v.Rx, v.ua, v.a, v.q, v.mu, status, sc, iters);
     k64_a_update<<<nr, 256, 0, st>>>(d, rays, v.q, v.Rx, v.ua, v.a, partial);
 }
 void launch64_udm_init(const SliceDesc* d, const BlockMap& rays, int nr, const double4_32a* t64, int ne,
                        const float4* meas, const F64Vecs& v, double rho_p, int iters, double abar, double mu0,
                        cudaStream_t st) {
-    k64_udm_init<<<nr * (256 / kRays64), kRays64, sizeof(double4_32a) * ne, st>>>(d, rays, t64, ne, meas, v.a, v.mu, rho_p,
-                                                                                  iters, abar, mu0);
+    k64_udm_init<<<nr * (256 / kRays64), kRays64, 2 * sizeof(double4_32a) * ne, st>>>(
+        d, rays, t64, ne, meas, v.a, v.mu, rho_p, iters, abar, mu0);
 }
 void launch64_image_update(const SliceDesc* d, const BlockMap& pix, int np, const SliceScalars* sc, double lam_c,
                            double lam_p, const F64Vecs& v, double* partial, cudaStream_t st) {
