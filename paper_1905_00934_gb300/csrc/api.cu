@@ -1186,17 +1186,32 @@ static dect_status enq_initialize(dect_admm* A, cudaStream_t st) {
 // View groups per tile of a batch with `tiles` 32-pixel tiles over its slices (`paired` of them when slices of one
 // geometry are taken two at a time, 0 if none are) and `views` views per slice on average. Few tiles want many
 // groups to fill the chip, but a group of less than about 6 views pays more for its start than it computes;
-// medium batches of few views take as many groups as give 11 CTAs per SM (6 of paired slices); large ones fill it
-// with any count and take fewer partial images. Between 4 and 16 groups the backprojector's time differs by a few
-// percent (512^2 alone: 0.71 to 0.76 ms per iteration, 8 of them: 2.57 to 2.67).
+// medium batches of few views take as many groups as give 11 CTAs per SM; several slices of one geometry the count
+// that fills whole waves of CTAs best (6 per SM when paired, 11 otherwise), against a start of four views per
+// group and the partial images; large ones fill the chip with any count and take fewer partial images. Between 6 and
+// 16 groups the backprojector's time differs by a few percent (512^2 x 720 views, ms per iteration: one slice 0.71 to
+// 0.76; two 0.97 at 6, 0.89 at 10 and 12, 0.91 at 16; four 1.41 at 6, 1.37 at 8 to 12, 1.43 at 16; eight 2.57 to 2.67).
 static int default_view_groups(int tiles, int paired, int views) {
+    constexpr int kCounts[] = {4, 6, 8, 10, 12, 16};
     if (tiles < 100) return views >= 150 ? 16 : (paired && tiles >= 75) ? 10 : views >= 75 ? 12 : 10;
     if (paired && tiles < 160) return 10;
-    const int units = paired ? paired : tiles, slots = paired ? 6 * 152 : 11 * 152;
-    if (4 * units <= slots && views < 390) {
+    if (paired && tiles < 1500) {
+        const double waves = paired <= 0.62 * tiles ? paired / (6.0 * 152.0) : tiles / (11.0 * 152.0);
+        int best = 0;
+        double least = 0.0;
+        for (int c : kCounts) {
+            const double w = c * waves, t = std::ceil(w - 1e-9) / w * (1.0 + 4.0 * c / views) * (1.0 + 0.004 * c);
+            if (!best || t < 0.99 * least) {
+                best = c;
+                least = t;
+            }
+        }
+        return best;
+    }
+    if (4 * tiles <= 11 * 152 && views < 390) {
         int C = 4;
-        for (int c : {6, 8, 10, 12, 16})
-            if (units * c <= slots) C = c;
+        for (int c : kCounts)
+            if (tiles * c <= 11 * 152) C = c;
         return C;
     }
     if (tiles < 480) return 12;
