@@ -66,6 +66,8 @@ __device__ __forceinline__ void kahan_add(float& sum, float& comp, float v) {
 // the exponentials are the bare instruction's, hence finite: zero weights then add zeros (the tables in shared memory
 // end in zeros up to a multiple of 8 bins).
 __host__ __device__ constexpr int padded(int ne) { return (ne + 7) & ~7; }
+// the tables' size in float4: t1, t2, then {largest |k_kn|, largest |k_p|} of each block of 8 bins
+__host__ __device__ constexpr int table_len(int ne) { return 2 * padded(ne) + (padded(ne) + 31) / 32 * 2; }
 
 // 2^x. FAST: the bare instruction, for x above the range that underflows (in_fast_range), where it is what exp2f
 // returns; exp2f's scaling for the rest costs three more instructions per bin.
@@ -77,9 +79,19 @@ __device__ __forceinline__ float exp2_bin(float x) {
     return r;
 }
 
-// |k_kn a_c + k_p a_p| stays below 125 for every bin, so no exponential underflows (false for a NaN)
-__device__ __forceinline__ bool in_fast_range(const SpecDev& sp, float ac, float ap) {
-    return fmaf(sp.kc_max, fabsf(ac), sp.kp_max * fabsf(ap)) < 125.0f;
+// |k_kn a_c + k_p a_p| stays below 125 where |k_kn| <= kc, |k_p| <= kp, so that no exponential underflows (false for a
+// NaN)
+__device__ __forceinline__ bool in_fast_range(float kc, float kp, float ac, float ap) {
+    return fmaf(kc, fabsf(ac), kp * fabsf(ap)) < 125.0f;
+}
+
+// one choice per warp (the threads of a warp that reach it decide together)
+template <int R>
+__device__ __forceinline__ bool warp_fast(float kc, float kp, const float (&ac)[R], const float (&ap)[R]) {
+    bool f = true;
+#pragma unroll
+    for (int k = 0; k < R; ++k) f = f && in_fast_range(kc, kp, ac[k], ap[k]);
+    return __all_sync(__activemask(), f);
 }
 
 // one bin's terms: W = 3 both spectra, 1 the high one only, 2 the low one only
@@ -142,9 +154,85 @@ struct Sums {
     float sh[R], sl[R], shc[R], shp[R], slc[R], slp[R];
 };
 
+// one block of 8 energies
+template <int R, bool FAST>
+__device__ __forceinline__ void block_jac(const float4* __restrict__ t1, const float4* __restrict__ t2,
+                                          const SpecDev& sp, int e0, const float (&ac)[R], const float (&ap)[R],
+                                          float (&bh)[R], float (&bl)[R], Sums<R>& o) {
+    if (FAST ? e0 < sp.n_both : e0 + 8 <= sp.n_both) {
+        // both spectra: the sum pairs {b_h, b_l}, {s_hc, s_hp}, {s_lc, s_lp} advance as packed float32
+        // pairs, each sum taking bin_jac<3>'s terms in its order (the same bits, half the instructions)
+        f32x2 bhl[R], sh2[R], sl2[R];
+#pragma unroll
+        for (int k = 0; k < R; ++k) {
+            bhl[k] = pack2(0.f, 0.f);
+            sh2[k] = pack2(o.shc[k], o.shp[k]);
+            sl2[k] = pack2(o.slc[k], o.slp[k]);
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const float4 a = t1[e0 + u];
+            const float4 b = t2[e0 + u];
+#pragma unroll
+            for (int k = 0; k < R; ++k) {
+                const float t = exp2_bin<FAST>(-fmaf(a.x, ac[k], a.y * ap[k]));
+                const f32x2 tt = pack2(t, t);
+                bhl[k] = fma2(pack2(a.z, a.w), tt, bhl[k]);
+                sh2[k] = fma2(pack2(b.x, b.y), tt, sh2[k]);
+                sl2[k] = fma2(pack2(b.z, b.w), tt, sl2[k]);
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < R; ++k) {
+            const float2 x = unpack2(bhl[k]), y = unpack2(sh2[k]), z = unpack2(sl2[k]);
+            bh[k] = x.x;
+            bl[k] = x.y;
+            o.shc[k] = y.x;
+            o.shp[k] = y.y;
+            o.slc[k] = z.x;
+            o.slp[k] = z.y;
+        }
+    } else if (FAST ? e0 < sp.n_end : e0 >= sp.n_both && e0 + 8 <= sp.n_end) {
+        if (sp.tail_high) {
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const float4 a = t1[e0 + u], b = t2[e0 + u];
+#pragma unroll
+                for (int k = 0; k < R; ++k)
+                    bin_jac<1, FAST>(a, b, ac[k], ap[k], bh[k], bl[k], o.shc[k], o.shp[k], o.slc[k], o.slp[k]);
+            }
+        } else {
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const float4 a = t1[e0 + u], b = t2[e0 + u];
+#pragma unroll
+                for (int k = 0; k < R; ++k)
+                    bin_jac<2, FAST>(a, b, ac[k], ap[k], bh[k], bl[k], o.shc[k], o.shp[k], o.slc[k], o.slp[k]);
+            }
+        }
+    } else if (!FAST) {
+        const int e1 = min(e0 + 8, sp.n_end);
+        for (int e = e0; e < e1; ++e) {
+            const float4 a = t1[e], b = t2[e];
+#pragma unroll
+            for (int k = 0; k < R; ++k) {
+                if (e < sp.n_both)
+                    bin_jac<3, FAST>(a, b, ac[k], ap[k], bh[k], bl[k], o.shc[k], o.shp[k], o.slc[k], o.slp[k]);
+                else if (sp.tail_high)
+                    bin_jac<1, FAST>(a, b, ac[k], ap[k], bh[k], bl[k], o.shc[k], o.shp[k], o.slc[k], o.slp[k]);
+                else
+                    bin_jac<2, FAST>(a, b, ac[k], ap[k], bh[k], bl[k], o.shc[k], o.shp[k], o.slc[k], o.slp[k]);
+            }
+        }
+    }
+}
+
+// FAST: every block; otherwise each block by its own coefficients, which fall with the energy: a ray through metal
+// underflows in the lowest blocks only
 template <int R, bool FAST>
 __device__ __forceinline__ void sums_jac(const float4* __restrict__ t1, const float4* __restrict__ t2,
                                          const SpecDev& sp, const float (&ac)[R], const float (&ap)[R], Sums<R>& o) {
+    const float2* kb = reinterpret_cast<const float2*>(t1 + 2 * padded(sp.ne));
     float ch[R], cl[R];
 #pragma unroll
     for (int k = 0; k < R; ++k) ch[k] = cl[k] = o.sh[k] = o.sl[k] = o.shc[k] = o.shp[k] = o.slc[k] = o.slp[k] = 0.f;
@@ -152,72 +240,10 @@ __device__ __forceinline__ void sums_jac(const float4* __restrict__ t1, const fl
         float bh[R], bl[R];
 #pragma unroll
         for (int k = 0; k < R; ++k) bh[k] = bl[k] = 0.f;
-        if (FAST ? e0 < sp.n_both : e0 + 8 <= sp.n_both) {
-            // both spectra: the sum pairs {b_h, b_l}, {s_hc, s_hp}, {s_lc, s_lp} advance as packed float32
-            // pairs, each sum taking bin_jac<3>'s terms in its order (the same bits, half the instructions)
-            f32x2 bhl[R], sh2[R], sl2[R];
-#pragma unroll
-            for (int k = 0; k < R; ++k) {
-                bhl[k] = pack2(0.f, 0.f);
-                sh2[k] = pack2(o.shc[k], o.shp[k]);
-                sl2[k] = pack2(o.slc[k], o.slp[k]);
-            }
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const float4 a = t1[e0 + u];
-                const float4 b = t2[e0 + u];
-#pragma unroll
-                for (int k = 0; k < R; ++k) {
-                    const float t = exp2_bin<FAST>(-fmaf(a.x, ac[k], a.y * ap[k]));
-                    const f32x2 tt = pack2(t, t);
-                    bhl[k] = fma2(pack2(a.z, a.w), tt, bhl[k]);
-                    sh2[k] = fma2(pack2(b.x, b.y), tt, sh2[k]);
-                    sl2[k] = fma2(pack2(b.z, b.w), tt, sl2[k]);
-                }
-            }
-#pragma unroll
-            for (int k = 0; k < R; ++k) {
-                const float2 x = unpack2(bhl[k]), y = unpack2(sh2[k]), z = unpack2(sl2[k]);
-                bh[k] = x.x;
-                bl[k] = x.y;
-                o.shc[k] = y.x;
-                o.shp[k] = y.y;
-                o.slc[k] = z.x;
-                o.slp[k] = z.y;
-            }
-        } else if (FAST ? e0 < sp.n_end : e0 >= sp.n_both && e0 + 8 <= sp.n_end) {
-            if (sp.tail_high) {
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const float4 a = t1[e0 + u], b = t2[e0 + u];
-#pragma unroll
-                    for (int k = 0; k < R; ++k)
-                        bin_jac<1, FAST>(a, b, ac[k], ap[k], bh[k], bl[k], o.shc[k], o.shp[k], o.slc[k], o.slp[k]);
-                }
-            } else {
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const float4 a = t1[e0 + u], b = t2[e0 + u];
-#pragma unroll
-                    for (int k = 0; k < R; ++k)
-                        bin_jac<2, FAST>(a, b, ac[k], ap[k], bh[k], bl[k], o.shc[k], o.shp[k], o.slc[k], o.slp[k]);
-                }
-            }
-        } else if (!FAST) {
-            const int e1 = min(e0 + 8, sp.n_end);
-            for (int e = e0; e < e1; ++e) {
-                const float4 a = t1[e], b = t2[e];
-#pragma unroll
-                for (int k = 0; k < R; ++k) {
-                    if (e < sp.n_both)
-                        bin_jac<3, FAST>(a, b, ac[k], ap[k], bh[k], bl[k], o.shc[k], o.shp[k], o.slc[k], o.slp[k]);
-                    else if (sp.tail_high)
-                        bin_jac<1, FAST>(a, b, ac[k], ap[k], bh[k], bl[k], o.shc[k], o.shp[k], o.slc[k], o.slp[k]);
-                    else
-                        bin_jac<2, FAST>(a, b, ac[k], ap[k], bh[k], bl[k], o.shc[k], o.shp[k], o.slc[k], o.slp[k]);
-                }
-            }
-        }
+        if (FAST || warp_fast<R>(kb[e0 / 8].x, kb[e0 / 8].y, ac, ap))
+            block_jac<R, true>(t1, t2, sp, e0, ac, ap, bh, bl, o);
+        else
+            block_jac<R, false>(t1, t2, sp, e0, ac, ap, bh, bl, o);
 #pragma unroll
         for (int k = 0; k < R; ++k) {
             kahan_add(o.sh[k], ch[k], bh[k]);
@@ -227,8 +253,53 @@ __device__ __forceinline__ void sums_jac(const float4* __restrict__ t1, const fl
 }
 
 template <int R, int EXP>
+__device__ __forceinline__ void block_val(const float4* __restrict__ t1, const SpecDev& sp, int e0,
+                                          const float (&ac)[R], const float (&ap)[R], float (&bh)[R], float (&bl)[R]) {
+    if (EXP == EXP_FAST ? e0 < sp.n_both : e0 + 8 <= sp.n_both) {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const float4 a = t1[e0 + u];
+#pragma unroll
+            for (int k = 0; k < R; ++k) bin_val<3, EXP>(a, ac[k], ap[k], bh[k], bl[k]);
+        }
+    } else if (EXP == EXP_FAST ? e0 < sp.n_end : e0 >= sp.n_both && e0 + 8 <= sp.n_end) {
+        if (sp.tail_high) {
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const float4 a = t1[e0 + u];
+#pragma unroll
+                for (int k = 0; k < R; ++k) bin_val<1, EXP>(a, ac[k], ap[k], bh[k], bl[k]);
+            }
+        } else {
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const float4 a = t1[e0 + u];
+#pragma unroll
+                for (int k = 0; k < R; ++k) bin_val<2, EXP>(a, ac[k], ap[k], bh[k], bl[k]);
+            }
+        }
+    } else if (EXP != EXP_FAST) {
+        const int e1 = min(e0 + 8, sp.n_end);
+        for (int e = e0; e < e1; ++e) {
+            const float4 a = t1[e];
+#pragma unroll
+            for (int k = 0; k < R; ++k) {
+                if (e < sp.n_both)
+                    bin_val<3, EXP>(a, ac[k], ap[k], bh[k], bl[k]);
+                else if (sp.tail_high)
+                    bin_val<1, EXP>(a, ac[k], ap[k], bh[k], bl[k]);
+                else
+                    bin_val<2, EXP>(a, ac[k], ap[k], bh[k], bl[k]);
+            }
+        }
+    }
+}
+
+// EXP_FULL: each block by its own coefficients, as in sums_jac
+template <int R, int EXP>
 __device__ __forceinline__ void sums_val(const float4* __restrict__ t1, const SpecDev& sp, const float (&ac)[R],
                                          const float (&ap)[R], float (&sh)[R], float (&sl)[R]) {
+    const float2* kb = reinterpret_cast<const float2*>(t1 + 2 * padded(sp.ne));
     float ch[R], cl[R];
 #pragma unroll
     for (int k = 0; k < R; ++k) ch[k] = cl[k] = sh[k] = sl[k] = 0.f;
@@ -236,44 +307,10 @@ __device__ __forceinline__ void sums_val(const float4* __restrict__ t1, const Sp
         float bh[R], bl[R];
 #pragma unroll
         for (int k = 0; k < R; ++k) bh[k] = bl[k] = 0.f;
-        if (EXP == EXP_FAST ? e0 < sp.n_both : e0 + 8 <= sp.n_both) {
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const float4 a = t1[e0 + u];
-#pragma unroll
-                for (int k = 0; k < R; ++k) bin_val<3, EXP>(a, ac[k], ap[k], bh[k], bl[k]);
-            }
-        } else if (EXP == EXP_FAST ? e0 < sp.n_end : e0 >= sp.n_both && e0 + 8 <= sp.n_end) {
-            if (sp.tail_high) {
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const float4 a = t1[e0 + u];
-#pragma unroll
-                    for (int k = 0; k < R; ++k) bin_val<1, EXP>(a, ac[k], ap[k], bh[k], bl[k]);
-                }
-            } else {
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const float4 a = t1[e0 + u];
-#pragma unroll
-                    for (int k = 0; k < R; ++k) bin_val<2, EXP>(a, ac[k], ap[k], bh[k], bl[k]);
-                }
-            }
-        } else if (EXP != EXP_FAST) {
-            const int e1 = min(e0 + 8, sp.n_end);
-            for (int e = e0; e < e1; ++e) {
-                const float4 a = t1[e];
-#pragma unroll
-                for (int k = 0; k < R; ++k) {
-                    if (e < sp.n_both)
-                        bin_val<3, EXP>(a, ac[k], ap[k], bh[k], bl[k]);
-                    else if (sp.tail_high)
-                        bin_val<1, EXP>(a, ac[k], ap[k], bh[k], bl[k]);
-                    else
-                        bin_val<2, EXP>(a, ac[k], ap[k], bh[k], bl[k]);
-                }
-            }
-        }
+        if (EXP == EXP_FULL && warp_fast<R>(kb[e0 / 8].x, kb[e0 / 8].y, ac, ap))
+            block_val<R, EXP_FAST>(t1, sp, e0, ac, ap, bh, bl);
+        else
+            block_val<R, EXP>(t1, sp, e0, ac, ap, bh, bl);
 #pragma unroll
         for (int k = 0; k < R; ++k) {
             kahan_add(sh[k], ch[k], bh[k]);
@@ -282,21 +319,12 @@ __device__ __forceinline__ void sums_val(const float4* __restrict__ t1, const Sp
     }
 }
 
-// The same with the exponential chosen by the range of the warp's rays (one choice per warp; the threads of a
-// warp that reach it decide together).
-template <int R>
-__device__ __forceinline__ bool warp_fast(const SpecDev& sp, const float (&ac)[R], const float (&ap)[R]) {
-    bool f = true;
-#pragma unroll
-    for (int k = 0; k < R; ++k) f = f && in_fast_range(sp, ac[k], ap[k]);
-    return __all_sync(__activemask(), f);
-}
-
+// The same with the exponential chosen by the range of the warp's rays
 template <int R>
 __device__ __forceinline__ void spectral_sums_jac(const float4* __restrict__ t1, const float4* __restrict__ t2,
                                                   const SpecDev& sp, const float (&ac)[R], const float (&ap)[R],
                                                   Sums<R>& o) {
-    if (warp_fast<R>(sp, ac, ap))
+    if (warp_fast<R>(sp.kc_max, sp.kp_max, ac, ap))
         sums_jac<R, true>(t1, t2, sp, ac, ap, o);
     else
         sums_jac<R, false>(t1, t2, sp, ac, ap, o);
@@ -305,7 +333,7 @@ __device__ __forceinline__ void spectral_sums_jac(const float4* __restrict__ t1,
 template <int R>
 __device__ __forceinline__ void spectral_sums(const float4* __restrict__ t1, const SpecDev& sp, const float (&ac)[R],
                                               const float (&ap)[R], float (&sh)[R], float (&sl)[R]) {
-    if (warp_fast<R>(sp, ac, ap))
+    if (warp_fast<R>(sp.kc_max, sp.kp_max, ac, ap))
         sums_val<R, EXP_FAST>(t1, sp, ac, ap, sh, sl);
     else
         sums_val<R, EXP_FULL>(t1, sp, ac, ap, sh, sl);
@@ -541,6 +569,13 @@ __device__ __forceinline__ void load_tables(const SpecDev& sp, float4* t1, float
         t2[e] = in ? __ldg(sp.t2 + e) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
     __syncthreads();
+    float2* kb = reinterpret_cast<float2*>(t1 + 2 * padded(sp.ne));
+    for (int b = threadIdx.x; b < padded(sp.ne) / 8; b += blockDim.x) {
+        float2 m = make_float2(0.f, 0.f);
+        for (int u = 0; u < 8; ++u) m = make_float2(fmaxf(m.x, fabsf(t1[8 * b + u].x)), fmaxf(m.y, fabsf(t1[8 * b + u].y)));
+        kb[b] = m;
+    }
+    __syncthreads();
 }
 
 // CTAs per SM that two rays per thread leave room for: holds the registers at 102 (126 otherwise; four, five, six CTAs:
@@ -558,7 +593,7 @@ __global__ void __launch_bounds__(kRaysPerBlock / R, R == 2 ? kUdmCtas : 4)
     extern __shared__ float4 tabs[];
     float4* t1 = tabs;
     float4* t2 = tabs + padded(sp.ne);
-    double4_32a* w1 = reinterpret_cast<double4_32a*>(tabs + 2 * padded(sp.ne));
+    double4_32a* w1 = reinterpret_cast<double4_32a*>(tabs + table_len(sp.ne));
     double4_32a* w2 = w1 + sp.ne;
     if (F64)
         for (int e = threadIdx.x; e < sp.ne; e += blockDim.x) {
@@ -767,7 +802,7 @@ __global__ void __launch_bounds__(kRaysPerBlock) k_lm_trial(const SliceDesc* __r
     block_partials<1>(acc, partial);
 }
 
-static size_t tab_bytes(const SpecDev& sp) { return 2 * sizeof(float4) * (size_t)padded(sp.ne); }
+static size_t tab_bytes(const SpecDev& sp) { return sizeof(float4) * (size_t)table_len(sp.ne); }
 // ---- Eq. 4's data term, per ray -------------------------------------------------------------------
 
 // partial[blk] = sum over the block's rays of 1/2 (w_h r_h^2 + w_l r_l^2), r = f(q) - m at the
