@@ -140,16 +140,11 @@ def joseph_weight_count(g) -> int:
 # the workload both arms of the bench line name (the reference arm times a bounded sample of it)
 WORKLOAD = "fan 512x512, 720 views x 1024 bins, 40 objects, I0 2e5, UDM1-PCG1 x 100 + init"
 
-# Shared-memory wavefronts per slice of the backprojector sweep on the same workload (ncu
-# l1tex__data_pipe_lsu_wavefronts_mem_shared.sum), keyed by (tile side, slices per CTA); the count
-# follows the samples and staged rays, not the view-group count. The SM serves one wavefront per clock.
-SWEEP_SMEM_WAVEFRONTS = {(32, 2): 8.01e7}
-
-# DRAM bytes (read + write) per launch of the backprojector sweep at the bench workload (8 slices),
-# keyed by the launch shape they were captured with (slices, view groups, tile side, cluster form,
-# slices per CTA, reduced form); from the counter captures in profiles/k_bp_sweep_512x720x1024.txt.
-# Reported only when the run uses one of these shapes.
-SWEEP_TRAFFIC = {(8, 6, 32, 0, 2, 1): 56.4e6, (8, 8, 32, 0, 2, 1): 57.8e6, (8, 10, 32, 0, 2, 1): 58.3e6}
+# DRAM bytes (read + write) per launch of the backprojector at the bench workload (8 slices), keyed by the
+# launch shape they were captured with (slices, view groups, tile side, cluster form, slices per CTA,
+# reduced form); from the counter capture in profiles/k_bp_gather_512x720x1024.txt. Reported only when
+# the run uses one of these shapes.
+GATHER_TRAFFIC = {(8, 6, 32, 0, 4, 1): 57.7e6}
 
 
 # ------------------------------------------------------------------------------------------------
@@ -479,25 +474,16 @@ def run_dect(args):
     pr_ms, pr_tf, pr_gbs, pr_bytes = kernel_roof("project", 1)
     cfg.update({"project_tflops": pr_tf, "project_tflops_frac": pr_tf / fp32_peak, "project_hbm_gbs": pr_gbs,
                 "project_hbm_frac": pr_gbs / peak, "backproject_hbm_frac": bp_gbs / peak})
-    traffic = SWEEP_TRAFFIC.get((B, st0["bp_view_groups"], st0["bp_tile"], st0["bp_cluster"], st0["bp_slices"],
-                                 st0["bp_reduce"]))
+    traffic = GATHER_TRAFFIC.get((B, st0["bp_view_groups"], st0["bp_tile"], st0["bp_cluster"], st0["bp_slices"],
+                                  st0["bp_reduce"]))
     roof = {"kernel": "backproject" if top == "backproject" else top, "bound": "alu", "achieved": bp_tf,
             "peak": fp32_peak, "unit": "TFLOP/s", "frac": bp_tf / fp32_peak,
             "traffic": traffic, "traffic_source": "stored ncu capture of this kernel and launch shape "
-                                                  "(profiles/k_bp_sweep_512x720x1024.txt)" if traffic else None,
+                                                  "(profiles/k_bp_gather_512x720x1024.txt)" if traffic else None,
             "peak_kind": f"derived: {n_sm} SMs x 128 FP32 lanes x 2 flop x max SM clock",
             "avg_launch_ms": bp_ms, "algorithmic_flops_per_launch": B * 4 * nnz,
             "algorithmic_bytes_per_launch": bp_bytes, "hbm_achieved_gbs": bp_gbs, "hbm_peak_gbs": peak,
             "hbm_frac": bp_gbs / peak, "hbm_peak_kind": peak_kind}
-    wf = SWEEP_SMEM_WAVEFRONTS.get((st0["bp_tile"], st0["bp_slices"]))
-    if wf and top == "backproject":
-        # the sweep's actual limit: shared-memory wavefronts (accumulator read-modify-writes and staging)
-        clk = (clocks.get("sm_max_mhz") or 2070.0) * 1e6
-        achieved_wf = B * wf / (bp_ms / 1e3)
-        roof["onchip"] = {"resource": "shared-memory wavefronts", "per_launch": B * wf,
-                          "achieved_per_s": achieved_wf, "peak_per_s": n_sm * clk, "frac": achieved_wf / (n_sm * clk),
-                          "source": "per-slice count from a stored ncu capture "
-                                    "(profiles/k_bp_sweep_512x720x1024.txt); peak one per SM per clock"}
     # the HBM-bound phases (data read and written once per iteration; 8 slices exceed L2): the four
     # element-wise kernels of an iteration (b = a + u^a - R x: 32 B/ray; x, R x += alpha p, q: 24 B/pixel
     # + 24 B/ray; y, z, u^y, u^z of Eq. 9-11 with x: 104 B/pixel; the dual rescale moves nothing when
