@@ -1505,6 +1505,7 @@ extern "C" dect_status dect_admm_create(dect_geom* const* geoms, int32_t B, cons
             DECT_FAIL(DECT_EUNSUPPORTED, "dect_admm_create: the solver supports images up to 2048 x 2048");
     }
     cudaError_t fe = P->storage == DECT_STORE_F64 ? solver64_init_attributes() : fft_init_attributes();
+    if (fe == cudaSuccess && P->udm_f64) fe = udm_f64_init_attributes();
     if (fe != cudaSuccess) DECT_FAIL(DECT_ECUDA, std::string("dect_admm_create: ") + cudaGetErrorString(fe));
 
     dect_admm* A = new dect_admm();

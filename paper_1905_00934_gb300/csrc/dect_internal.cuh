@@ -198,6 +198,7 @@ constexpr int kRaysPerBlock = 256;
 constexpr int kPixPerBlock = 256;
 
 // udm.cu
+cudaError_t udm_f64_init_attributes();  // per device: the float64 decomposition's dynamic shared memory
 void launch_udm_admm(const SliceDesc* dsl, const BlockMap& map, int nblk, const SpecDev& sp, const float4* meas,
                      const void* Rx, void* ua, void* a, float* mu, uint8_t* status,
                      const SliceScalars* sc, int iters, double* partial, int prec, bool f64, cudaStream_t st);

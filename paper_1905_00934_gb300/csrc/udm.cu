@@ -944,13 +944,28 @@ void launch_forward_model(const SpecDev& sp, const double4_32a* t64, int64_t n, 
 // against one: 737280 rays 491 / 517 us, 184320 143 / 163, 46080 90 / 82, 8640 82 / 68)
 static int rays_per_thread(int64_t rays) { return rays >= (1 << 17) ? 2 : 1; }
 
+// the tables of the float64 arithmetic: the float32 ones and the float64 weights behind them
+static size_t tab64_bytes(int ne) { return sizeof(float4) * (size_t)table_len(ne) + 2 * sizeof(double4_32a) * (size_t)ne; }
+
+cudaError_t udm_f64_init_attributes() {
+    // more than the 48 KB that a kernel gets unasked from 497 energies on (1 KB of it is static)
+    const int bytes = (int)tab64_bytes(kMaxEnergies);
+    cudaError_t e = cudaSuccess;
+    for (cudaError_t r : {cudaFuncSetAttribute(k_udm_admm<float2, true, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes),
+                          cudaFuncSetAttribute(k_udm_admm<__half2, true, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes),
+                          cudaFuncSetAttribute(k_udm_admm<__nv_bfloat162, true, 1>,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize, bytes)})
+        if (e == cudaSuccess) e = r;
+    return e;
+}
+
 template <class S2>
 static void udm_admm_t(const SliceDesc* dsl, const BlockMap& map, int nblk, const SpecDev& sp, const float4* meas,
                        const S2* Rx, S2* ua, S2* a, float* mu, uint8_t* status, const SliceScalars* sc, int iters,
                        double* partial, bool f64, cudaStream_t st) {
     if (f64)
-        k_udm_admm<S2, true, 1><<<nblk, kRaysPerBlock, tab_bytes(sp) + 2 * sizeof(double4_32a) * (size_t)sp.ne, st>>>(
-            dsl, map, sp, meas, Rx, ua, a, mu, status, sc, iters, partial);
+        k_udm_admm<S2, true, 1><<<nblk, kRaysPerBlock, tab64_bytes(sp.ne), st>>>(dsl, map, sp, meas, Rx, ua, a, mu, status,
+                                                                                 sc, iters, partial);
     else if (rays_per_thread((int64_t)nblk * kRaysPerBlock) == 2)
         k_udm_admm<S2, false, 2><<<nblk, kRaysPerBlock / 2, tab_bytes(sp), st>>>(dsl, map, sp, meas, Rx, ua, a, mu, status,
                                                                                sc, iters, partial);
