@@ -85,13 +85,13 @@ __device__ __forceinline__ bool in_fast_range(float kc, float kp, float ac, floa
     return fmaf(kc, fabsf(ac), kp * fabsf(ap)) < 125.0f;
 }
 
-// one choice per warp (the threads of a warp that reach it decide together)
+// one choice per warp, taken by all its lanes together: a kernel that forms sums keeps every lane up to its stores
 template <int R>
 __device__ __forceinline__ bool warp_fast(float kc, float kp, const float (&ac)[R], const float (&ap)[R]) {
     bool f = true;
 #pragma unroll
     for (int k = 0; k < R; ++k) f = f && in_fast_range(kc, kp, ac[k], ap[k]);
-    return __all_sync(__activemask(), f);
+    return __all_sync(0xffffffffu, f);
 }
 
 // one bin's terms: W = 3 both spectra, 1 the high one only, 2 the low one only
@@ -383,7 +383,9 @@ __device__ __forceinline__ float diff_of_products(float a, float b, float c, flo
 //
 // The sums at a trial point are those of the next iteration's point if the step is kept, and a dropped step leaves
 // the sums at the old point valid, so each iteration takes one pass over the energies (with the Jacobian's sums,
-// which only the last one does without): the first iteration adds the pass at the starting point.
+// which only the last one does without): the first iteration adds the pass at the starting point. The lanes of a
+// warp choose the exponential together, so a lane whose rays are done stays until all are (its rays' sums, at the
+// origin, go nowhere).
 template <int R>
 __device__ void lm_rays(const float4* __restrict__ t1, const float4* __restrict__ t2, const SpecDev& sp,
                         const RayIn (&in)[R], int iters, LmState (&s)[R]) {
@@ -428,13 +430,13 @@ __device__ void lm_rays(const float4* __restrict__ t1, const float4* __restrict_
             const float aq0 = diff_of_products(j3, u0, j1, u1), aq1 = diff_of_products(j0, u1, j2, u0);
             const float n0 = fmaf(whl * dJ, ar0, aq0) + e1 * g0;
             const float n1 = fmaf(whl * dJ, ar1, aq1) + e0 * g1;
-            tc[k] = s[k].ac - n0 / det;
-            tp[k] = s[k].ap - n1 / det;
+            tc[k] = done[k] ? 0.f : s[k].ac - n0 / det;
+            tp[k] = done[k] ? 0.f : s[k].ap - n1 / det;
         }
         bool all_done = true;
 #pragma unroll
         for (int k = 0; k < R; ++k) all_done = all_done && done[k];
-        if (all_done) break;
+        if (__all_sync(0xffffffffu, all_done)) break;
         Sums<R> tr;  // at the trial point
         const bool last = it == iters - 1;
         if (last)
@@ -753,13 +755,13 @@ __global__ void __launch_bounds__(kRaysPerBlock) k_lm_rays(const SliceDesc* __re
     int local;
     const int s = slice_of(map, blockIdx.x, local);
     const SliceDesc& d = dsl[s];
-    const int64_t r = (int64_t)local * kRaysPerBlock + threadIdx.x;
-    if (r >= (int64_t)d.g.nv * d.g.nb) return;
-    const int64_t e = d.sino_off + r;
+    const int64_t r = (int64_t)local * kRaysPerBlock + threadIdx.x, n = (int64_t)d.g.nv * d.g.nb;
+    const int64_t e = d.sino_off + min(r, n - 1);  // (a lane past the last ray repeats it, unstored)
     const float4 m = __ldg(meas + e);
     const float2 a = __ldg(Rx + e);
     float sh, sl, shc, shp, slc, slp;
     spectral_sums_jac(t1, t2, sp, a.x, a.y, sh, sl, shc, shp, slc, slp);
+    if (r >= n) return;
     const float rh = neg_log_ratio(sh, expf(-m.x)), rl = neg_log_ratio(sl, expf(-m.y));
     const float jh = (b ? shp : shc) / sh, jl = (b ? slp : slc) / sl;
     ew[e] = m.z * rh * jh + m.w * rl * jl;
@@ -783,16 +785,16 @@ __global__ void __launch_bounds__(kRaysPerBlock) k_lm_trial(const SliceDesc* __r
     int local;
     const int s = slice_of(map, blockIdx.x, local);
     const SliceDesc& d = dsl[s];
-    const int64_t r = (int64_t)local * kRaysPerBlock + threadIdx.x;
+    const int64_t r = (int64_t)local * kRaysPerBlock + threadIdx.x, n = (int64_t)d.g.nv * d.g.nb;
+    const int64_t e = d.sino_off + min(r, n - 1);  // (a lane past the last ray repeats it, uncounted)
+    const float4 m = __ldg(meas + e);
+    float2 a = __ldg(Rx + e);
+    if (b) a.y += __ldg(Rd + e); else a.x += __ldg(Rd + e);
+    const float ac[1] = {a.x}, ap[1] = {a.y};
+    float shv[1], slv[1];
+    spectral_sums<1>(t1, sp, ac, ap, shv, slv);
     double acc[1] = {0.0};
-    if (r < (int64_t)d.g.nv * d.g.nb) {
-        const int64_t e = d.sino_off + r;
-        const float4 m = __ldg(meas + e);
-        float2 a = __ldg(Rx + e);
-        if (b) a.y += __ldg(Rd + e); else a.x += __ldg(Rd + e);
-        const float ac[1] = {a.x}, ap[1] = {a.y};
-        float shv[1], slv[1];
-        spectral_sums<1>(t1, sp, ac, ap, shv, slv);
+    if (r < n) {
         const float sh = shv[0], sl = slv[0];
         const float2 o = __ldg(s0 + e);
         const float r0h = neg_log_ratio(o.x, expf(-m.x)), r0l = neg_log_ratio(o.y, expf(-m.y));
@@ -860,17 +862,19 @@ __global__ void __launch_bounds__(kRaysPerBlock) k_forward_model_f32(SpecDev sp,
     float4* t2 = tabs + padded(sp.ne);
     load_tables(sp, t1, t2);
     const int64_t r = (int64_t)blockIdx.x * kRaysPerBlock + threadIdx.x;
-    if (r >= n) return;
-    const float a[1] = {__ldg(ac + r)}, p[1] = {__ldg(ap + r)};
+    const int64_t e = min(r, n - 1);  // (a lane past the last ray repeats it, unstored)
+    const float a[1] = {__ldg(ac + e)}, p[1] = {__ldg(ap + e)};
     if (!jac && !oc) {  // (half of the sums, the same bits)
         float sh[1], sl[1];
         spectral_sums<1>(t1, sp, a, p, sh, sl);
+        if (r >= n) return;
         if (fh) fh[r] = (float)(-log((double)sh[0]));
         if (fl) fl[r] = (float)(-log((double)sl[0]));
         return;
     }
     float sh, sl, shc, shp, slc, slp;
     spectral_sums_jac(t1, t2, sp, a[0], p[0], sh, sl, shc, shp, slc, slp);
+    if (r >= n) return;
     const double ish = 1.0 / (double)sh, isl = 1.0 / (double)sl;
     const double j0 = shc * ish, j1 = shp * ish, j2 = slc * isl, j3 = slp * isl;
     if (fh) fh[r] = (float)(-log((double)sh));
