@@ -121,14 +121,13 @@ SliceDesc geom_single_of(const dect_geom* g) { return g->single(); }
 
 struct dect_spectra {
     int ne = 0;
-    float4* t1 = nullptr;
-    float4* t2 = nullptr;
+    float4* tab = nullptr;  // see SpecDev
     double4_32a* t64 = nullptr;  // {S_h, S_l, f_KN, f_p}, unit-sum spectra
     double4_32a* w64 = nullptr;  // [2][ne]: {S_h, S_l, S_h f_KN, S_h f_p}, {S_l f_KN, S_l f_p, 0, 0}
     double abar_low = 1.0;  // sum_E S_l f_KN (unit-sum S_l)
     int n_both = 0, n_end = 0, tail_high = 1;  // supports of the spectra (see SpecDev)
     float kc_max = 0.f, kp_max = 0.f;
-    SpecDev dev() const { return SpecDev{ne, t1, t2, w64, w64 + ne, n_both, n_end, tail_high, kc_max, kp_max}; }
+    SpecDev dev() const { return SpecDev{ne, tab, w64, w64 + ne, n_both, n_end, tail_high, kc_max, kp_max}; }
 };
 
 extern "C" const char* dect_version(void) { return "dect 0.1 sm_103a"; }
@@ -292,7 +291,9 @@ extern "C" dect_status dect_spectra_create(int32_t ne, const double* S_h, const 
     }
     if (!(th > 0.0) || !(tl > 0.0)) DECT_FAIL(DECT_EINVAL, "dect_spectra_create: spectra must have positive sums");
     const double log2e = 1.4426950408889634;
-    std::vector<float4> t1(ne), t2(ne);
+    std::vector<float4> tab(table_len(ne), make_float4(0.f, 0.f, 0.f, 0.f));
+    float4 *t1 = tab.data(), *t2 = t1 + padded(ne);
+    float2* block_max = reinterpret_cast<float2*>(t2 + padded(ne));
     std::vector<double4_32a> t64(ne), w64(2 * (size_t)ne);
     double abar = 0.0;
     for (int e = 0; e < ne; ++e) {
@@ -307,9 +308,12 @@ extern "C" dect_status dect_spectra_create(int32_t ne, const double* S_h, const 
     dect_spectra* s = new dect_spectra();
     s->ne = ne;
     s->abar_low = abar;
-    for (const float4& t : t1) {
-        s->kc_max = std::max(s->kc_max, std::fabs(t.x));
-        s->kp_max = std::max(s->kp_max, std::fabs(t.y));
+    for (int e = 0; e < ne; ++e) {
+        float2& m = block_max[e / 8];
+        m.x = std::max(m.x, std::fabs(t1[e].x));
+        m.y = std::max(m.y, std::fabs(t1[e].y));
+        s->kc_max = std::max(s->kc_max, m.x);
+        s->kp_max = std::max(s->kp_max, m.y);
     }
     int last_h = 0, last_l = 0;  // one past the last non-zero bin of each spectrum
     for (int e = 0; e < ne; ++e) {
@@ -319,10 +323,8 @@ extern "C" dect_status dect_spectra_create(int32_t ne, const double* S_h, const 
     s->n_both = std::min(last_h, last_l);
     s->n_end = std::max(last_h, last_l);
     s->tail_high = last_h >= last_l ? 1 : 0;
-    cudaError_t e = dalloc(&s->t1, ne);
-    if (e == cudaSuccess) e = dalloc(&s->t2, ne);
-    if (e == cudaSuccess) e = cudaMemcpy(s->t1, t1.data(), sizeof(float4) * ne, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(s->t2, t2.data(), sizeof(float4) * ne, cudaMemcpyHostToDevice);
+    cudaError_t e = dalloc(&s->tab, tab.size());
+    if (e == cudaSuccess) e = cudaMemcpy(s->tab, tab.data(), sizeof(float4) * tab.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = dalloc(&s->t64, ne);
     if (e == cudaSuccess) e = cudaMemcpy(s->t64, t64.data(), sizeof(double4_32a) * ne, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = dalloc(&s->w64, 2 * (size_t)ne);
@@ -338,8 +340,7 @@ extern "C" dect_status dect_spectra_create(int32_t ne, const double* S_h, const 
 
 extern "C" void dect_spectra_destroy(dect_spectra* s) {
     if (!s) return;
-    cudaFree(s->t1);
-    cudaFree(s->t2);
+    cudaFree(s->tab);
     cudaFree(s->t64);
     cudaFree(s->w64);
     delete s;

@@ -108,14 +108,17 @@ struct LmScalars {
 // n_both, n_end, tail_high: the supports of the spectra (bins past a spectrum's last non-zero entry
 // contribute exact zeros to its sums): both may be non-zero below n_both, only the high spectrum
 // (tail_high) or only the low one in [n_both, n_end), neither from n_end on.
+// tab = T1, then T2, each ending in zeros up to a multiple of 8 bins, then {largest |k_kn|, largest |k_p|} of each block
+// of 8 bins.
+__host__ __device__ constexpr int padded(int ne) { return (ne + 7) & ~7; }
+__host__ __device__ constexpr int table_len(int ne) { return 2 * padded(ne) + (padded(ne) + 31) / 32 * 2; }  // in float4
 struct SpecDev {
     int ne;
-    const float4* t1;
-    const float4* t2;
+    const float4* tab;
     const double4_32a* w1;
     const double4_32a* w2;
     int n_both, n_end, tail_high;
-    float kc_max, kp_max;  // largest |k_kn| and |k_p| of t1
+    float kc_max, kp_max;  // largest |k_kn| and |k_p| of all bins
 };
 
 // Epilogue modes of the backprojector.

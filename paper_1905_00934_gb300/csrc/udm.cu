@@ -63,11 +63,8 @@ __device__ __forceinline__ void kahan_add(float& sum, float& comp, float v) {
 // terms are exact zeros, so skipping them leaves every sum bit for bit as it was; the compensated
 // additions still run once per block of 8 bins over all ne bins, so the blocking is unchanged too.
 // Blocks that lie wholly in one range run an unrolled body without per-bin tests. So does every other block where
-// the exponentials are the bare instruction's, hence finite: zero weights then add zeros (the tables in shared memory
-// end in zeros up to a multiple of 8 bins).
-__host__ __device__ constexpr int padded(int ne) { return (ne + 7) & ~7; }
-// the tables' size in float4: t1, t2, then {largest |k_kn|, largest |k_p|} of each block of 8 bins
-__host__ __device__ constexpr int table_len(int ne) { return 2 * padded(ne) + (padded(ne) + 31) / 32 * 2; }
+// the exponentials are the bare instruction's, hence finite: zero weights then add zeros (the tables end in zeros up to
+// a multiple of 8 bins, table_len).
 
 // 2^x. FAST: the bare instruction, for x above the range that underflows (in_fast_range), where it is what exp2f
 // returns; exp2f's scaling for the rest costs three more instructions per bin.
@@ -564,19 +561,10 @@ __device__ void lm_ray64(const float4* __restrict__ t1, const double4_32a* __res
     s.mu = (float)m;
 }
 
-__device__ __forceinline__ void load_tables(const SpecDev& sp, float4* t1, float4* t2) {
-    for (int e = threadIdx.x; e < padded(sp.ne); e += blockDim.x) {
-        const bool in = e < sp.ne;
-        t1[e] = in ? __ldg(sp.t1 + e) : make_float4(0.f, 0.f, 0.f, 0.f);
-        t2[e] = in ? __ldg(sp.t2 + e) : make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-    __syncthreads();
-    float2* kb = reinterpret_cast<float2*>(t1 + 2 * padded(sp.ne));
-    for (int b = threadIdx.x; b < padded(sp.ne) / 8; b += blockDim.x) {
-        float2 m = make_float2(0.f, 0.f);
-        for (int u = 0; u < 8; ++u) m = make_float2(fmaxf(m.x, fabsf(t1[8 * b + u].x)), fmaxf(m.y, fabsf(t1[8 * b + u].y)));
-        kb[b] = m;
-    }
+// (as it lies in global memory: when every CTA formed the blocks' maxima itself, eight shared loads of one bank per lane,
+// the vjp of 130000 rays of 121 bins took 17.4 us instead of 16.5, of 33 rays 6.8 instead of 5.4)
+__device__ __forceinline__ void load_tables(const SpecDev& sp, float4* tabs) {
+    for (int e = threadIdx.x; e < table_len(sp.ne); e += blockDim.x) tabs[e] = __ldg(sp.tab + e);
     __syncthreads();
 }
 
@@ -602,7 +590,7 @@ __global__ void __launch_bounds__(kRaysPerBlock / R, R == 2 ? kUdmCtas : 4)
             w1[e] = sp.w1[e];
             w2[e] = sp.w2[e];
         }
-    load_tables(sp, t1, t2);
+    load_tables(sp, tabs);
     int local;
     const int s = slice_of(map, blockIdx.x, local);
     const SliceDesc& d = dsl[s];
@@ -667,7 +655,7 @@ __global__ void __launch_bounds__(kRaysPerBlock / R, R == 2 ? kUdmCtas : 4)
     extern __shared__ float4 tabs[];
     float4* t1 = tabs;
     float4* t2 = tabs + padded(sp.ne);
-    load_tables(sp, t1, t2);
+    load_tables(sp, tabs);
     int local;
     const int s = slice_of(map, blockIdx.x, local);
     const SliceDesc& d = dsl[s];
@@ -707,7 +695,7 @@ __global__ void __launch_bounds__(kRaysPerBlock / R, R == 2 ? kUdmCtas : 4)
     extern __shared__ float4 tabs[];
     float4* t1 = tabs;
     float4* t2 = tabs + padded(sp.ne);
-    load_tables(sp, t1, t2);
+    load_tables(sp, tabs);
     const int64_t r0 = (int64_t)blockIdx.x * kRaysPerBlock + threadIdx.x;
     RayIn in[R];
     LmState st[R];
@@ -751,7 +739,7 @@ __global__ void __launch_bounds__(kRaysPerBlock) k_lm_rays(const SliceDesc* __re
     extern __shared__ float4 tabs[];
     float4* t1 = tabs;
     float4* t2 = tabs + padded(sp.ne);
-    load_tables(sp, t1, t2);
+    load_tables(sp, tabs);
     int local;
     const int s = slice_of(map, blockIdx.x, local);
     const SliceDesc& d = dsl[s];
@@ -781,7 +769,7 @@ __global__ void __launch_bounds__(kRaysPerBlock) k_lm_trial(const SliceDesc* __r
     extern __shared__ float4 tabs[];
     float4* t1 = tabs;
     float4* t2 = tabs + padded(sp.ne);
-    load_tables(sp, t1, t2);
+    load_tables(sp, tabs);
     int local;
     const int s = slice_of(map, blockIdx.x, local);
     const SliceDesc& d = dsl[s];
@@ -817,7 +805,7 @@ __global__ void __launch_bounds__(kRaysPerBlock) k_objective_rays(const SliceDes
     extern __shared__ float4 tabs[];
     float4* t1 = tabs;
     float4* t2 = tabs + padded(sp.ne);
-    load_tables(sp, t1, t2);
+    load_tables(sp, tabs);
     int local;
     const SliceDesc& d = dsl[slice_of(map, blockIdx.x, local)];
     const int64_t r = (int64_t)local * kRaysPerBlock + threadIdx.x;
@@ -860,7 +848,7 @@ __global__ void __launch_bounds__(kRaysPerBlock) k_forward_model_f32(SpecDev sp,
     extern __shared__ float4 tabs[];
     float4* t1 = tabs;
     float4* t2 = tabs + padded(sp.ne);
-    load_tables(sp, t1, t2);
+    load_tables(sp, tabs);
     const int64_t r = (int64_t)blockIdx.x * kRaysPerBlock + threadIdx.x;
     const int64_t e = min(r, n - 1);  // (a lane past the last ray repeats it, unstored)
     const float a[1] = {__ldg(ac + e)}, p[1] = {__ldg(ap + e)};
