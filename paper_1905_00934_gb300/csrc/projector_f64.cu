@@ -139,6 +139,7 @@ __global__ void __launch_bounds__(32 * kPixGroups) k_backproject_f64(GeomDev g, 
     if (i < g.nx) {
         // a ray with a weight here passes within one pixel of the centre along its across direction
         const float xc = ((float)i - g.cx) * g.pix, yc = ((float)j - g.cy) * g.pix;
+        const double di = (double)i, dj = (double)j, di1 = (double)(i - 1), dj1 = (double)(j - 1);
         for (int v = grp; v < g.nv; v += kPixGroups) {
             const float4 V = __ldg(g.views + v);
             const CandRange cr = rect_candidates(g, V.x, V.y, xc, yc, g.pix, g.pix);
@@ -153,9 +154,13 @@ __global__ void __launch_bounds__(32 * kPixGroups) k_backproject_f64(GeomDev g, 
                 const double4_32a P = rays[r];
                 // the ray's own axis bit: near 45 degrees the two tables may differ
                 const bool ax64 = P.w != 0.0;
-                const double q = __fma_rn((double)(ax64 ? j : i), P.y, P.x);
-                const double wgt = 1.0 - fabs(q - (double)(ax64 ? i : j));
-                if (!(wgt > 0.0)) continue;
+                const double q = __fma_rn(ax64 ? dj : di, P.y, P.x), at = ax64 ? di : dj;
+                // R's weights from the same exact differences: 1 - (q - floor q) or q - floor q
+                // (float64 comparisons take the float64 pipe: the signs are read as integers)
+                const double dist = q - at;
+                const bool below = __double_as_longlong(dist) < 0;
+                const double wgt = (below ? q : 1.0) - (below ? (ax64 ? di1 : dj1) : dist);
+                if (__double_as_longlong(wgt) <= 0) continue;
 #pragma unroll
                 for (int c = 0; c < NCH; ++c) acc[c] += P.z * wgt * __ldg(sino + c * n + r);
             }
