@@ -12,8 +12,9 @@
 //
 // What bounds them: the float64 pipe (two lanes per clock and SM) and latency at small sizes. R^T first tests a
 // candidate ray by its fixed-point position, so float64 work is done only for rays that weigh something; a
-// pixel's candidates are the bins of the square of one pixel around its centre. Measured on GB300: 64^2 x 90 x 96,
-// both bases: R 67 -> 26 us, R^T 300 -> 38; 128^2 x 180 x 256: R 207 -> 141, R^T 862 -> 273.
+// pixel's candidates are the bins of the square of one pixel around its centre. Measured on GB300, fan, both bases, against
+// a thread per ray and per pixel: 64^2 x 89 x 128: R 71 -> 21 us, R^T 333 -> 37; 128^2 x 179 x 256: R 203 -> 119 (one
+// channel 104 -> 97), R^T 678 -> 193; 256^2 x 358 x 512: R 1694 -> 547, R^T 3309 -> 1237.
 #include <cuda_runtime.h>
 #include <math.h>
 
@@ -86,14 +87,17 @@ __global__ void __launch_bounds__(kRayThreads) k_project_f64(GeomDev g, const do
         w = P.z;
         const bool ax = P.w != 0.0;
         const int n_along = ax ? g.ny : g.nx, n_across = ax ? g.nx : g.ny;
-        // indices whose positions lie in (-1, n_across): the only ones with a non-zero weight
+        // the indices whose positions lie in (-1, n_across) are the only ones with a non-zero weight. Bounded in float32,
+        // 1/16 pixel and one index wide of them (float32's error here is below 2e-3 pixel); two float64 divisions in
+        // each of a ray's lanes took longer than what they left out
+        const float q0 = (float)P.x, slope = (float)P.y;
         int lo = 0, hi = n_along - 1;
-        if (P.y != 0.0) {
-            const double t0 = (-1.0 - P.x) / P.y, t1 = ((double)n_across - P.x) / P.y;
+        if (slope != 0.f) {
+            const float t0 = (-1.0625f - q0) / slope, t1 = ((float)n_across + 0.0625f - q0) / slope;
             // (both bounded before the conversion: a nearly axis-parallel ray far outside has ends at +-1e17)
-            lo = max(lo, (int)floor(fmin(fmax(fmin(t0, t1), -1.0), (double)n_along)));
-            hi = min(hi, (int)ceil(fmax(fmin(fmax(t0, t1), (double)n_along), -1.0)));
-        } else if (!(P.x > -1.0 && P.x < n_across)) {
+            lo = max(lo, (int)floorf(fminf(fmaxf(fminf(t0, t1), -1.f), (float)n_along)));
+            hi = min(hi, (int)ceilf(fmaxf(fminf(fmaxf(t0, t1), (float)n_along), -1.f)));
+        } else if (!(q0 > -1.0625f && q0 < (float)n_across + 0.0625f)) {
             hi = -1;
         }
         const size_t plane = (size_t)g.nx * g.ny;
@@ -109,7 +113,7 @@ __global__ void __launch_bounds__(kRayThreads) k_project_f64(GeomDev g, const do
             for (int c = 0; c < NCH; ++c) {
                 const double a = in0 ? __ldg(im + c * plane) : 0.0;
                 const double b = in1 ? __ldg(im + c * plane + s_across) : 0.0;
-                acc[c] += (1.0 - f) * a + f * b;
+                acc[c] = __fma_rn(f, b, __fma_rn(1.0 - f, a, acc[c]));
             }
         }
     }
