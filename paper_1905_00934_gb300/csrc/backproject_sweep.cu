@@ -20,6 +20,9 @@
 // shared memory (each sample a read-modify-write of two rows) and was bound by shared-memory wavefronts; measured
 // on GB300, 512 x 512 x 720 x 1024, both bases, per application: one slice 439 -> 359 us, 8 slices of one
 // geometry 2509 -> 1286 us; 93 x 70 x 61 x 131: 97 -> 8 us (the old kernel's two warps per tile left the chip empty).
+// Detectors coarser than three pixels per bin are the one place where the predecessor was faster (its work went by the
+// rays, this one's by pixels and views): 512^2 x 720 views, bins of 3 / 4 / 16 pixels 193 / 172 / 124 -> 198 / 185 / 162
+// us. No workload here has them.
 #include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -63,9 +66,10 @@ struct GatherShape {
     static constexpr int kCh = NCH * SG;                 // channels per staged ray
     static constexpr int kVec = kCh < 4 ? kCh : 4;       // channels per staged vector
     // rays per trip of the gather loop and CTAs per SM the register allocation must allow, measured together (one
-    // slice: 362 us at 3 and 5, 392 at 2 and 6, 428 at 1 and 8; two: 3.16 ms per iteration of 8 slices at 1 and 5,
-    // 3.39 at 2 and 4; four: 2.62 at 2 and 3, 2.69 at 4 and 3, 2.88 at 1 and 4)
-    static constexpr int kUnroll = SG == 1 ? 3 : (SG == 2 ? 1 : 2);
+    // slice of 512^2 x 720 views, bins of 0.9 pixels: 303 us at 2 and 5, 313 at 3 and 5; one channel of it 296, 309, 308
+    // at 3 and 6, 295 at 1 and 5. Several slices, before rays were fetched by windows: two, 3.16 ms per iteration of 8
+    // slices at 1 and 5, 3.39 at 2 and 4; four, 2.62 at 2 and 3, 2.69 at 4 and 3, 2.88 at 1 and 4)
+    static constexpr int kUnroll = SG == 2 ? 1 : 2;
     static constexpr int kMinCtas = TILE == 64 ? 1 : (SG == 4 ? 3 : 5);
     // stages of {w s} and of {position, slope} per band, their segment lists, the accumulator tiles
     static constexpr size_t kStageW = kStages * (size_t)kCap * kCh * sizeof(float);
@@ -272,13 +276,19 @@ __global__ void __launch_bounds__(GatherShape<TILE, NCH, SG>::kThreads, GatherSh
         int batch = 0;  // batches published so far (both axes)
         int fill = 0, nseg = 0;
         float check = 0.f;  // becomes NaN with the first non-finite product
-        // the rays being fetched: kRays per lane, at stage indices p_at + lane + 32 i below p_at + p_n (the staging
-        // warps take the segments of a batch in turn)
-        constexpr int kRays = 2;
+        // Rays are fetched kRays per lane, kWin consecutive stage indices at a time whatever segments these belong to
+        // (the staging warps take such windows in turn): with the few rays per view of a coarse detector the loads of
+        // many views are then in flight together, and those of a fine one fill every lane. 512^2 x 720 views, both
+        // bases, one call, a segment at a time against windows (with the gather loop's 2 rays per trip): bins of 16
+        // pixels 220 -> 162 us, of 4 pixels 235 -> 185, of 0.9 pixels 316 -> 303.
+        constexpr int kRays = 2, kWin = 32 * kRays;
+        // the window [base, base + kWin): its rays (e), as far as the segments so far reach; bit i of mix: of a mixed view
+        unsigned e[kRays] = {};
+        int base = 0, mix = 0;
+        // the window in flight: stage indices p_at + lane + 32 i below p_at + p_n
         int4 P[kRays];
         float x[kRays][CH];
-        int p_at = 0, p_n = 0, axis = 0;
-        bool p_mixed = false;
+        int p_at = 0, p_n = 0, p_mix = 0, axis = 0;
         auto flush = [&]() {  // stages them
             const int t0 = axis ? tj : ti;
             const long long a0q = (long long)(axis ? ti : tj) << 30;
@@ -300,7 +310,7 @@ __global__ void __launch_bounds__(GatherShape<TILE, NCH, SG>::kThreads, GatherSh
                     const long long q = ray_pos(P[i], t0 + 32 * b) - a0q;
                     p[b] = make_int4((int)(unsigned)(unsigned long long)q, (int)(q >> 32), P[i].z, 0);
                 }
-                if (p_mixed && ray_axis(P[i]) != (axis != 0)) {  // the other axis' ray: a null one, far off
+                if ((p_mix >> i & 1) && ray_axis(P[i]) != (axis != 0)) {  // the other axis' ray: a null one, far off
 #pragma unroll
                     for (int q = 0; q < CH; ++q) x[i][q] = 0.f;
 #pragma unroll
@@ -318,8 +328,35 @@ __global__ void __launch_bounds__(GatherShape<TILE, NCH, SG>::kThreads, GatherSh
             }
             p_n = 0;
         };
+        auto fetch = [&](int n) {  // the first n rays of the window; they are in flight until the next one's turn
+            if (Sh::kProd == 32 || base / kWin % (Sh::kProd / 32) == ptid / 32) {
+                flush();
+#pragma unroll
+                for (int i = 0; i < kRays; ++i) {
+                    if (lane + 32 * i >= n) break;
+                    P[i] = __ldg(g.rays + e[i]);
+                    if constexpr (NCH == 2) {
+#pragma unroll
+                        for (int q = 0; q < SG; ++q) {
+                            const float2 sv = q < count ? load_pair(sn[q], e[i], n_rays) : make_float2(0.f, 0.f);
+                            x[i][2 * q] = sv.x;
+                            x[i][2 * q + 1] = sv.y;
+                        }
+                    } else {
+                        x[i][0] = __ldg(sn[0] + e[i]);
+                        if (rw) x[i][0] *= __ldg(rw + d.sino_off + e[i]);
+                    }
+                }
+                p_at = base;
+                p_n = n;
+                p_mix = mix;
+            }
+            base += kWin;
+        };
         auto publish = [&](int flags) {
+            if (fill > base) fetch(fill - base);
             flush();
+            base = 0;
             const int s = batch % kStages;
             const bool bad = __any_sync(0xffffffffu, check != 0.f);
             if (lane == 0 && bad) flags |= 2;
@@ -392,29 +429,17 @@ __global__ void __launch_bounds__(GatherShape<TILE, NCH, SG>::kThreads, GatherSh
                             // a segment that does not fit goes to the next batch, whole if it can
                             if (nseg == kBatchSegs || (fill > 0 && left > CAP - fill)) publish(0);
                             const int take = min(left, CAP - fill), s = batch % kStages;
-                            const bool my_turn = Sh::kProd == 32 || nseg % (Sh::kProd / 32) == ptid / 32;
-                            for (int r0 = 0; my_turn && r0 < take; r0 += kRays * 32) {
-                                // (the loads of these rays are in flight until the next ones' turn)
-                                flush();
+                            for (;;) {  // its rays into the window, which is fetched when full
 #pragma unroll
                                 for (int i = 0; i < kRays; ++i) {
-                                    const unsigned e = row + (unsigned)(k0 + min(r0 + lane + 32 * i, take - 1));
-                                    P[i] = __ldg(g.rays + e);
-                                    if constexpr (NCH == 2) {
-#pragma unroll
-                                        for (int q = 0; q < SG; ++q) {
-                                            const float2 sv = q < count ? load_pair(sn[q], e, n_rays) : make_float2(0.f, 0.f);
-                                            x[i][2 * q] = sv.x;
-                                            x[i][2 * q + 1] = sv.y;
-                                        }
-                                    } else {
-                                        x[i][0] = __ldg(sn[0] + e);
-                                        if (rw) x[i][0] *= __ldg(rw + d.sino_off + e);
+                                    const int j = base + lane + 32 * i - fill;
+                                    if ((unsigned)j < (unsigned)take) {
+                                        e[i] = row + (unsigned)(k0 + j);
+                                        mix = mixed ? mix | 1 << i : mix & ~(1 << i);
                                     }
                                 }
-                                p_at = fill + r0;
-                                p_n = take - r0;
-                                p_mixed = mixed;
+                                if (fill + take < base + kWin) break;
+                                fetch(kWin);
                             }
                             const int n = min(vwin, take);
                             if (ptid == 0)
