@@ -900,7 +900,7 @@ def main():
                     help="backprojector view groups per tile (0: autotuned, -1: occupancy rule)")
     ap.add_argument("--bp-tile", type=int, default=0, help="backprojector tile side, 32 or 64 (0: autotuned)")
     ap.add_argument("--bp-cluster", type=int, default=0, help="1 cluster form, -1 plain form, 0 autotuned")
-    ap.add_argument("--bp-slices", type=int, default=0, help="slices per backprojector CTA, 1 or 2 (0: autotuned)")
+    ap.add_argument("--bp-slices", type=int, default=0, help="slices per backprojector CTA, 1, 2 or 4 (0: autotuned)")
     ap.add_argument("--proj-views", type=int, default=0, help="views per projector CTA, 2, 4 or 8 (0: autotuned)")
     ap.add_argument("--bp-reduce", type=int, default=0,
                     help="-1: the finalize pass sums the view groups' partial images; 0/1: the last CTA of a tile does")

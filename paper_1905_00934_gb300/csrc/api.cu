@@ -1473,11 +1473,13 @@ extern "C" dect_status dect_admm_create(dect_geom* const* geoms, int32_t B, cons
         DECT_FAIL(DECT_EINVAL, "dect_admm_create: bp_tile must be 0 (autotuned), 32 or 64");
     if (P->bp_cluster < -1 || P->bp_cluster > 1)
         DECT_FAIL(DECT_EINVAL, "dect_admm_create: bp_cluster must be -1 (off), 0 (autotuned) or 1 (on)");
-    if (P->bp_slices < 0 || P->bp_slices > 2)
-        DECT_FAIL(DECT_EINVAL, "dect_admm_create: bp_slices must be 0 (autotuned), 1 or 2");
-    if (P->bp_cluster == 1 && P->bp_slices == 2)
+    if (P->bp_slices != 0 && P->bp_slices != 1 && P->bp_slices != 2 && P->bp_slices != 4)
+        DECT_FAIL(DECT_EINVAL, "dect_admm_create: bp_slices must be 0 (autotuned), 1, 2 or 4");
+    if (P->bp_cluster == 1 && P->bp_slices > 1)
         DECT_FAIL(DECT_EINVAL, "dect_admm_create: bp_cluster = 1 (the cluster form takes one slice per CTA) "
-                               "excludes bp_slices = 2");
+                               "excludes bp_slices = 2 and 4");
+    if (P->bp_tile == 64 && P->bp_slices == 4)
+        DECT_FAIL(DECT_EINVAL, "dect_admm_create: bp_slices = 4 takes 32-pixel tiles, not bp_tile = 64");
     if (P->bp_reduce < -1 || P->bp_reduce > 1)
         DECT_FAIL(DECT_EINVAL, "dect_admm_create: bp_reduce must be -1 (off), 0 (default: on) or 1 (on)");
     if (P->proj_views != 0 && P->proj_views != 2 && P->proj_views != 4 && P->proj_views != 8)
@@ -1557,11 +1559,13 @@ extern "C" dect_status dect_admm_create(dect_geom* const* geoms, int32_t B, cons
             }
         }
         const bool sg_ok = largest > 1 && P->scheme == DECT_SCHEME_UDM_PCG && P->storage != DECT_STORE_F64;
-        if (P->bp_slices == 2 && sg_ok) A->sg_cands = {2};
+        if (P->bp_slices > 1 && sg_ok) A->sg_cands = {P->bp_slices};
         else if (P->bp_slices == 0 && sg_ok && P->bp_cluster != 1) {
             A->sg_cands = {1, 2};
             if (largest > 2 && P->bp_tile != 64) A->sg_cands.push_back(4);  // 32-pixel tiles only
         } else A->sg_cands = {1};
+        if (A->sg_cands[0] == 4) tune_tiles = {32};
+        if (A->sg_cands[0] > 1) A->cluster_cands = {0};  // (several slices per CTA were asked for)
         A->sweep_sg = A->sg_cands.size() == 1 ? A->sg_cands[0] : 1;
         if (P->storage == DECT_STORE_F64) {
             A->sweep_C = 1;  // the float64 path has its own backprojector; no sweep, no partial images
