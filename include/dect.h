@@ -136,11 +136,11 @@ dect_status dect_project(dect_geom* g, int32_t n_channels, int32_t dtype, const 
  * this is a library convenience for callers that cannot call cudaMalloc (code
  * running during CUDA stream capture, code whose device memory belongs to its
  * own pool or framework allocator, fixed-budget deployments). Same operation,
- * layouts and results as dect_project, but its scratch (pair textures and an
- * interleaved image copy, 16*(nx*(ny+3) + ny*(nx+3)) + 8*nx*ny bytes) lives in
- * a fixed DECT_NOALLOC_SCRATCH_BYTES array of device global memory inside the
+ * layouts and results as dect_project, but its scratch (pair textures,
+ * 16*(nx*(ny+3) + ny*(nx+3)) bytes) lives in a fixed
+ * DECT_NOALLOC_SCRATCH_BYTES array of device global memory inside the
  * library, which every GPU that loads the library holds until exit; images up
- * to about 320 x 320 fit. Larger images are rejected with DECT_EINVAL and a
+ * to 360 x 360 fit. Larger images are rejected with DECT_EINVAL and a
  * message, before anything is launched. The first call on a device looks up
  * the array's device address (cudaGetSymbolAddress) with that device current;
  * make that first call before any stream capture. All calls share the array:

@@ -1,6 +1,6 @@
 // dect_project_noalloc: the forward projector for callers that cannot allocate device memory.
 //
-// dect_project keeps its scratch (the pair textures and the interleaved copy of the image) in
+// dect_project keeps its scratch (the pair textures of the image) in
 // the geometry handle and allocates it with cudaMalloc on first use. Some callers cannot allow
 // that: code running while a CUDA stream is being captured into a graph (cudaMalloc is not a
 // stream operation and breaks or invalidates the capture), code whose device memory is handed
@@ -22,8 +22,8 @@
 
 namespace dect {
 
-// Scratch of the no-allocation projector: TX [nx][ny+3] float4, TY [ny][nx+3] float4 and the
-// interleaved image [ny][nx] float2, packed in that order.
+// Scratch of the no-allocation projector: TX [nx][ny+3] float4 and TY [ny][nx+3] float4, packed in that order (one
+// channel uses half of each).
 static __device__ __align__(256) unsigned char g_noalloc_scratch[DECT_NOALLOC_SCRATCH_BYTES];
 
 // Device address of g_noalloc_scratch per device, looked up once with that device current.
@@ -47,7 +47,7 @@ static cudaError_t noalloc_scratch(unsigned char** out) {
 }
 
 size_t noalloc_bytes(int nx, int ny) {
-    return sizeof(float4) * ((size_t)nx * (ny + 3) + (size_t)ny * (nx + 3)) + sizeof(float2) * (size_t)nx * ny;
+    return sizeof(float4) * ((size_t)nx * (ny + 3) + (size_t)ny * (nx + 3));
 }
 
 }  // namespace dect

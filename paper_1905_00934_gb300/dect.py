@@ -272,7 +272,7 @@ def project_noalloc(geom, x, out, stream=None):
     """Like project, but with the library's fixed scratch array instead of any allocation.
 
     For callers that must not allocate device memory (e.g. while a stream is being captured).
-    Images must fit the fixed scratch (about 320 x 320); calls must not overlap on the GPU.
+    Images must fit the fixed scratch (360 x 360); calls must not overlap on the GPU.
     geom is a geometry handle or a solver.Geometry; with the latter the shapes are checked too.
     x: float32 [nch, ny, nx], out: float32 [nch, n_views, n_bins] (CUDA, contiguous), nch 1 or 2.
     """
