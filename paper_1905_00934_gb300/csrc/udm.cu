@@ -568,14 +568,17 @@ __device__ __forceinline__ void load_tables(const SpecDev& sp, float4* tabs) {
     __syncthreads();
 }
 
-// CTAs per SM that two rays per thread leave room for: holds the registers at 102 (126 otherwise; four, five, six CTAs:
-// 10 iterations of 737280 rays 468 / 453 / 477 us, one in the solver 0.600 / 0.545 / 0.597 ms)
-constexpr int kUdmCtas = 5;
+// CTAs per SM that the registers must allow: two rays per thread are held at 96 (126 otherwise; four, five, six CTAs:
+// 10 iterations of 737280 rays 468 / 453 / 477 us, one in the solver 0.600 / 0.545 / 0.597 ms when they were
+// compared), one ray at 64 with some spilled (10 iterations of 120000 rays 107 us, 111 at three CTAs and no spills; 4000
+// rays 43.0 and 41.9), the float64 arithmetic as many as it takes (80; at 64 it spilled: 512^2 slice 1899 -> 1910 us).
+template <int R, bool F64 = false>
+constexpr int kUdmCtas = F64 ? 1 : (R == 2 ? 5 : 4);
 
 // ADMM a-update fused with the a-block of the dual update (Eq. 11) and the a-block residual sums:
 // partial[4*blk + {0,1}] = sum (a - Rx)^2 (c, p); partial[4*blk + {2,3}] = sum (a - a_old)^2.
 template <class S2, bool F64, int R>
-__global__ void __launch_bounds__(kRaysPerBlock / R, R == 2 ? kUdmCtas : 4)
+__global__ void __launch_bounds__(kRaysPerBlock / R, kUdmCtas<R, F64>)
     k_udm_admm(const SliceDesc* __restrict__ dsl, BlockMap map, SpecDev sp, const float4* __restrict__ meas,
                const S2* __restrict__ Rx, S2* __restrict__ ua, S2* __restrict__ a, float* __restrict__ mu,
                uint8_t* __restrict__ status, const SliceScalars* __restrict__ sc, int iters,
@@ -649,7 +652,7 @@ __global__ void __launch_bounds__(kRaysPerBlock / R, R == 2 ? kUdmCtas : 4)
 
 // Initial decomposition: rho = (0, rho_p), v = 0, from a = (m_l / abar, 0), mu = mu0.
 template <class S2, int R>
-__global__ void __launch_bounds__(kRaysPerBlock / R, R == 2 ? kUdmCtas : 4)
+__global__ void __launch_bounds__(kRaysPerBlock / R, kUdmCtas<R>)
     k_udm_init(const SliceDesc* __restrict__ dsl, BlockMap map, SpecDev sp, const float4* __restrict__ meas,
                S2* __restrict__ a, float* __restrict__ mu, double rho_p, int iters, float abar, float mu0) {
     extern __shared__ float4 tabs[];
@@ -687,7 +690,7 @@ __global__ void __launch_bounds__(kRaysPerBlock / R, R == 2 ? kUdmCtas : 4)
 
 // Public per-ray entry point (planar float arrays).
 template <int R>
-__global__ void __launch_bounds__(kRaysPerBlock / R, R == 2 ? kUdmCtas : 4)
+__global__ void __launch_bounds__(kRaysPerBlock / R, kUdmCtas<R>)
     k_udm_rays(SpecDev sp, int64_t n, const float* __restrict__ mh, const float* __restrict__ ml,
                const float* __restrict__ wh, const float* __restrict__ wl, const float* __restrict__ vc,
                const float* __restrict__ vp, double rho_c, double rho_p, int iters, float* ac, float* ap, float* mu,
