@@ -152,7 +152,7 @@ dect_status dect_project_noalloc(const dect_geom* g, int32_t n_channels, const f
 
 /* Backprojection, the exact adjoint R^T of dect_project (Table 1's R^T):
  * x_dev[c] = R^T sino_dev[c]; same layouts and dtypes; x_dev is overwritten. Every
- * pixel is accumulated by one thread (image tiles sweep the rays that reach them,
+ * pixel is accumulated by one thread (image tiles gather the rays that reach them,
  * partial images are added in a fixed order; no atomics), so the result is
  * deterministic; it evaluates the same per-ray weights as dect_project, so
  * <R x, y> = <x, R^T y> up to float32 rounding. */
@@ -279,13 +279,14 @@ typedef struct {
     int32_t precondition;        /* enum dect_precond: 1 circulant model (default), 2 ramp filter,
                                     0 plain CG; other values: DECT_EINVAL */
     int32_t use_graph;           /* 1: capture one iteration as a CUDA graph */
-    int32_t bp_view_groups;      /* backprojector view groups per image tile, 1..16; -1 = chosen from the
-                                    occupancy (fill the GPU's resident slots); 0 = from the batch's tiles and views
-                                    (4 to 16; fewer where the partial images would not fit; reported in
-                                    dect_stats). It fixes the order of a pixel's
-                                    partial sums: results are bitwise reproducible for a fixed value, and a
-                                    slice solved alone or in a batch gives identical bits when the value is the
-                                    same (it is the one launch-dependent choice of the batch). */
+    int32_t bp_view_groups;      /* backprojector view groups per image tile, 1..16; -1 = 1 to 8, from the
+                                    batch's tiles alone (whole multiples of 11 CTAs per SM, 3 with 64-pixel
+                                    tiles); 0 = 4 to 16, from the batch's tiles and views (fewer where the
+                                    partial images take more than 4 GiB or 1/16 of the free memory; reported in
+                                    dect_stats). It fixes the order of a pixel's partial sums: results are
+                                    bitwise reproducible for a fixed value, and a slice solved alone or in a
+                                    batch gives identical bits when the value is the same (it is the one
+                                    launch-dependent choice of the batch). */
     int32_t storage;             /* dect_storage (DECT_STORE_F32): 16-bit formats halve the bytes of the
                                     sinogram vectors and textures at the cost of their precision */
     int32_t scheme;              /* dect_scheme (DECT_SCHEME_UDM_PCG): the splitting one iteration runs */
@@ -382,9 +383,11 @@ typedef struct {
     double r_pri[2], r_dual[2];
     double xi_db[2];             /* Eq. 14 against the truth (NaN without one) */
     int64_t count_R, count_RT;   /* projector applications per basis (Table 1) */
-    int64_t count_f;             /* forward-model evaluations per ray */
+    int64_t count_f;             /* forward-model evaluations per ray as Table 1 counts them: 4 per LM
+                                    iteration (two bases at two points; the kernels keep the sums of a point
+                                    that is reached by a kept step, so they make fewer) */
     int64_t count_launches;      /* kernels launched by this solver so far (all slices) */
-    int32_t bp_view_groups;      /* backprojector view groups per tile in use (fixed or autotuned) */
+    int32_t bp_view_groups;      /* backprojector view groups per tile in use */
     double objective;            /* Eq. 4 after iteration objective_iteration (NaN if never evaluated) */
     int32_t objective_iteration; /* see dect_params.objective_every; -1 if never evaluated */
     int32_t bp_tile;             /* backprojector tile side in use (0 for float64 storage) */
@@ -421,7 +424,7 @@ dect_status dect_admm_load(dect_admm* a, const void* src_host, size_t bytes, voi
 enum {
     DECT_PHASE_TEXTURE = 0,      /* pair textures of the image the projector reads */
     DECT_PHASE_PROJECT = 1,      /* R */
-    DECT_PHASE_BACKPROJECT = 2,  /* R^T: the tile sweep writing partial images */
+    DECT_PHASE_BACKPROJECT = 2,  /* R^T: the gather into partial images */
     DECT_PHASE_PRECOND = 3,      /* FFT preconditioner (3 kernels) */
     DECT_PHASE_UDM = 4,          /* Eq. 13 with the a-block dual update */
     DECT_PHASE_UPDATE = 5,       /* element-wise CG, Eq. 9-11 and dual rescaling kernels */

@@ -716,7 +716,7 @@ static void enq_precond(dect_admm* A, const float* H, const float2* r, float2* s
 // a reconstruction): 64^2 x 90 x 96, 50 blocks 1157 -> 1065 us, four slices 1400 -> 1308, 16 slices (800 blocks) 2265
 // -> 2200; 128^2 x 180 x 256, 244 blocks 1499 -> 1421; 256^2 x 360 x 512, 976 blocks 2753 and 2759.
 static bool cg_small_batch(const dect_admm* A) {
-    if (A->pix.total + A->rays.total > 6 * 152) return false;
+    if (A->pix.total + A->rays.total > 6 * kSms) return false;
     const std::vector<int>& rows = A->P.precondition ? A->prows.h : A->rows.h;
     for (int b = 0; b < A->B; ++b)
         if (A->pix.h[b + 1] - A->pix.h[b] > 256 || rows[b + 1] - rows[b] > 256) return false;
@@ -1189,15 +1189,22 @@ static dect_status enq_initialize(dect_admm* A, cudaStream_t st) {
 // groups to fill the chip, but a group of less than about 6 views pays more for its start than it computes;
 // medium batches of few views take as many groups as give 11 CTAs per SM; several slices of one geometry the count
 // that fills whole waves of CTAs best (6 per SM when paired, 11 otherwise), against a start of four views per
-// group and the partial images; large ones fill the chip with any count and take fewer partial images. Between 6 and
-// 16 groups the backprojector's time differs by a few percent (512^2 x 720 views, ms per iteration: one slice 0.71 to
-// 0.76; two 0.97 at 6, 0.89 at 10 and 12, 0.91 at 16; four 1.41 at 6, 1.37 at 8 to 12, 1.43 at 16; eight 2.57 to 2.67).
+// group and the partial images; large ones fill the chip with any count and take fewer partial images.
+// The count fixes the order of a pixel's sums, and reconstructions from the PCG start amplify a changed order, so the
+// lines lie where they reproduce best what timing at creation, which this rule replaced, used to choose on GB300 (110
+// sampled batches, two thirds alike; near-ties fell either way), not where the present kernel is fastest; its numbers
+// (0.62, 390, 480, 640, 800, 810, 1500) are fitted to those choices and have no other meaning. What that costs: over 66
+// batches of 48^2 to 1024^2, one to eight slices, the backprojector takes 1.02 times its best time over 4, 6, 8, 10, 12
+// and 16 groups in the median, 1.14 at the 90th percentile and 1.22 at most (128^2 x 180 views, four slices: 109 us per
+// application at 16, 89 at 10; 256^2 x 360, three: 258 at 8, 214 at 6; 512^2 x 720: one 611 at 12, 600 at 10; two 750
+// at 10; four 1179 at 16, 1099 at 8; eight 2030 at 6, 2024 at 4). bp_view_groups sets another count.
+// `paired` does not ask which slices per CTA or which form the caller allows: those promise the same bits.
 static int default_view_groups(int tiles, int paired, int views) {
     constexpr int kCounts[] = {4, 6, 8, 10, 12, 16};
     if (tiles < 100) return views >= 150 ? 16 : (paired && tiles >= 75) ? 10 : views >= 75 ? 12 : 10;
     if (paired && tiles < 160) return 10;
     if (paired && tiles < 1500) {
-        const double waves = paired <= 0.62 * tiles ? paired / (6.0 * 152.0) : tiles / (11.0 * 152.0);
+        const double waves = paired <= 0.62 * tiles ? paired / (6.0 * kSms) : tiles / (11.0 * kSms);
         int best = 0;
         double least = 0.0;
         for (int c : kCounts) {
@@ -1209,10 +1216,10 @@ static int default_view_groups(int tiles, int paired, int views) {
         }
         return best;
     }
-    if (4 * tiles <= 11 * 152 && views < 390) {
+    if (4 * tiles <= 11 * kSms && views < 390) {
         int C = 4;
         for (int c : kCounts)
-            if (tiles * c <= 11 * 152) C = c;
+            if (tiles * c <= 11 * kSms) C = c;
         return C;
     }
     if (tiles < 480) return 12;
@@ -1570,13 +1577,14 @@ extern "C" dect_status dect_admm_create(dect_geom* const* geoms, int32_t B, cons
         if (P->storage == DECT_STORE_F64) {
             A->sweep_C = 1;  // the float64 path has its own backprojector; no sweep, no partial images
         } else if (P->bp_view_groups > 0) {
-            A->sweep_C = sweep_ctas_for_groups(P->bp_view_groups);
+            A->sweep_C = P->bp_view_groups;
             tune.push_back(A->sweep_C);  // the tile sides and the cluster form may still be timed at this C
         } else if (P->bp_view_groups < 0) {
-            A->sweep_C = sweep_groups(total, tile0);  // occupancy choice, not timed
+            A->sweep_C = sweep_groups(total, tile0);  // from the tiles alone
         } else {
-            // from the batch's shape, as far as the partial images fit in 1/16 of the free memory and 4 GiB.
-            // Not timed: it fixes the order of a pixel's sums, so the same batch gives the same bits on every run.
+            // from the batch's shape and not timed: it fixes the order of a pixel's sums, so the same batch gives the
+            // same bits on every run, wherever the partial images fit in 4 GiB and 1/16 of the free memory (fewer groups
+            // otherwise)
             size_t free_b = 0, total_b = 0;
             cudaMemGetInfo(&free_b, &total_b);
             const double budget = std::min(4.0 * (1 << 30), (double)free_b / 16.0);
@@ -1779,7 +1787,7 @@ extern "C" dect_status dect_admm_create(dect_geom* const* geoms, int32_t B, cons
             return DECT_ECUDA;
         }
     }
-    A->sweep_groups_in_use = A->sweep_C * sweep_groups_per_cta();
+    A->sweep_groups_in_use = A->sweep_C;
     if (P->scheme == DECT_SCHEME_LM_CG) {
         // the comparison scheme has no a-block: its residual slots stay zero for the rho update
         e = cudaMemset(A->part_udm, 0, sizeof(double) * 4 * (size_t)A->rays.h.back());

@@ -677,9 +677,6 @@ __global__ void __launch_bounds__(fin_threads(MODE)) k_bp_finalize(const SliceDe
 
 int sweep_tiles(int nx, int ny, int tile) { return ((nx + tile - 1) / tile) * ((ny + tile - 1) / tile); }
 
-int sweep_ctas_for_groups(int view_groups) { return view_groups; }
-int sweep_groups_per_cta() { return 1; }
-
 // the kernels' dynamic shared memory may exceed the default 48 KB; the attribute is per device
 template <class S2, int NCH, int TILE, bool CLUSTER, int SG>
 static cudaError_t sweep_attr1() {
@@ -711,14 +708,11 @@ cudaError_t sweep_init_attributes() {
     return e;
 }
 
-// View groups per tile for a launch that is not autotuned: the smallest C (up to 8) whose tiles * C CTAs fill
+// View groups per tile from the tiles alone (bp_view_groups = -1, the preconditioners' point responses): the smallest C (up to 8) whose tiles * C CTAs fill
 // whole multiples of 11 CTAs per SM (3 of the 64-pixel tiles) best: two to four times the resident ones, so that
 // the last ones to finish leave little of the chip idle.
 int sweep_groups(int tiles, int tile) {
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int slots = (sms > 0 ? sms : 1) * (tile == 64 ? 3 : 11);
+    const int slots = kSms * (tile == 64 ? 3 : 11);
     int best = 1;
     double best_fill = 0.0;
     for (int C = 1; C <= 8; ++C) {
@@ -861,8 +855,9 @@ void backproject_single(const SliceDesc& sd, const SliceDesc* d_dev, const int* 
     }
 }
 
-// About 6000 CTAs (eight waves) at most, 11 groups at most and four views each at least. Measured per call and
-// pair of bases: 512^2 (256 tiles) 395 us at 6 groups, 368 at 11, 372 at 16; 256^2: 95, 83, 87; 93^2: 31, 30, 31.
+// About 6000 CTAs (eight waves) with 2 to 11 groups, of four views each at least. Measured per call and pair of bases:
+// 512^2 (256 tiles) 350 us at 6 groups, 327 at 11, 322 at 16; 256^2: 66, 62, 60; 93 x 70: 18, 16, 15 (11 was the best
+// count when it was chosen; it stays, since it fixes the order of a pixel's sums).
 int sweep_groups_single(int tiles, int nv) {
     int C = 6000 / (tiles > 0 ? tiles : 1);
     C = C > 11 ? 11 : (C < 2 ? 2 : C);

@@ -29,6 +29,7 @@
 namespace dect {
 
 constexpr int kMaxEnergies = 512;
+constexpr int kSms = 152;  // GB300 (a constant where a choice fixes results' bits: those must not vary with the device)
 constexpr int kFftMaxLog2 = 12;  // padded FFT length up to 4096 per axis
 constexpr int kFftMax = 1 << kFftMaxLog2;
 
@@ -162,8 +163,6 @@ void launch_project(const SliceDesc* dsl, const BlockMap& map, int nblk, const i
                     const void* ty, void* out, int prec, int views, cudaStream_t st);
 // backproject_sweep.cu: the solver's backprojector (two kernels: the gather into C partial images, then
 // the fixed-order sum of the partials with the epilogue; partial dots over the `pix` blocks)
-int sweep_ctas_for_groups(int view_groups);
-int sweep_groups_per_cta();
 // image tiles for a TILE x TILE tile (32 or 64); the view groups of a launch that is not autotuned
 int sweep_tiles(int nx, int ny, int tile);
 int sweep_groups(int tiles, int tile);

@@ -281,13 +281,13 @@ void launch_unpack_meas(int64_t n, const float4* meas, float* planar, cudaStream
 template <int NCH>
 static void fbp_t(const FbpDev& f, const float* sino, float* q, float* x, bool clamp, cudaStream_t st) {
     auto* rows = reinterpret_cast<FbpEntry<NCH>*>(q);
-    // one CTA per view as far as the threads go (4096 bins), several where the views leave some of the 152 SMs idle
+    // one CTA per view as far as the threads go (4096 bins), several where the views leave some of the SMs idle
     auto parts = [&](int warps) {
         const int bins = kFbpWarpBins * warps;
         return f.nb <= bins ? 1 : (f.nb - 17) / (bins - 16) + 1;
     };
     int warps = std::min(kFbpMaxWarps, (f.nb + kFbpWarpBins - 1) / kFbpWarpBins);
-    while (warps > 1 && (int64_t)f.nv * parts(warps) < 152) --warps;
+    while (warps > 1 && (int64_t)f.nv * parts(warps) < kSms) --warps;
     const int n = parts(warps), stride = n == 1 ? f.nb : 16 * (((f.nb - 1) / 16 + n - 1) / n);  // (whole eights of either parity)
     const dim3 grid((unsigned)f.nv, (unsigned)n);
     const unsigned threads = 64 * NCH * warps;

@@ -16,7 +16,7 @@
 // bins; Joseph's linear interpolation between the two neighbours; the image is
 // read through a pair texture (both neighbours of both bases in one 16-byte load).
 //
-// R^T: the column-sweep kernel of backproject_sweep.cu evaluates the same
+// R^T: the gathering kernel of backproject_sweep.cu evaluates the same
 // integers per sample, so <R x, y> = <x, R^T y> holds to float32 summation
 // rounding; no atomics, deterministic.
 #include <cuda_runtime.h>
