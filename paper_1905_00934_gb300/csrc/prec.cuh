@@ -48,12 +48,8 @@ __device__ __forceinline__ void st2(float* p, float2 v) { *p = v.x; }  // single
 __device__ __forceinline__ void st2(__half2* p, float2 v) { *p = __float22half2_rn(v); }
 __device__ __forceinline__ void st2(__nv_bfloat162* p, float2 v) { *p = __float22bfloat162_rn(v); }
 
-// pair-texture texels: {c(lo), p(lo), c(hi), p(hi)}; single-channel texels float2 {lo, hi}
+// pair-texture texels: {c(lo), p(lo), c(hi), p(hi)} (single-channel texels are float2 {lo, hi})
 __device__ __forceinline__ float4 ldtex(const float4* p) { return __ldg(p); }
-__device__ __forceinline__ float4 ldtex(const float2* p) {
-    const float2 v = __ldg(p);
-    return make_float4(v.x, 0.f, v.y, 0.f);
-}
 __device__ __forceinline__ float4 ldtex(const TexH* p) {
     const uint2 u = __ldg(reinterpret_cast<const uint2*>(p));
     const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&u.x));
