@@ -333,7 +333,9 @@ __global__ void __launch_bounds__(GatherShape<TILE, NCH, SG>::kThreads, GatherSh
                 flush();
 #pragma unroll
                 for (int i = 0; i < kRays; ++i) {
-                    if (lane + 32 * i >= n) break;
+                    // (past the n-th: the last window's ray, unused. One channel is faster by 2 to 3 % without the test, two
+                    // by 0.5 % with it)
+                    if (NCH == 2 && lane + 32 * i >= n) break;
                     P[i] = __ldg(g.rays + e[i]);
                     if constexpr (NCH == 2) {
 #pragma unroll
