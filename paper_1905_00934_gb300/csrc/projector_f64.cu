@@ -78,9 +78,10 @@ __global__ void __launch_bounds__(kRayThreads) k_project_f64(GeomDev g, const do
     const int64_t n = (int64_t)g.nv * g.nb;
     const int64_t r = ((int64_t)blockIdx.x * kRayThreads + threadIdx.x) / kLanesPerRay;
     const int sub = threadIdx.x % kLanesPerRay;
-    double acc[NCH];
+    // the lower and the upper neighbours' products in sums of their own: one rounding per product, at half the sum's size
+    double acc[NCH], up[NCH];
 #pragma unroll
-    for (int c = 0; c < NCH; ++c) acc[c] = 0.0;
+    for (int c = 0; c < NCH; ++c) acc[c] = up[c] = 0.0;
     double w = 0.0;
     if (r < n) {
         const double4_32a P = rays[r];
@@ -113,14 +114,17 @@ __global__ void __launch_bounds__(kRayThreads) k_project_f64(GeomDev g, const do
             for (int c = 0; c < NCH; ++c) {
                 const double a = in0 ? __ldg(im + c * plane) : 0.0;
                 const double b = in1 ? __ldg(im + c * plane + s_across) : 0.0;
-                acc[c] = __fma_rn(f, b, __fma_rn(1.0 - f, a, acc[c]));
+                acc[c] = __fma_rn(1.0 - f, a, acc[c]);
+                up[c] = __fma_rn(f, b, up[c]);
             }
         }
     }
 #pragma unroll
-    for (int c = 0; c < NCH; ++c)
+    for (int c = 0; c < NCH; ++c) {
+        acc[c] += up[c];
 #pragma unroll
         for (int o = 1; o < kLanesPerRay; o <<= 1) acc[c] += __shfl_xor_sync(0xffffffffu, acc[c], o);
+    }
     if (r < n && sub == 0)
 #pragma unroll
         for (int c = 0; c < NCH; ++c) out[c * n + r] = w * acc[c];
