@@ -144,7 +144,7 @@ WORKLOAD = "fan 512x512, 720 views x 1024 bins, 40 objects, I0 2e5, UDM1-PCG1 x 
 # launch shape they were captured with (slices, view groups, tile side, cluster form, slices per CTA,
 # reduced form); from the counter capture in profiles/k_bp_gather_512x720x1024.txt. Reported only when
 # the run uses one of these shapes.
-GATHER_TRAFFIC = {(8, 6, 32, 0, 4, 1): 57.7e6}
+GATHER_TRAFFIC = {(8, 6, 32, 0, 4, 1): 57.4e6}
 
 
 # ------------------------------------------------------------------------------------------------

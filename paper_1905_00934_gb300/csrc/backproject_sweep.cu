@@ -1,4 +1,5 @@
-// Gathering backprojector R^T of the ADMM solver (Table 1's R^T, with the CG epilogues of Eq. 12).
+// Gathering backprojector R^T of the ADMM solver (Table 1's R^T, with the CG epilogues of Eq. 12). (The file and the
+// host functions keep the name of the sweep that it replaced.)
 //
 // A CTA owns a pixel tile (32 x 32 or 64 x 64) and a group of views. It takes the rays sampled once per
 // column (axis 0) and then those sampled once per row (axis 1): staging warps write the rays of each view that can
@@ -18,8 +19,8 @@
 // What bounds it: the FP32 pipe (the packed pair instruction takes two cycles of it) with 2.2 of the 5.5 rays a
 // block takes per view weighing anything at a given pixel, then issue. Its predecessor kept the tile's sums in
 // shared memory (each sample a read-modify-write of two rows) and was bound by shared-memory wavefronts; measured
-// on GB300, 512 x 512 x 720 x 1024, both bases, per application: one slice 439 -> 359 us, 8 slices of one
-// geometry 2509 -> 1286 us; 93 x 70 x 61 x 131: 97 -> 8 us (the old kernel's two warps per tile left the chip empty).
+// on GB300, 512 x 512 x 720 x 1024, both bases, per application: one slice 439 -> 351 us, 8 slices of one
+// geometry 2509 -> 1180 us; 93 x 70 x 61 x 131: 97 -> 8 us (the old kernel's two warps per tile left the chip empty).
 // Detectors coarser than three pixels per bin are the one place where the predecessor was faster (its work went by the
 // rays, this one's by pixels and views): 512^2 x 720 views, bins of 3 / 4 / 16 pixels 193 / 172 / 124 -> 198 / 185 / 162
 // us. No workload here has them.

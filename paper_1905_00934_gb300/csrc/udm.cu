@@ -6,10 +6,11 @@
 // and f_h, f_l at the trial point a + delta enter, the 4 evaluations of f of Table 1; the
 // sums at a trial point that is kept are the next iteration's sums at a, so an iteration
 // makes one pass over the energies (one exp2 and eight FMAs per bin), not two.
-// What bounds it: issue and the FMA pipe (a packed pair takes it for two cycles). Measured on GB300, 737280 rays
-// of 121 bins: 10 iterations 878 -> 453 us (one pass per iteration, two rays per thread and five CTAs, the bare
-// exponential where nothing underflows, no per-bin tests there, no division to choose the logarithm); one iteration
-// inside the solver, 8 slices: 0.739 -> 0.545 ms.
+// What bounds it: issue and the FMA pipe (a packed pair takes it for two cycles); in warps whose exponentials underflow
+// in some blocks of energies the instruction cache, which does not hold both forms of a block's body. Measured on
+// GB300, 737280 rays of 121 bins: 10 iterations 878 -> 437 us (one pass per iteration, two rays per thread and five
+// CTAs, the bare exponential where nothing underflows, no per-bin tests there, no division to choose the logarithm, a
+// warp's lanes kept together); one iteration inside the solver, one slice: 100 -> 74 us.
 // Energy
 // sums are float32 (compensated). Residuals come from the ratio of a spectral
 // sum to the measured transmission t = e^{-m}: f - m = -log(s / t), from
