@@ -563,7 +563,7 @@ __device__ void lm_ray64(const float4* __restrict__ t1, const double4_32a* __res
 }
 
 // (as it lies in global memory: when every CTA formed the blocks' maxima itself, eight shared loads of one bank per lane,
-// the vjp of 130000 rays of 121 bins took 17.4 us instead of 16.5, of 33 rays 6.8 instead of 5.4)
+// the vjp of 130000 rays of 121 bins took 17.4 us instead of 16.5 in blocks of 256, of 33 rays 6.8 instead of 5.4)
 __device__ __forceinline__ void load_tables(const SpecDev& sp, float4* tabs) {
     for (int e = threadIdx.x; e < table_len(sp.ne); e += blockDim.x) tabs[e] = __ldg(sp.tab + e);
     __syncthreads();
@@ -843,17 +843,21 @@ void launch_lm_trial(const SliceDesc* dsl, const BlockMap& map, int nblk, const 
 // float32: the LM kernel's sums (compensated, float32 exponentials), logs and ratios in float64.
 // float64: tables and exponentials in float64 (t64 = {S_h, S_l, f_KN, f_p} per energy, unit-sum S).
 
-__global__ void __launch_bounds__(kRaysPerBlock) k_forward_model_f32(SpecDev sp, int64_t n, const float* __restrict__ ac,
-                                                                     const float* __restrict__ ap, float* __restrict__ fh,
-                                                                     float* __restrict__ fl, float* __restrict__ jac,
-                                                                     const float* __restrict__ gh,
-                                                                     const float* __restrict__ gl, float* __restrict__ oc,
-                                                                     float* __restrict__ op) {
+// Blocks of 128 rays: the float64 tail binds, and with 256 some SMs take four blocks where the average is 3.3. vjp, 121
+// energies, 256 / 128 / 64 rays a block: 1000 rays 6.3 / 5.3 / 5.6 us, 130000 rays 16.6 / 15.4 / 15.7, 300000 rays 25.2 /
+// 25.5 / 25.8, 737280 rays 47.5 / 47.8 / 48.2.
+constexpr int kModelRays = 128;
+__global__ void __launch_bounds__(kModelRays) k_forward_model_f32(SpecDev sp, int64_t n, const float* __restrict__ ac,
+                                                                  const float* __restrict__ ap, float* __restrict__ fh,
+                                                                  float* __restrict__ fl, float* __restrict__ jac,
+                                                                  const float* __restrict__ gh,
+                                                                  const float* __restrict__ gl, float* __restrict__ oc,
+                                                                  float* __restrict__ op) {
     extern __shared__ float4 tabs[];
     float4* t1 = tabs;
     float4* t2 = tabs + padded(sp.ne);
     load_tables(sp, tabs);
-    const int64_t r = (int64_t)blockIdx.x * kRaysPerBlock + threadIdx.x;
+    const int64_t r = (int64_t)blockIdx.x * kModelRays + threadIdx.x;
     const int64_t e = min(r, n - 1);  // (a lane past the last ray repeats it, unstored)
     const float a[1] = {__ldg(ac + e)}, p[1] = {__ldg(ap + e)};
     if (!jac && !oc) {  // (half of the sums, the same bits)
@@ -926,7 +930,7 @@ void launch_forward_model(const SpecDev& sp, const double4_32a* t64, int64_t n, 
                           void* op, cudaStream_t st) {
     if (n <= 0) return;
     if (dtype == DECT_F32)
-        k_forward_model_f32<<<(unsigned)((n + kRaysPerBlock - 1) / kRaysPerBlock), kRaysPerBlock, tab_bytes(sp), st>>>(
+        k_forward_model_f32<<<(unsigned)((n + kModelRays - 1) / kModelRays), kModelRays, tab_bytes(sp), st>>>(
             sp, n, (const float*)ac, (const float*)ap, (float*)fh, (float*)fl, (float*)jac, (const float*)gh,
             (const float*)gl, (float*)oc, (float*)op);
     else
